@@ -267,6 +267,69 @@ __device__ __forceinline__ double warp_reduce_scatter4(double v0, double v1, dou
     return k;
 }
 
+// One column pair by the whole CTA (rows, cols <= 2 blockDim): the warps split the rows, one or two
+// register elements per thread and column, the partial dot products meeting in red4 (double-buffered
+// by buf: a warp writes buffer b of pair k + 2 only after the barrier of pair k + 1, which every warp
+// reaches after reading buffer b of pair k). Returns whether it rotated. low2, th2: a pair with a column
+// of squared norm <= low2 also counts as orthogonal once |gamma|^2 <= th2 max(alpha, beta).
+__device__ __forceinline__ bool jacobi_relaxed(double al, double be, double g2, double low2, double th2) {
+    return fmin(al, be) <= low2 && g2 <= th2 * fmax(al, be);
+}
+__device__ __forceinline__ bool jacobi_pair_cta(int rows, int cols, zd* ap, zd* aq, zd* vp, zd* vq, double tol,
+                                                double low2, double th2, double (*red4)[8][4], int& buf) {
+    const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, nsub = nthr >> 5;
+    const bool two = rows > nthr || cols > nthr;  // second element per thread needed
+    zd xa[2], ya[2], xv[2], yv[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int i = tid + nthr * t;
+        const bool ua = (t == 0 || two) && i < rows, uv = (t == 0 || two) && i < cols;
+        xa[t] = ua ? ldcg(ap + i) : mk(0.0, 0.0);
+        ya[t] = ua ? ldcg(aq + i) : mk(0.0, 0.0);
+        xv[t] = uv ? ldcg(vp + i) : mk(0.0, 0.0);
+        yv[t] = uv ? ldcg(vq + i) : mk(0.0, 0.0);
+    }
+    double al = norm2(xa[0]), be = norm2(ya[0]);
+    zd ga = fmac(mk(0.0, 0.0), xa[0], ya[0]);
+    if (two) {
+        al += norm2(xa[1]);
+        be += norm2(ya[1]);
+        ga = fmac(ga, xa[1], ya[1]);
+    }
+    const double ws = warp_reduce_scatter4(al, be, ga.re, ga.im, lane);
+    const int w = tid >> 5;
+    if ((lane & 7) == 0) red4[buf][w][lane >> 3] = ws;
+    __syncthreads();
+    // every warp adds the nsub partials itself, in the same order, so all warps
+    // hold bit-identical rotation scalars without another barrier: lane l takes
+    // value l & 3 of warp l >> 2
+    double x = (lane >> 2) < nsub ? red4[buf][lane >> 2][lane & 3] : 0.0;
+    buf ^= 1;
+    for (int o = 4; o < 4 * nsub; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    al = __shfl_sync(0xffffffffu, x, 0);
+    be = __shfl_sync(0xffffffffu, x, 1);
+    const double gr = __shfl_sync(0xffffffffu, x, 2), gi = __shfl_sync(0xffffffffu, x, 3);
+    double c, sr, si;
+    if (low2 >= 0.0 && jacobi_relaxed(al, be, fma(gr, gr, gi * gi), low2, th2)) return false;
+    if (!jacobi_rotation(al, be, gr, gi, tol, c, sr, si)) return false;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int i = tid + nthr * u;
+        if (u == 1 && !two) break;
+        if (i < rows) {
+            jacobi_apply(c, sr, si, xa[u], ya[u]);
+            ap[i] = xa[u];
+            aq[i] = ya[u];
+        }
+        if (i < cols) {
+            jacobi_apply(c, sr, si, xv[u], yv[u]);
+            vp[i] = xv[u];
+            vq[i] = yv[u];
+        }
+    }
+    return true;
+}
+
 __global__ void __launch_bounds__(256) jacobi_kernel(int rows, int cols, zd* __restrict__ A, zd* __restrict__ Vm,
                                                      int max_sweeps, double tol, int* __restrict__ flags,
                                                      int* __restrict__ sweeps_out, GridBar bar) {
@@ -277,8 +340,6 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int rows, int cols, zd* __r
     const int nsub = blockDim.x >> 5;
     const int gwarp = nsub > 1 ? (int)blockIdx.x : (int)(blockIdx.x * nsub + (threadIdx.x >> 5));
     const int nwarps = nsub > 1 ? (int)gridDim.x : (int)(gridDim.x * nsub);
-    // per-warp partial sums, double-buffered: a warp writes buffer b of pair k + 2 only after the
-    // barrier of pair k + 1, which every warp reaches after reading buffer b of pair k
     __shared__ double red4[2][8][4];
     int buf = 0;
     const int P = cols + (cols & 1);
@@ -306,58 +367,8 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int rows, int cols, zd* __r
                 zd* vp = Vm + (int64_t)p * cols;
                 zd* vq = Vm + (int64_t)q * cols;
                 if (rows <= 256 && cols <= 256 && nsub > 1) {
-                    // the CTA's warps split the rows: one register element per lane per column
-                    // (rows <= 32 * nsub * 2); partial dot products meet in shared memory
-                    const int tid = threadIdx.x, nthr = blockDim.x;
-                    const bool two = rows > nthr || cols > nthr;  // second element per thread needed
-                    zd xa[2], ya[2], xv[2], yv[2];
-#pragma unroll
-                    for (int t = 0; t < 2; ++t) {
-                        const int i = tid + nthr * t;
-                        const bool ua = (t == 0 || two) && i < rows, uv = (t == 0 || two) && i < cols;
-                        xa[t] = ua ? ldcg(ap + i) : mk(0.0, 0.0);
-                        ya[t] = ua ? ldcg(aq + i) : mk(0.0, 0.0);
-                        xv[t] = uv ? ldcg(vp + i) : mk(0.0, 0.0);
-                        yv[t] = uv ? ldcg(vq + i) : mk(0.0, 0.0);
-                    }
-                    double al = norm2(xa[0]), be = norm2(ya[0]);
-                    zd ga = fmac(mk(0.0, 0.0), xa[0], ya[0]);
-                    if (two) {
-                        al += norm2(xa[1]);
-                        be += norm2(ya[1]);
-                        ga = fmac(ga, xa[1], ya[1]);
-                    }
-                    const double ws = warp_reduce_scatter4(al, be, ga.re, ga.im, lane);
-                    const int w = tid >> 5;
-                    if ((lane & 7) == 0) red4[buf][w][lane >> 3] = ws;
-                    __syncthreads();
-                    // every warp adds the nsub partials itself, in the same order, so all warps
-                    // hold bit-identical rotation scalars without another barrier: lane l takes
-                    // value l & 3 of warp l >> 2
-                    double x = (lane >> 2) < nsub ? red4[buf][lane >> 2][lane & 3] : 0.0;
-                    buf ^= 1;
-                    for (int o = 4; o < 4 * nsub; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                    al = __shfl_sync(0xffffffffu, x, 0);
-                    be = __shfl_sync(0xffffffffu, x, 1);
-                    const double gr = __shfl_sync(0xffffffffu, x, 2), gi = __shfl_sync(0xffffffffu, x, 3);
-                    double c, sr, si;
-                    if (!jacobi_rotation(al, be, gr, gi, tol, c, sr, si)) continue;
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        const int i = tid + nthr * u;
-                        if (u == 1 && !two) break;
-                        if (i < rows) {
-                            jacobi_apply(c, sr, si, xa[u], ya[u]);
-                            ap[i] = xa[u];
-                            aq[i] = ya[u];
-                        }
-                        if (i < cols) {
-                            jacobi_apply(c, sr, si, xv[u], yv[u]);
-                            vp[i] = xv[u];
-                            vq[i] = yv[u];
-                        }
-                    }
-                    if (tid == 0) atomicOr(&flags[sweep & 1], 1);
+                    if (jacobi_pair_cta(rows, cols, ap, aq, vp, vq, tol, -1.0, 0.0, red4, buf) && threadIdx.x == 0)
+                        atomicOr(&flags[sweep & 1], 1);
                     continue;
                 }
                 double al = 0.0, be = 0.0;
@@ -397,6 +408,216 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int rows, int cols, zd* __r
     if (blockIdx.x == 0 && threadIdx.x == 0) *sweeps_out = sweep + 1;
 }
 
+// The same rotations with the pairs of a sweep chosen beforehand, for the Hankel SVD (rows, cols <= 256).
+// Each sweep first screens all pairs with a column that changed since their last screening (a warp per
+// pair); the run ends when no pair needs a rotation. The pairs that do are taken in the round-robin order
+// of jacobi_kernel, the e-th of them by CTA e mod gridDim, without barriers between the rounds: a pair
+// waits until its two columns have been through their earlier pairs (a counter per column, and the pair's
+// rank among its column's pairs). The order of the rotations on every column is fixed, so the result does not
+// depend on timing; the first unfinished pair never waits, so the CTAs cannot wait for one another in a
+// circle. Every wait is bounded as the grid barrier's is.
+//
+// A pair needs a rotation when |gamma| > tol sqrt(alpha beta), as in jacobi_kernel, except that a
+// pair with a column of norm <= sqrt(low2) |R_00| (a tenth of the rank threshold: its triplet is not used, only
+// its singular value is reported) needs none once |gamma| <= sqrt(th2) |R_00| max(|a_p|, |a_q|). What such a
+// pair leaves is a component of at most sqrt(th2) |R_00| of the smaller column along the larger one, a fifth
+// of the truncation that the QR applies elsewhere (1e-14 |R_00|). The moments' rounding noise
+// fills the Hankel matrix with columns of norm 1e-15 to 1e-14 sigma_1, and orthogonalising those
+// against each other to full relative accuracy was most of the work.
+constexpr int kScreenMax = 256;     // rows and columns at most
+struct ScreenWork {
+    int count[2];                                    // pairs that need a rotation, by sweep parity
+    int changed[kScreenMax];                         // column rotated since the last screening
+    int done[kScreenMax];                            // pairs that the column has been through
+    unsigned int mask[kScreenMax][4];                // per round, its pairs that need a rotation
+    int rank[kScreenMax][kScreenMax];                // [column][round]: done[] before that round's pair
+    unsigned char need[kScreenMax * kScreenMax];     // [p * cols + q], p < q
+};
+size_t jacobi_screen_bytes(int n) { return n <= kScreenMax ? sizeof(ScreenWork) : 0; }
+
+__global__ void __launch_bounds__(128) jacobi_screened_kernel(int rows, int cols, zd* __restrict__ A, zd* __restrict__ Vm,
+                                                              int max_sweeps, double tol, double low2, double th2,
+                                                              ScreenWork* __restrict__ sw,
+                                                              int* __restrict__ sweeps_out, GridBar bar) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    __shared__ double red4[2][8][4];
+    __shared__ unsigned int msk[kScreenMax][4];
+    __shared__ int base[kScreenMax + 1];  // pairs before each round
+    __shared__ int chg[kScreenMax];
+    int buf = 0;
+    const int P = cols + (cols & 1), G = gridDim.x, R = P - 1;
+    unsigned int epoch = 0;
+    const double s1 = norm2(ldcg(A));
+    low2 *= s1;
+    th2 *= s1;
+    auto pos = [&](int k, int r) { return k == 0 ? 0 : ((k - 1 + r) % R) + 1; };  // round r, place k: column
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + tid; t < (int64_t)cols * cols; t += (int64_t)G * blockDim.x)
+        Vm[t] = mk((t % cols) == (t / cols) ? 1.0 : 0.0, 0.0);
+    if (blockIdx.x == 0) {
+        for (int i = tid; i < kScreenMax; i += blockDim.x) sw->changed[i] = 1, sw->done[i] = 0;
+        if (tid < 2) sw->count[tid] = 0;
+    }
+    grid_barrier(bar, epoch);
+    int sweep = 0;
+    for (; sweep < max_sweeps; ++sweep) {
+        // a warp per (column p, four columns q > p): p in registers, up to eight rows a lane
+        int found = 0;
+        for (int e = tid; e < kScreenMax; e += blockDim.x) chg[e] = __ldcg(&sw->changed[e]);
+        __syncthreads();
+        const int qg = (cols + 3) / 4;
+        for (int t = (int)blockIdx.x * nw + warp; t < cols * qg; t += G * nw) {
+            const int p = t % cols, q0 = 4 * (t / cols);
+            if (q0 + 3 <= p) continue;
+            const int cp = chg[p];
+            bool any = false, todo[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = q0 + u;
+                const bool in = q > p && q < cols;
+                todo[u] = in && (cp | chg[in ? q : p]);
+                any |= todo[u];
+                if (in && !todo[u]) found += __ldcg(&sw->need[p * cols + q]) != 0;
+            }
+            if (!any) continue;
+            double al = 0.0, be[4] = {0.0, 0.0, 0.0, 0.0};
+            zd ga[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) ga[u] = mk(0.0, 0.0);
+            const zd* ap = A + (int64_t)p * rows;
+            const zd* aq = A + (int64_t)q0 * rows;
+            for (int i = lane; i < rows; i += 32) {
+                const zd x = ldcg(ap + i);
+                zd y[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) y[u] = todo[u] ? ldcg(aq + (int64_t)u * rows + i) : mk(0.0, 0.0);
+                al += norm2(x);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    be[u] += norm2(y[u]);
+                    ga[u] = fmac(ga[u], x, y[u]);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const double ws = warp_reduce_scatter4(al, be[u], ga[u].re, ga[u].im, lane);
+                const double a1 = __shfl_sync(0xffffffffu, ws, 0), b1 = __shfl_sync(0xffffffffu, ws, 8);
+                const double gr = __shfl_sync(0xffffffffu, ws, 16), gi = __shfl_sync(0xffffffffu, ws, 24);
+                const double g2 = fma(gr, gr, gi * gi);
+                if (todo[u]) {
+                    const bool need =
+                        g2 > (tol * tol) * (a1 * b1) && a1 != 0.0 && b1 != 0.0 && !jacobi_relaxed(a1, b1, g2, low2, th2);
+                    if (lane == 0) sw->need[p * cols + q0 + u] = need ? 1 : 0;
+                    found += need;
+                }
+            }
+        }
+        if (lane == 0 && found) atomicAdd(&sw->count[sweep & 1], found);
+        grid_barrier(bar, epoch);
+        if (__ldcg(&sw->count[sweep & 1]) == 0) break;
+        if (blockIdx.x == 0 && tid == 0) sw->count[(sweep + 1) & 1] = 0;
+        if (blockIdx.x == 0)
+            for (int i = tid; i < kScreenMax; i += blockDim.x) sw->changed[i] = 0;
+        auto needed = [&](int a, int b) {
+            return a < cols && b < cols && __ldcg(&sw->need[min(a, b) * cols + max(a, b)]) != 0;
+        };
+        // a warp per round: its pairs; a warp per column: the ranks of its pairs
+        for (int t = (int)blockIdx.x * nw + warp; t < R + cols; t += G * nw) {
+            if (t < R) {
+                for (int w = 0; w < 4; ++w) {
+                    const int k = 32 * w + lane;
+                    const unsigned int b =
+                        __ballot_sync(0xffffffffu, k < P / 2 && needed(pos(k, t), pos(P - 1 - k, t)));
+                    if (lane == 0) sw->mask[t][w] = b;
+                }
+            } else {
+                const int c = t - R;
+                int at = __ldcg(&sw->done[c]);
+                for (int r0 = 0; r0 < R; r0 += 32) {
+                    const int r = r0 + lane;
+                    bool nd = false;
+                    if (r < R) {
+                        int k = 0;  // the column's place in round r
+                        if (c) {
+                            k = (c - 1 - r) % R;
+                            k = (k < 0 ? k + R : k) + 1;
+                        }
+                        nd = needed(c, pos(P - 1 - k, r));
+                    }
+                    const unsigned int b = __ballot_sync(0xffffffffu, nd);
+                    if (r < R) sw->rank[c][r] = at + __popc(b & ((1u << lane) - 1u));
+                    at += __popc(b);
+                }
+            }
+        }
+        grid_barrier(bar, epoch);
+        for (int e = tid; e < 4 * R; e += blockDim.x) msk[e >> 2][e & 3] = __ldcg(&sw->mask[e >> 2][e & 3]);
+        __syncthreads();
+        if (warp == 0) {
+            int at = 0;
+            for (int r0 = 0; r0 < R; r0 += 32) {
+                const int r = r0 + lane;
+                const int c = r < R ? __popc(msk[r][0]) + __popc(msk[r][1]) + __popc(msk[r][2]) + __popc(msk[r][3]) : 0;
+                int x = c;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += y;
+                }
+                if (r < R) base[r] = at + x - c;
+                at += __shfl_sync(0xffffffffu, x, 31);
+            }
+            if (lane == 0) base[R] = at;
+        }
+        __syncthreads();
+        const int total = min(base[R], cols * cols);
+        int r = 0;
+        for (int e = blockIdx.x; e < total; e += G) {
+            while (r + 1 < R && base[r + 1] <= e) ++r;
+            int left = e - base[r], k = 0;  // the left-th pair of round r
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+                const int c = __popc(msk[r][w]);
+                if (left >= 0 && left < c) {
+                    unsigned int b = msk[r][w];
+                    for (; left > 0; --left) b &= b - 1;
+                    k = 32 * w + __ffs(b) - 1;
+                    left = -1;
+                } else if (left >= 0) {
+                    left -= c;
+                }
+            }
+            int p = pos(k, r), q = pos(P - 1 - k, r);
+            if (p > q) { const int t = p; p = q; q = t; }
+            if (q >= cols) continue;
+            const int mine = lane == 0 ? p : q, rk = __ldcg(&sw->rank[mine][r]);
+            if (tid < 2) {  // thread 0 waits for column p, thread 1 for column q
+                volatile int* vd = &sw->done[mine];
+                volatile int* ve = bar.err;
+                long long spins = 0;
+                while (*vd < rk) {
+                    if (*ve) break;
+                    if (++spins > bar.limit) {
+                        atomicExch(bar.err, 1);
+                        break;
+                    }
+                }
+                __threadfence();
+            }
+            __syncthreads();
+            const bool rot = jacobi_pair_cta(rows, cols, A + (int64_t)p * rows, A + (int64_t)q * rows,
+                                             Vm + (int64_t)p * cols, Vm + (int64_t)q * cols, tol, low2, th2, red4, buf);
+            __syncthreads();  // the columns are written
+            if (tid < 2) {
+                if (rot) sw->changed[mine] = 1;
+                __threadfence();
+                *(volatile int*)&sw->done[mine] = rk + 1;
+            }
+        }
+        grid_barrier(bar, epoch);
+    }
+    if (blockIdx.x == 0 && tid == 0) *sweeps_out = sweep + 1;
+}
+
+// (every CTA finds the norms and ranks itself and writes its share of U and W)
 // sigma_i = |a_i|, descending order; U(:, r) = a_(i)/sigma, W(:, r) = V(:, i) for rank r of i.
 __global__ void svd_finish_kernel(int rows, int cols, const zd* __restrict__ A, const zd* __restrict__ Vm,
                                   zd* __restrict__ U, zd* __restrict__ W, double* __restrict__ sigma) {
@@ -415,16 +636,17 @@ __global__ void svd_finish_kernel(int rows, int cols, const zd* __restrict__ A, 
         int rank = 0;
         for (int k = 0; k < cols; ++k) rank += (nrm[k] > nrm[i]) || (nrm[k] == nrm[i] && k < i);
         rk[i] = rank;
-        sigma[rank] = nrm[i];
+        if (blockIdx.x == 0) sigma[rank] = nrm[i];
     }
     __syncthreads();
+    const int64_t e0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     if (U)
-        for (int64_t e = threadIdx.x; e < (int64_t)rows * cols; e += blockDim.x) {
+        for (int64_t e = e0; e < (int64_t)rows * cols; e += step) {
             const int i = (int)(e / rows), r = (int)(e - (int64_t)i * rows);
             const double inv = nrm[i] > 0 ? 1.0 / nrm[i] : 0.0;
             U[(int64_t)rk[i] * rows + r] = inv * A[e];
         }
-    for (int64_t e = threadIdx.x; e < (int64_t)cols * cols; e += blockDim.x) {
+    for (int64_t e = e0; e < (int64_t)cols * cols; e += step) {
         const int i = (int)(e / cols), r = (int)(e - (int64_t)i * cols);
         W[(int64_t)rk[i] * cols + r] = Vm[e];
     }
@@ -627,8 +849,10 @@ static bool launch_jacobi_cluster(int rows, int cols, zd* A, zd* Vm, int max_swe
     return false;
 }
 
-// A is destroyed; U (rows x cols) may be nullptr; W (cols x cols); sigma (cols).
-int jacobi_svd(int rows, int cols, zd* A, zd* U, zd* W, double* sigma, JacobiWork w, cudaStream_t st) {
+// A is destroyed; U (rows x cols) may be nullptr; W (cols x cols); sigma (cols). low, theta > 0 (with
+// w.screen): the relaxed rule of jacobi_screened_kernel for columns of norm <= low |A(0,0)|.
+static int jacobi_svd_run(int rows, int cols, zd* A, zd* U, zd* W, double* sigma, JacobiWork w, double low,
+                          double theta, cudaStream_t st) {
     if (cols <= 0) return NEP_OK;
     NEP_CUDA(cudaMemsetAsync(w.flags, 0, 2 * sizeof(int), st));
     NEP_CUDA(cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), st));
@@ -648,14 +872,28 @@ int jacobi_svd(int rows, int cols, zd* A, zd* U, zd* W, double* sigma, JacobiWor
     // rotation angle is rounding noise
     double tol = std::max(rows, 1) * 2.220446049250313e-16;
     // the cooperative grid, or one cluster with distributed shared memory where asked for and it fits
-    if (!launch_jacobi_cluster(rows, cols, A, w.Vm, max_sweeps, tol, w.sweeps, st)) {
+    if (low > 0.0 && w.screen && rows <= kScreenMax && cols <= kScreenMax) {
+        NEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_screened_kernel, 128, 0));
+        blocks = std::max(1, std::min(P / 2, sms * std::max(per_sm, 1)));
+        double low2 = low * low, th2 = theta * theta;
+        ScreenWork* sw = static_cast<ScreenWork*>(w.screen);
+        max_sweeps = 60;
+        void* args[] = {&rows, &cols, &A, &w.Vm, &max_sweeps, &tol, &low2, &th2, &sw, &w.sweeps, &gb};
+        NEP_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_screened_kernel, dim3(blocks), dim3(128), args, 0, st));
+        count_launch();
+    } else if (!launch_jacobi_cluster(rows, cols, A, w.Vm, max_sweeps, tol, w.sweeps, st)) {
         void* args[] = {&rows, &cols, &A, &w.Vm, &max_sweeps, &tol, &w.flags, &w.sweeps, &gb};
         NEP_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_kernel, dim3(blocks), dim3(tpb), args, 0, st));
         count_launch();
     }
-    svd_finish_kernel<<<1, 256, (sizeof(double) + sizeof(int)) * cols, st>>>(rows, cols, A, w.Vm, U, W, sigma);
+    const int fin = std::max(1, std::min(16, ceil_div((int64_t)rows * cols, 2048)));
+    svd_finish_kernel<<<fin, 256, (sizeof(double) + sizeof(int)) * cols, st>>>(rows, cols, A, w.Vm, U, W, sigma);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
+}
+
+int jacobi_svd(int rows, int cols, zd* A, zd* U, zd* W, double* sigma, JacobiWork w, cudaStream_t st) {
+    return jacobi_svd_run(rows, cols, A, U, W, sigma, w, 0.0, 0.0, st);
 }
 
 // ------------------------------------------------------------------ QR with column pivoting
@@ -792,12 +1030,16 @@ __global__ void __launch_bounds__(32) qrcp_kernel(int rows, int cols, zd* __rest
 // k and p exchange them through their swap buffers; the owner of column k builds the reflector;
 // every CTA copies it and applies H_k^H to its columns j > k, one warp per column with the lane
 // order of qrcp_kernel, and recomputes their remaining norms. On exit A, tau, perm and the step
-// count are as qrcp_kernel leaves them.
+// count are as qrcp_kernel leaves them, except that it also stops, with kQrcpKept added to the step
+// count, once ||R_22||_F^2 <= keep2 |R_00|^2 within the first 2/5 of the columns: R_22 is then a full block
+// that the caller keeps. (Later, dropping the columns below stop2 saves more than their reduction costs.)
+constexpr int kQrcpKept = 1 << 30;
 constexpr int kQrcpClusterThreads = 128;
 namespace cg = cooperative_groups;
 __global__ void __launch_bounds__(kQrcpClusterThreads) qrcp_cluster_kernel(int rows, int cols, zd* __restrict__ A,
                                                                            zd* __restrict__ tau,
                                                                            int* __restrict__ perm, double stop2,
+                                                                           double keep2,
                                                                            int* __restrict__ steps_out) {
     cg::cluster_group cluster = cg::this_cluster();
     const int CS = (int)cluster.num_blocks();
@@ -831,6 +1073,7 @@ __global__ void __launch_bounds__(kQrcpClusterThreads) qrcp_cluster_kernel(int r
     }
     const int steps = min(rows, cols);
     int done = steps;
+    bool kept = false;
     for (int k = 0; k < steps; ++k) {
         __syncthreads();
         if (warp == 0) {  // this CTA's best remaining column and the sum of its remaining norms
@@ -875,12 +1118,13 @@ __global__ void __launch_bounds__(kQrcpClusterThreads) qrcp_cluster_kernel(int r
                 if (bi >= cols) bi = k;  // NaN norms match no column
                 if (k == 0) b_first = best;
                 b_p = bi;
-                b_stop = rest <= stop2 * b_first;
+                b_stop = rest <= stop2 * b_first ? 1 : (5 * k <= 2 * cols && rest <= keep2 * b_first) ? 2 : 0;
             }
         }
         cluster.sync();  // every CTA has read the slots before they are written again
         if (b_stop) {
             done = k;
+            kept = b_stop == 2;
             break;
         }
         const int p = b_p;
@@ -977,15 +1221,15 @@ __global__ void __launch_bounds__(kQrcpClusterThreads) qrcp_cluster_kernel(int r
     }
     if (rank == 0) {
         for (int k = done + tid; k < steps; k += blockDim.x) tau[k] = mk(0.0, 0.0);  // H_k = I beyond the stop
-        if (tid == 0) *steps_out = done;
+        if (tid == 0) *steps_out = done + (kept ? kQrcpKept : 0);
     }
     cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
 // Launches qrcp_cluster_kernel on the largest cluster the GPU takes (16 or 8 CTAs) whose columns
 // fit in shared memory; returns false (nothing launched) when none does.
-static bool launch_qrcp_cluster(int rows, int cols, zd* A, zd* tau, int* perm, double stop2, int* steps_dev,
-                                cudaStream_t st) {
+static bool launch_qrcp_cluster(int rows, int cols, zd* A, zd* tau, int* perm, double stop2, double keep2,
+                                int* steps_dev, cudaStream_t st) {
     // 16 if non-portable cluster sizes are accepted, else 8 (set once, thread-safe), and the dynamic
     // shared memory limit raised once to the opt-in maximum: a per-call limit races between host
     // threads launching different sizes
@@ -1022,7 +1266,7 @@ static bool launch_qrcp_cluster(int rows, int cols, zd* A, zd* tau, int* perm, d
             cudaGetLastError();
             continue;
         }
-        if (cudaLaunchKernelEx(&cfg, qrcp_cluster_kernel, rows, cols, A, tau, perm, stop2, steps_dev) != cudaSuccess) {
+        if (cudaLaunchKernelEx(&cfg, qrcp_cluster_kernel, rows, cols, A, tau, perm, stop2, keep2, steps_dev) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
@@ -1032,12 +1276,12 @@ static bool launch_qrcp_cluster(int rows, int cols, zd* A, zd* tau, int* perm, d
     return false;
 }
 
-// R^H of the upper triangle of A (n x n): Rh(i, j) = conj(A(j, i)) for i >= j, 0 above.
-__global__ void rh_from_qr_kernel(int n, int ncols, const zd* __restrict__ A, zd* __restrict__ Rh) {
+// R^H after nref steps of the QR (n x n): Rh(i, j) = conj(A(j, i)) for i >= min(j, nref), 0 above.
+__global__ void rh_from_qr_kernel(int n, int ncols, int nref, const zd* __restrict__ A, zd* __restrict__ Rh) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)n * ncols) return;
     const int i = (int)(t % n), j = (int)(t / n);
-    Rh[t] = i >= j ? conj(A[j + (int64_t)n * i]) : mk(0.0, 0.0);
+    Rh[t] = i >= min(j, nref) ? conj(A[j + (int64_t)n * i]) : mk(0.0, 0.0);
 }
 
 // U(:, c) = [Wj(:, c); 0] for c < mq (Wj: mq x mq), zero columns c >= mq of U and W, sigma[c] = 0
@@ -1103,8 +1347,13 @@ __global__ void permute_rows_kernel(int n, int ncols, const int* __restrict__ pe
 // norm <= trunc |R_00|: its rows of R are dropped, which moves every singular value by at most
 // ||R_22||_2 <= trunc |R_00| <= trunc sigma_1 (Weyl), and Jacobi runs on the n x mq matrix
 // R(0:mq, :)^H only. Singular values and vectors beyond mq are returned as zero.
+// With keep > trunc (and w.screen, n <= 256) the QR already stops where ||R_22||_F <= keep |R_00|, and Jacobi
+// takes the unreduced block with the rest: columns that small only need their singular values
+// (jacobi_screened_kernel's relaxed rule), for which reducing them further is wasted. Their U and W columns
+// are then not orthogonal to full accuracy; those of larger columns are.
 int qrcp_jacobi_svd(int n, zd* A, zd* U, zd* W, double* sigma, zd* work1, zd* work2, zd* work3, zd* tau, int* perm,
-                    double* nrm2, int* steps_dev, int* steps_host, double trunc, JacobiWork w, cudaStream_t st) {
+                    double* nrm2, int* steps_dev, int* steps_host, double trunc, double keep, JacobiWork w,
+                    cudaStream_t st) {
     if (n <= 0) return NEP_OK;
     NEP_CUDA(cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), st));
     int dev = 0, sms = 0;
@@ -1116,25 +1365,30 @@ int qrcp_jacobi_svd(int n, zd* A, zd* U, zd* W, double* sigma, zd* work1, zd* wo
     GridBar gb{w.bar, w.bar + 1, w.err, wait_limit()};
     int rows = n, cols = n;
     double stop2 = trunc * trunc;
+    // (NEP_JACOBI_CLUSTER=1 keeps the full sweeps, on one cluster)
+    const char* jc = std::getenv("NEP_JACOBI_CLUSTER");
+    const bool screen = w.screen && n <= kScreenMax && keep > trunc && !(jc && jc[0] == '1');
     // one cluster with distributed shared memory where it fits, else the cooperative grid
-    if (!launch_qrcp_cluster(rows, cols, A, tau, perm, stop2, steps_dev, st)) {
+    if (!launch_qrcp_cluster(rows, cols, A, tau, perm, stop2, screen ? keep * keep : 0.0, steps_dev, st)) {
         void* args[] = {&rows, &cols, &A, &tau, &perm, &nrm2, &stop2, &steps_dev, &gb};
         NEP_CUDA(cudaLaunchCooperativeKernel((const void*)qrcp_kernel, dim3(blocks), dim3(32), args, 0, st));
         count_launch();
     }
     NEP_CUDA(cudaMemcpyAsync(steps_host, steps_dev, sizeof(int), cudaMemcpyDeviceToHost, st));
     NEP_CUDA(cudaStreamSynchronize(st));
-    const int mq = std::max(0, std::min(n, *steps_host));
+    const bool kept = (*steps_host & kQrcpKept) != 0;
+    const int nref = std::max(0, std::min(n, *steps_host & ~kQrcpKept));
+    const int mq = kept ? n : nref;
     if (mq > 0) {
-        rh_from_qr_kernel<<<ceil_div((int64_t)n * mq, 256), 256, 0, st>>>(n, mq, A, work1);
+        rh_from_qr_kernel<<<ceil_div((int64_t)n * mq, 256), 256, 0, st>>>(n, mq, nref, A, work1);
         NEP_CHECK_LAUNCH();
         // Jacobi on R(0:mq, :)^H: work1 -> Uj (work2, n x mq), Wj (work3, mq x mq)
-        NEP_TRY(jacobi_svd(n, mq, work1, work2, work3, sigma, w, st));
+        NEP_TRY(jacobi_svd_run(n, mq, work1, work2, work3, sigma, w, kept ? keep : 0.0, 0.2 * trunc, st));
     }
     qr_pad_kernel<<<ceil_div((int64_t)n * n, 256), 256, 0, st>>>(n, mq, work3, U, W, sigma);
     NEP_CHECK_LAUNCH();
     if (mq > 0) {
-        apply_q_kernel<<<ceil_div(mq, 4), 128, 0, st>>>(n, mq, A, tau, mq, U);
+        apply_q_kernel<<<ceil_div(mq, 4), 128, 0, st>>>(n, nref, A, tau, mq, U);
         NEP_CHECK_LAUNCH();
         permute_rows_kernel<<<ceil_div((int64_t)n * mq, 256), 256, 0, st>>>(n, mq, perm, work2, W);
         NEP_CHECK_LAUNCH();

@@ -765,6 +765,7 @@ static int plan_alloc(nep_plan* p) {
     NEP_TRY(dalloc(&p->jw.sweeps, 1, st));
     NEP_TRY(dalloc(&p->jw.bar, 2, st));
     NEP_TRY(dalloc(&p->jw.err, 1, st));
+    if (jacobi_screen_bytes(LM)) NEP_TRY(dalloc_raw(&p->jw.screen, jacobi_screen_bytes(LM), st));
     if (g_dry) return NEP_OK;
     NEP_CUDA(cudaMemsetAsync(p->jw.err, 0, sizeof(int), st));
     p->h_pinned = pinned_slot_get();
@@ -780,7 +781,7 @@ static void plan_free(nep_plan* p) {
                     p->H, p->Hs, p->Hw, p->U, p->W, p->sigma, p->T1, p->Bred, p->theta, p->Tv, p->Z, p->cand,
                     p->XH, p->G, p->Gw, p->Wg, p->lamg, p->Q, p->Y0, p->AQ, p->Bs, p->lamn, p->Yn, p->Xc, p->Gx,
                     p->ok, p->its, p->order, p->scalars, p->eigstat, p->eta, p->part, p->newton_scratch, p->bs32,
-                    p->eig_scratch, p->jw.Vm, p->jw.flags, p->jw.sweeps, p->jw.bar, p->jw.err};
+                    p->eig_scratch, p->jw.Vm, p->jw.flags, p->jw.sweeps, p->jw.bar, p->jw.err, p->jw.screen};
     for (void* b : bufs)
         if (b) cudaFreeAsync(b, st);
     cudaStreamSynchronize(st);
@@ -1236,8 +1237,11 @@ static int run_extract(nep_plan* p, cudaStream_t st) {
     // sigma_1, the size of the FP64 rounding error of a dense SVD of this order (n eps sigma_1),
     // and Jacobi runs only on the numerically nonzero part
     const double trunc = std::min(1e-14, 1e-2 * p->o.rank_tol);
+    // columns this small (a tenth of the rank threshold at most) fall below the rank: only their
+    // singular values are wanted
+    const double keep = std::min(1e-13, 0.1 * p->o.rank_tol);
     NEP_TRY(qrcp_jacobi_svd(LM, p->Hw, p->U, p->W, p->sigma, p->T1, p->Bred, p->Tv, p->theta, p->its, p->lamg,
-                            p->scalars + 2, p->h_pinned + 8, trunc, p->jw, st));
+                            p->scalars + 2, p->h_pinned + 8, trunc, keep, p->jw, st));
     NEP_TRY(launch_rank(LM, p->sigma, p->o.rank_tol, p->scalars, st));
     int m = 0;
     NEP_TRY(read_scalar(p, p->scalars, &m, st));

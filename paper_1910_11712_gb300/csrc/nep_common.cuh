@@ -339,10 +339,12 @@ struct JacobiWork {
     int* sweeps;
     unsigned* bar;
     int* err;
+    void* screen = nullptr;  // jacobi_screen_bytes: pair screening of the Hankel SVD (optional)
 };
 int jacobi_svd(int rows, int cols, zd* A, zd* U, zd* W, double* sigma, JacobiWork w, cudaStream_t st);
 int qrcp_jacobi_svd(int n, zd* A, zd* U, zd* W, double* sigma, zd* work1, zd* work2, zd* work3, zd* tau, int* perm,
-                    double* nrm2, int* steps_dev, int* steps_host, double trunc, JacobiWork w, cudaStream_t st);
+                    double* nrm2, int* steps_dev, int* steps_host, double trunc, double keep, JacobiWork w, cudaStream_t st);
+size_t jacobi_screen_bytes(int n);
 template <typename T>
 int small_eig(int m, const zd* A, zd* eval, zd* evec, int* status, void* gbuf, cudaStream_t st);
 template <typename T>
