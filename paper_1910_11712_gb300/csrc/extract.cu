@@ -1031,8 +1031,11 @@ __global__ void __launch_bounds__(32) qrcp_kernel(int rows, int cols, zd* __rest
 // every CTA copies it and applies H_k^H to its columns j > k, one warp per column with the lane
 // order of qrcp_kernel, and recomputes their remaining norms. On exit A, tau, perm and the step
 // count are as qrcp_kernel leaves them, except that it also stops, with kQrcpKept added to the step
-// count, once ||R_22||_F^2 <= keep2 |R_00|^2 within the first 2/5 of the columns: R_22 is then a full block
-// that the caller keeps. (Later, dropping the columns below stop2 saves more than their reduction costs.)
+// count, once ||R_22||_F^2 <= keep2 |R_00|^2 has stopped falling (by less than half in kQrcpWindow steps: flat
+// rounding noise) within the first 3/8 of the columns: R_22 is then a full block that the caller keeps.
+// (Where it still falls, as with FP64 solves, a few more steps reach stop2 and leave a small matrix; later
+// than 3/8, dropping the columns below stop2 saves more than their reduction costs.)
+constexpr int kQrcpWindow = 4;
 constexpr int kQrcpKept = 1 << 30;
 constexpr int kQrcpClusterThreads = 128;
 namespace cg = cooperative_groups;
@@ -1052,7 +1055,7 @@ __global__ void __launch_bounds__(kQrcpClusterThreads) qrcp_cluster_kernel(int r
     zd* swp = vloc + rows;                       // rows: swap buffer
     double* lnorm = reinterpret_cast<double*>(swp + rows);  // ncl
     int* lperm = reinterpret_cast<int*>(lnorm + ncl);       // ncl
-    __shared__ double slot_best, slot_rest, b_first;
+    __shared__ double slot_best, slot_rest, b_first, hist[kQrcpWindow];
     __shared__ int slot_idx, swp_perm, b_p, b_stop;
     __shared__ zd tau_s, tau_b;
     auto col = [&](int c) { return colm + (size_t)c * rows; };
@@ -1118,7 +1121,10 @@ __global__ void __launch_bounds__(kQrcpClusterThreads) qrcp_cluster_kernel(int r
                 if (bi >= cols) bi = k;  // NaN norms match no column
                 if (k == 0) b_first = best;
                 b_p = bi;
-                b_stop = rest <= stop2 * b_first ? 1 : (5 * k <= 2 * cols && rest <= keep2 * b_first) ? 2 : 0;
+                const double before = k >= kQrcpWindow ? hist[k % kQrcpWindow] : 1e300;
+                hist[k % kQrcpWindow] = rest;
+                b_stop = rest <= stop2 * b_first ? 1
+                         : (8 * k <= 3 * cols && rest <= keep2 * b_first && rest > 0.5 * before) ? 2 : 0;
             }
         }
         cluster.sync();  // every CTA has read the slots before they are written again

@@ -28,8 +28,10 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <cooperative_groups.h>
 #include <cstdlib>
 #include <mutex>
+#include <type_traits>
 
 #include "band_util.cuh"
 #include "tc_ptx.cuh"
@@ -57,19 +59,181 @@ __device__ __forceinline__ void tile_rk(int f, int& r, int& k) {
 }
 }  // namespace
 
-size_t lu_tc_smem(int kl) {
-    const size_t rw = (size_t)kl + NB;
-    const size_t early = 8 * rw * NB;
+// Scratch beside the panel (step 2): each warp's 8 columns of U12 on their way to the output rows.
+namespace {
+constexpr int CST = NB + 1, CCOLS = 8;                           // a warp's U12 columns: CCOLS x CST
+constexpr size_t STAGE_BYTES = 8 * (size_t)16 * CCOLS * CST;     // 33 KB
+// bytes of the region shared by the steps, with the scratch or without
+__host__ __device__ inline size_t region_bytes(int kl, bool scratch) {
+    const size_t early = 8 * ((size_t)kl + NB) * NB + (scratch ? STAGE_BYTES : 0);
     const size_t late = 3 * (size_t)TILE_BYTES;
-    return 1024 + (early > late ? early : late) + sizeof(int) * (rw + NB);
+    return early > late ? early : late;
+}
+}  // namespace
+
+static size_t lu_tc_smem_of(int kl, bool scratch) {
+    return 1024 + region_bytes(kl, scratch) + sizeof(int) * ((size_t)kl + 2 * NB);
+}
+// bands whose panel and scratch fit (kl <= 700)
+static bool lu_tc_scratch(int kl) { return lu_tc_smem_of(kl, true) <= 224 * 1024; }
+size_t lu_tc_smem(int kl) { return lu_tc_smem_of(kl, lu_tc_scratch(kl)); }
+
+// The panel in shared memory with one barrier per column step. Rows stay where they are and carry their
+// index as a label: the pivot's label becomes k, row k's label the pivot's. Each warp holds one or two groups
+// of 32 rows (all of them for a share of the columns where there are fewer groups than warps); at step k it
+// finds the pivot among the groups' candidates, reads the pivot row in place (nobody writes it), and updates
+// its rows, column k + 1 first, whose candidates for the next pivot it publishes before the rest. The
+// column below the pivot keeps its values, so that every warp can form the multipliers itself; they are
+// scaled at the end, when the rows move to their labels' places. The operations per element are those of
+// a panel that swaps and scales at every step. At 160 rows the step's chain (pivot search, reciprocal,
+// one column) bounds it, not the 31 columns' arithmetic.
+constexpr int PW16 = 16;  // warps
+// a b, rounded the same wherever it is formed
+__device__ __forceinline__ zf mul_cx(zf a, zf b) {
+    return mk(__fmaf_rn(a.re, b.re, -__fmul_rn(a.im, b.im)), __fmaf_rn(a.re, b.im, __fmul_rn(a.im, b.re)));
+}
+template <int NR>  // row groups per warp: 1 (up to 512 rows) or 2
+__device__ __forceinline__ void panel_smem(int nbc, int pr, int RW, int kl, int kv, int ldab, int p0, bool writer,
+                                           zf* Ps, zf* ab, int* ipiv, int* piv_sh, int* info_s, unsigned (*wkey)[PW16],
+                                           int (*wlab)[PW16], int (*wphys)[PW16], int* diag_s, zf* rpv_sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int RG = (RW + 31) / 32;                 // row groups
+    const int CG = RG < PW16 ? PW16 / RG : 1;      // shares of the columns
+    const int cg = RG < PW16 ? warp / RG : 0;
+    const bool on = cg < CG;
+    int row[NR], lab[NR];
+#pragma unroll
+    for (int t = 0; t < NR; ++t) {
+        row[t] = t == 0 ? 32 * (RG < PW16 ? warp % RG : warp) + lane : 32 * (warp + PW16) + lane;
+        if (!on || row[t] >= RW) row[t] = -1;
+        lab[t] = row[t];
+    }
+    // candidates for pivot k: first row maximising |Re|+|Im| among labels k .. last (no NaN)
+    auto publish = [&](int k, const zf (&v)[NR]) __attribute__((always_inline)) {
+        const int last = min(k + kl, pr - 1), buf = k & 1;
+        unsigned key = 0;
+        int cl = 0x7fffffff, ph = 0;
+#pragma unroll
+        for (int t = 0; t < NR; ++t) {
+            if (row[t] < 0 || lab[t] < k || lab[t] > last) continue;
+            const float m = abs1(v[t]);
+            const unsigned mb = __float_as_uint(m);
+            if (m >= 0.0f && (mb > key || (mb == key && lab[t] < cl))) key = mb, cl = lab[t], ph = row[t];
+            if (lab[t] == k) diag_s[buf] = row[t];
+        }
+        const unsigned mx = __reduce_max_sync(0xffffffffu, key);
+        const int pl = (int)__reduce_min_sync(0xffffffffu, key == mx ? (unsigned)cl : 0x7fffffffu);
+        if (key == mx && cl == pl && pl != 0x7fffffff) wphys[buf][warp] = ph;
+        if (lane == 0) wkey[buf][warp] = mx, wlab[buf][warp] = pl;
+    };
+    if (tid < 2 * PW16) wkey[tid >> 4][tid & 15] = 0, wlab[tid >> 4][tid & 15] = 0x7fffffff;
+    __syncthreads();
+    if (cg == 0) {
+        zf v[NR];
+#pragma unroll
+        for (int t = 0; t < NR; ++t) v[t] = row[t] >= 0 ? Ps[row[t]] : mk(0.0f, 0.0f);
+        publish(0, v);
+    }
+#pragma unroll 1
+    for (int k = 0; k < nbc; ++k) {
+        const int last = min(k + kl, pr - 1), buf = k & 1;
+        __syncthreads();
+        const unsigned key = wkey[buf][lane & 15];
+        const int cl = wlab[buf][lane & 15];
+        const unsigned mx = __reduce_max_sync(0xffffffffu, key);
+        int pl = (int)__reduce_min_sync(0xffffffffu, key == mx ? (unsigned)cl : 0x7fffffffu);
+        const unsigned who = __ballot_sync(0xffffffffu, key == mx && cl == pl);
+        int ph = wphys[buf][(__ffs(who) - 1) & 15];
+        if (pl > last) pl = k, ph = diag_s[buf];  // a column of NaNs: keep the diagonal
+        const zf* prow = Ps + ph;
+        const zf pv = prow[RW * k];
+        const bool zero = pv.re == 0.0f && pv.im == 0.0f;  // then every candidate is zero: pl == k
+        const zf rpv = zero ? mk(0.0f, 0.0f) : pivot_recip(pv);
+        if (tid == 0) {
+            rpv_sh[k] = rpv;
+            piv_sh[k] = p0 + pl;
+            if (writer) ipiv[p0 + k] = p0 + pl;
+            if (zero && *info_s == 0) *info_s = p0 + k + 1;
+        }
+        zf l[NR];
+        bool act[NR];
+#pragma unroll
+        for (int t = 0; t < NR; ++t) {
+            if (row[t] >= 0) lab[t] = lab[t] == pl ? k : lab[t] == k ? pl : lab[t];
+            act[t] = row[t] >= 0 && lab[t] > k && lab[t] <= last;
+            l[t] = act[t] ? mul_cx(Ps[row[t] + RW * k], rpv) : mk(0.0f, 0.0f);
+        }
+        if (cg == 0 && k + 1 < nbc) {
+            const zf u = prow[RW * (k + 1)];
+            zf v[NR];
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                v[t] = mk(0.0f, 0.0f);
+                if (row[t] < 0) continue;
+                v[t] = Ps[row[t] + RW * (k + 1)];
+                if (act[t]) {
+                    v[t] = fms(v[t], l[t], u);
+                    Ps[row[t] + RW * (k + 1)] = v[t];
+                }
+            }
+            publish(k + 1, v);
+        }
+        if (on) {
+            if (writer && cg == CG - 1) {
+                zf* out = ab + (int64_t)(p0 + k) * ldab + kv + 1;
+#pragma unroll
+                for (int t = 0; t < NR; ++t)
+                    if (row[t] >= 0 && lab[t] > k && lab[t] <= k + kl) out[lab[t] - k - 1] = l[t];
+            }
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                if (!act[t]) continue;
+                const int q0 = k + 1 + (cg == 0 ? CG : cg), st = RW * CG;
+                zf* pc = Ps + row[t] + RW * q0;
+                const zf* pu = prow + RW * q0;
+#pragma unroll 4
+                for (int q = q0; q < nbc; q += CG, pc += st, pu += st) *pc = fms(*pc, l[t], *pu);
+            }
+        }
+    }
+    __syncthreads();
+    // rows to their labels' places, multipliers scaled, half the columns at a time
+    int r[NR], d[NR];
+#pragma unroll
+    for (int t = 0; t < NR; ++t) {
+        r[t] = cg == 0 ? row[t] : -1;
+        d[t] = lab[t];
+    }
+#pragma unroll 1
+    for (int h = 0; h < NB; h += 8) {
+        zf b[NR][8];
+#pragma unroll
+        for (int t = 0; t < NR; ++t)
+            if (r[t] >= 0)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    b[t][q] = Ps[r[t] + RW * (h + q)];
+                    if (h + q < nbc && h + q < d[t]) b[t][q] = mul_cx(b[t][q], rpv_sh[h + q]);
+                }
+        __syncthreads();
+#pragma unroll
+        for (int t = 0; t < NR; ++t)
+            if (r[t] >= 0)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) Ps[d[t] + RW * (h + q)] = b[t][q];
+        __syncthreads();
+    }
 }
 
 __global__ void __launch_bounds__(512, 1)
     lu_tc_kernel(int n, int kl, int ku, int ldab, zf* __restrict__ ab_all, int* __restrict__ ipiv_all,
                  int* __restrict__ info_all, const int* __restrict__ active, zf* __restrict__ win_all, int RWp,
                  int CWp, float* __restrict__ aimg_all, int nmt_max, const __grid_constant__ CUtensorMap tmap,
-                 int* __restrict__ err, const PointDesc* __restrict__ pd, int passes) {
-    const int j = blockIdx.x;  // also the point's operand image and its TMA coordinate
+                 int* __restrict__ err, const PointDesc* __restrict__ pd, int passes, int nsplit, int scratch_max_kl) {
+    // nsplit CTAs (a cluster) per point: each factors the panel itself and takes its share of the
+    // trailing columns; CTA 0 writes the panel's outputs. Each CTA has an operand image of its own.
+    const int j = blockIdx.x / nsplit, part = blockIdx.x - j * nsplit;
+    const int img = blockIdx.x;  // operand image and its TMA coordinate
     zf* ab = ab_all + (int64_t)j * n * ldab;
     int* ipiv = ipiv_all + (int64_t)j * n;
     int* info_out = info_all + j;
@@ -86,8 +250,13 @@ __global__ void __launch_bounds__(512, 1)
     const int kv = kl + ku;
     const int RW = kl + NB;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nthr = blockDim.x, nwarp = nthr >> 5;
-    float* aimg = aimg_all + (int64_t)j * nmt_max * (TILE_BYTES / 4);
-    auto wi = [&](int r, int c) -> int64_t { return (int64_t)(r % RWp) + (int64_t)RWp * (c % CWp); };
+    float* aimg = aimg_all + (int64_t)img * nmt_max * (TILE_BYTES / 4);
+    const bool fast = kl <= scratch_max_kl;  // the scratch fits beside the panel
+    // window slots of row p0 + i and column p0 + q of the current panel (rb, cbs: those of p0)
+    int rb = 0, cbs = 0;
+    auto rs = [&](int i) { return rb + i >= RWp ? rb + i - RWp : rb + i; };
+    auto cs_ = [&](int q) { return cbs + q >= CWp ? cbs + q - CWp : cbs + q; };
+    auto wi = [&](int i, int q) { return rs(i) + RWp * cs_(q); };
 
     extern __shared__ unsigned char smem_raw[];
     unsigned char* R = smem_raw + ((1024 - (tc::smem_u32(smem_raw) & 1023)) & 1023);
@@ -95,13 +264,14 @@ __global__ void __launch_bounds__(512, 1)
     float* Bimg = reinterpret_cast<float*>(R);                           // step 4: B (hi, lo)
     float* Abuf0 = reinterpret_cast<float*>(R + TILE_BYTES);             // step 4: A tiles
     float* Abuf1 = reinterpret_cast<float*>(R + 2 * TILE_BYTES);
-    const size_t early = 8 * (size_t)RW * NB;
-    const size_t region = early > 3 * (size_t)TILE_BYTES ? early : 3 * (size_t)TILE_BYTES;
-    int* src = reinterpret_cast<int*>(R + region);
+    zf* scr = Ps + (size_t)RW * NB;           // scratch of steps 1 and 2 (fast)
+    int* src = reinterpret_cast<int*>(R + region_bytes(kl, fast));
     int* plist = src + RW;
     __shared__ int piv_sh[NB];
     __shared__ int info_s, npart_s, abort_s;
-    __shared__ zf rpv_s;
+    __shared__ zf rpv_sh[NB];
+    __shared__ unsigned wkey[2][PW16];
+    __shared__ int wlab[2][PW16], wphys[2][PW16], diag_s[2];
     __shared__ uint32_t tmem_s;
     __shared__ __align__(8) uint64_t full_b[2], done_b[2], free_b[2];
 
@@ -148,91 +318,46 @@ __global__ void __launch_bounds__(512, 1)
         for (int r = r0 + warp; r < r1; r += nwarp) {
             const zf* srow = ab + (int64_t)r * ldab - (r - kl);  // srow[c] = A(r, c)
             const int clo = max(r - kl, 0), chi = min(r + ku, n - 1);
-            for (int c = clo + lane; c <= chi; c += 32) W[wi(r, c)] = srow[c];
+            for (int c = clo + lane; c <= chi; c += 32) W[wi(r, c)] = srow[c];  // (the first rows: no wrap)
         }
     };
-    for (int64_t e = tid; e < (int64_t)RWp * CWp; e += nthr) W[e] = mk(0.0f, 0.0f);
-    __syncthreads();
-    load_rows(0, min(RW, n));
-    __syncthreads();
+    auto csync = [&]() {  // every CTA of the point: window writes before it are visible after it
+        if (nsplit > 1) cooperative_groups::this_cluster().sync();
+        else __syncthreads();
+    };
+    for (int64_t e = tid + (int64_t)part * nthr; e < (int64_t)RWp * CWp; e += (int64_t)nsplit * nthr) W[e] = mk(0.0f, 0.0f);
+    csync();
+    if (part == 0) load_rows(0, min(RW, n));
+    csync();
 
     for (int p0 = 0; p0 < n; p0 += NB) {
         const int nbc = min(NB, n - p0);
         const int pr = min(RW, n - p0);
+        rb = p0 % RWp, cbs = p0 % CWp;
 
         // ---- 0. panel columns to shared memory (eight independent loads per lane, then the stores)
         for (int q = warp; q < nbc; q += nwarp) {
-            const zf* wc = W + (int64_t)RWp * ((p0 + q) % CWp);
+            const zf* wc = W + RWp * cs_(q);
             for (int i0 = 0; i0 < RW; i0 += 256) {
                 zf v[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int i = i0 + lane + 32 * u;
-                    v[u] = i < pr ? wc[(p0 + i) % RWp] : mk(0.0f, 0.0f);
+                    v[u] = i < pr ? wc[rs(i)] : mk(0.0f, 0.0f);
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int i = i0 + lane + 32 * u;
-                    if (i < RW) Ps[i + (int64_t)RW * q] = v[u];
+                    if (i < RW) Ps[i + RW * q] = v[u];
                 }
             }
         }
         __syncthreads();
-
-        // ---- 1. panel factorisation (pivot: first row maximising |Re|+|Im| among rows k .. k+kl)
-        for (int k = 0; k < nbc; ++k) {
-            const int c = p0 + k;
-            const int last = min(k + kl, pr - 1), cnt = last - k + 1;
-            zf* colk = Ps + (int64_t)RW * k;
-            if (warp == 0) {
-                float best = -1.0f;
-                int bi = 0x7fffffff;
-                for (int i = lane; i < cnt; i += 32) {
-                    const float m = abs1(colk[k + i]);
-                    if (m > best) { best = m; bi = i; }
-                }
-                const unsigned mb = best < 0 ? 0u : __float_as_uint(best);
-                const unsigned mx = __reduce_max_sync(0xffffffffu, mb);
-                int p = (int)__reduce_min_sync(0xffffffffu, mb == mx ? (unsigned)bi : 0xffffffffu);
-                if (p >= cnt) p = 0;  // a column of NaNs matches no row: keep the diagonal
-                const zf pv = colk[k + p];
-                const bool zero = pv.re == 0.0f && pv.im == 0.0f;
-                if (zero) p = 0;
-                if (p != 0)
-                    for (int q = lane; q < nbc; q += 32) {
-                        zf* pq = Ps + (int64_t)RW * q;
-                        const zf t = pq[k];
-                        pq[k] = pq[k + p];
-                        pq[k + p] = t;
-                    }
-                if (lane == 0) {
-                    ipiv[c] = c + p;
-                    piv_sh[k] = c + p;
-                    if (zero && info_s == 0) info_s = c + 1;
-                    rpv_s = zero ? mk(0.0f, 0.0f) : cdiv(mk(1.0f, 0.0f), pv);
-                }
-            }
-            __syncthreads();
-            {
-                const zf rpv = rpv_s;
-                zf* out = ab + (int64_t)c * ldab + kv + 1;
-                for (int i = tid; i < kl; i += nthr) {
-                    zf l = mk(0.0f, 0.0f);
-                    if (k + 1 + i <= last) {
-                        l = colk[k + 1 + i] * rpv;
-                        colk[k + 1 + i] = l;
-                    }
-                    out[i] = l;
-                }
-            }
-            __syncthreads();
-            for (int q = k + 1 + warp; q < nbc; q += nwarp) {
-                zf* pq = Ps + (int64_t)RW * q;
-                const zf u = pq[k];
-                for (int i = k + 1 + lane; i <= last; i += 32) pq[i] = fms(pq[i], colk[i], u);
-            }
-            __syncthreads();
-        }
+        // ---- 1. panel factorisation
+        if (RW <= 32 * PW16)
+            panel_smem<1>(nbc, pr, RW, kl, kv, ldab, p0, part == 0, Ps, ab, ipiv, piv_sh, &info_s, wkey, wlab, wphys, diag_s, rpv_sh);
+        else
+            panel_smem<2>(nbc, pr, RW, kl, kv, ldab, p0, part == 0, Ps, ab, ipiv, piv_sh, &info_s, wkey, wlab, wphys, diag_s, rpv_sh);
 
         // ---- the panel's interchanges as one permutation: local row l receives old row src[l]
         for (int l = tid; l < RW; l += nthr) src[l] = l;
@@ -258,6 +383,9 @@ __global__ void __launch_bounds__(512, 1)
         const int npart = npart_s;
         const int cend = min(p0 + nbc + kv, n), rend = min(p0 + nbc + kl, n);
         const int mr = rend - (p0 + nbc);
+        // this CTA's trailing columns [clo, chi)
+        const int ctot = cend - (p0 + nbc), cmid = nsplit > 1 ? (ctot / 2 + 15) / 16 * 16 : 0;
+        const int clo = p0 + nbc + (part ? min(cmid, ctot) : 0), chi = nsplit > 1 && part == 0 ? p0 + nbc + min(cmid, ctot) : cend;
 
         // ---- 2. interchanges and U12 = L~11^{-1} A12, one warp per trailing column with lane k on
         // row p0 + k: u_i -= l_ik u_k for k ascending (the substitution's order of operations), the
@@ -268,42 +396,69 @@ __global__ void __launch_bounds__(512, 1)
             const int prow = lane < npart ? src[plist[lane]] : 0;
             const int dst = lane < npart ? plist[lane] : 0;
             const zf* lrow = Ps + lane;
-            for (int q0 = p0 + nbc + 4 * warp; q0 < cend; q0 += 4 * nwarp) {
-                zf u[4], x[4];
+            const int wsrc = rs(srow), wprow = rs(prow), wdst = rs(dst), wlane = rs(lane);
+            zf* cw = scr + (size_t)warp * CCOLS * CST;
+            // eight columns per warp in two groups of four; the next group's loads run ahead
+            auto load4 = [&](int q0, zf (&u)[4], zf (&x)[4]) __attribute__((always_inline)) {
 #pragma unroll
                 for (int m = 0; m < 4; ++m) {
                     const int q = q0 + m;
-                    u[m] = q < cend && lane < nbc ? W[wi(p0 + srow, q)] : mk(0.0f, 0.0f);
-                    x[m] = q < cend && lane < npart ? W[wi(p0 + prow, q)] : mk(0.0f, 0.0f);
+                    u[m] = q < chi && lane < nbc ? W[wsrc + RWp * cs_(q - p0)] : mk(0.0f, 0.0f);
+                    x[m] = q < chi && lane < npart ? W[wprow + RWp * cs_(q - p0)] : mk(0.0f, 0.0f);
                 }
-                __syncwarp();
+            };
+            zf u[4], x[4];
+            load4(clo + 8 * warp, u, x);
+            for (int qb = clo + 8 * warp; qb < chi; qb += 8 * nwarp) {
 #pragma unroll
-                for (int m = 0; m < 4; ++m)
-                    if (q0 + m < cend && lane < npart) W[wi(p0 + dst, q0 + m)] = x[m];
-                for (int k = 0; k + 1 < nbc; ++k) {
-                    const zf l = lrow[(int64_t)RW * k];
-                    const bool act = lane > k && lane < nbc;
+                for (int g4 = 0; g4 < 2; ++g4) {
+                    const int q0 = qb + 4 * g4;
+                    zf un[4], xn[4];
+                    load4(g4 == 0 ? q0 + 4 : qb + 8 * nwarp, un, xn);
+                    __syncwarp();  // every lane has read this group's rows
+#pragma unroll
+                    for (int m = 0; m < 4; ++m)
+                        if (q0 + m < chi && lane < npart) W[wdst + RWp * cs_(q0 + m - p0)] = x[m];
+                    for (int k = 0; k + 1 < nbc; ++k) {
+                        const zf l = lrow[RW * k];
+                        const bool act = lane > k && lane < nbc;
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            const zf uk = shfl_cx(u[m], k);
+                            if (act) u[m] = fms(u[m], l, uk);
+                        }
+                    }
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
-                        const zf uk = shfl_cx(u[m], k);
-                        if (act) u[m] = fms(u[m], l, uk);
+                        if (q0 + m < chi && lane < nbc) W[wlane + RWp * cs_(q0 + m - p0)] = u[m];
+                        if (fast) cw[(4 * g4 + m) * CST + lane] = u[m];
                     }
-                }
 #pragma unroll
-                for (int m = 0; m < 4; ++m)
-                    if (q0 + m < cend && lane < nbc) W[wi(p0 + lane, q0 + m)] = u[m];
+                    for (int m = 0; m < 4; ++m) u[m] = un[m], x[m] = xn[m];
+                }
+                if (fast) {  // the eight columns to the output rows: lanes over columns, then rows
+                    __syncwarp();
+                    const int m = lane & 7, q = qb + m;
+#pragma unroll
+                    for (int k0 = 0; k0 < NB; k0 += 4) {
+                        const int k = k0 + (lane >> 3), r = p0 + k;
+                        if (k < nbc && q < chi && q - r <= kv) ab[(int64_t)r * ldab + (q - r)] = cw[m * CST + k];
+                    }
+                    __syncwarp();
+                }
             }
         }
         __syncthreads();
         // U12 rows to the output band (warps over rows, lanes over columns)
-        for (int k = warp; k < nbc; k += nwarp) {
-            const int r = p0 + k;
-            for (int q = p0 + nbc + lane; q < cend; q += 32)
-                if (q - r <= kv) ab[(int64_t)r * ldab + (q - r)] = W[wi(r, q)];
-        }
+        if (!fast)
+            for (int k = warp; k < nbc; k += nwarp) {
+                const int r = p0 + k;
+                for (int q = clo + lane; q < chi; q += 32)
+                    if (q - r <= kv) ab[(int64_t)r * ldab + (q - r)] = W[wi(k, q - p0)];
+            }
 
         // ---- the panel part of the finished rows: U(r, r .. p0+nbc-1), zeros beyond the band
-        for (int k = warp; k < nbc; k += nwarp) {
+        for (int k = part == 0 ? warp : nbc; k < nbc; k += nwarp) {
             const int r = p0 + k;
             zf* out = ab + (int64_t)r * ldab;
             for (int q = k + lane; q < nbc; q += 32) out[q - k] = Ps[k + (int64_t)RW * q];
@@ -313,7 +468,7 @@ __global__ void __launch_bounds__(512, 1)
 
         // ---- 3. A operand image of L~21 (global, the tensor core's layout), tiles of 64 rows
         const int nmt = mr > 0 ? (mr + MT - 1) / MT : 0;
-        const int ntn = (cend > p0 + nbc && mr > 0) ? (cend - (p0 + nbc) + NT - 1) / NT : 0;
+        const int ntn = (chi > clo && mr > 0) ? (chi - clo + NT - 1) / NT : 0;
         if (ntn > 0) {
             for (int e = tid; e < nmt * PART; e += nthr) {
                 const int mt = e / PART, f = e - mt * PART;
@@ -338,20 +493,19 @@ __global__ void __launch_bounds__(512, 1)
 
         // ---- 4. A22 -= L~21 U12 on the tensor core
         for (int nt = 0; nt < ntn; ++nt) {
-            const int c0 = p0 + nbc + nt * NT;
-            const int ncol = min(NT, cend - c0);
+            const int c0 = clo + nt * NT;
+            const int ncol = min(NT, chi - c0);
             if (tid == 0 && !*abort_v)
                 for (int q = 0; q < min(2, nmt); ++q) {
                     const int b = (int)((g + q) & 1);
                     float* dst = b ? Abuf1 : Abuf0;
                     tc::mbar_arrive_expect_tx(&full_b[b], TILE_BYTES);
-                    tc::tma_load_3d(dst, &tmap, &full_b[b], 0, q * 256, j);
+                    tc::tma_load_3d(dst, &tmap, &full_b[b], 0, q * 256, img);
                     ++tma_issued[b];
                 }
             // the C rows of the first A tile towards L2 while B is built (lane q: column q of its group)
             if ((warp >> 2) * 32 + lane < ncol && 16 * (warp & 3) < mr)
-                tc::prefetch_l2(W + (int64_t)((p0 + nbc + 16 * (warp & 3)) % RWp) +
-                                (int64_t)RWp * ((c0 + (warp >> 2) * 32 + lane) % CWp));
+                tc::prefetch_l2(W + wi(nbc + 16 * (warp & 3), c0 - p0 + (warp >> 2) * 32 + lane));
             // B: row rn of the operand = complex column c0 + rn of U12, K = [Ur ; Ui]; lanes over the
             // 32 rows of U12 (contiguous in the window), eight independent loads, then the stores
             for (int e0 = 0; e0 < NB * NT; e0 += 8 * nthr) {
@@ -359,7 +513,7 @@ __global__ void __launch_bounds__(512, 1)
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
                     const int e = e0 + tid + s * nthr, kk = e & (NB - 1), rn = e >> 5;
-                    u[s] = rn < ncol && kk < nbc ? W[wi(p0 + kk, c0 + rn)] : mk(0.0f, 0.0f);
+                    u[s] = rn < ncol && kk < nbc ? W[wi(kk, c0 - p0 + rn)] : mk(0.0f, 0.0f);
                 }
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
@@ -408,7 +562,7 @@ __global__ void __launch_bounds__(512, 1)
                 if (t + 1 < nmt && cb + lane < ncol) {
                     const int i = (t + 1) * MT + 16 * (warp & 3);
                     if (i < mr)
-                        tc::prefetch_l2(W + (int64_t)((p0 + nbc + i) % RWp) + (int64_t)RWp * ((c0 + cb + lane) % CWp));
+                        tc::prefetch_l2(W + wi(nbc + i, c0 - p0 + cb + lane));
                 }
                 if (tid == 0) {
                     if (t == 0) issue(0);
@@ -420,7 +574,7 @@ __global__ void __launch_bounds__(512, 1)
                 if (tid == 0 && ok && t + 2 < nmt) {
                     float* dst = b ? Abuf1 : Abuf0;
                     tc::mbar_arrive_expect_tx(&full_b[b], TILE_BYTES);
-                    tc::tma_load_3d(dst, &tmap, &full_b[b], 0, (t + 2) * 256, j);
+                    tc::tma_load_3d(dst, &tmap, &full_b[b], 0, (t + 2) * 256, img);
                     ++tma_issued[b];
                 }
                 __syncwarp();
@@ -447,9 +601,9 @@ __global__ void __launch_bounds__(512, 1)
                     const int rr = (warp & 3) * 32 + lane;
                     const int i = t * MT + (rr >> 1);
                     if (i < mr) {
-                        zf* wrow = W + (int64_t)((p0 + nbc + i) % RWp);
+                        zf* wrow = W + rs(nbc + i);
                         const int h = odd ? 16 : 0;
-                        const int cs = (c0 + cb + h) % CWp;
+                        const int cs = cs_(c0 - p0 + cb + h);
                         zf cur[16];
 #pragma unroll
                         for (int q = 0; q < 16; ++q) {
@@ -470,36 +624,38 @@ __global__ void __launch_bounds__(512, 1)
         if (*abort_v) break;
 
         // ---- 5. next window: rows [p0+RW, p0+RW+NB) and columns [p0+RW.., ) enter
+        if (nsplit > 1) csync();  // the other CTA is done with the rows and columns that leave
         if (p0 + NB < n) {
             const int CW = kv + NB;
             const int rn0 = p0 + RW;
-            for (int e = tid; e < NB * RWp; e += nthr) {
-                const int jc = e / RWp, i = e - jc * RWp;
-                W[(int64_t)i + (int64_t)RWp * ((p0 + CW + jc) % CWp)] = mk(0.0f, 0.0f);
+            const int nws = nwarp * nsplit, wid = part * nwarp + warp;  // warps of all CTAs
+            for (int jc = wid; jc < NB; jc += nws) {
+                zf* wc = W + RWp * ((p0 + CW + jc) % CWp);
+                for (int i = lane; i < RWp; i += 32) wc[i] = mk(0.0f, 0.0f);
             }
-            __syncthreads();
+            csync();
             // column slot s holds the column c in [p0 + NB, p0 + NB + CWp) with c = s (mod CWp)
-            const int r = rn0 + lane;
-            const int per = (CWp + nwarp - 1) / nwarp;
-            const int cbase = p0 + NB;
-            for (int s0 = warp * per; s0 < min(CWp, (warp + 1) * per); s0 += 8) {
+            const int r = rn0 + lane, rslot = r % RWp;
+            const int per = (CWp + nws - 1) / nws;
+            const int cbase = p0 + NB, cb0 = cbase % CWp, send = min(CWp, (wid + 1) * per);
+            for (int s0 = wid * per; s0 < send; s0 += 8) {
                 zf v[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int s = s0 + u;
-                    const int c = cbase + posmod(s - cbase, CWp);
-                    v[u] = (s < min(CWp, (warp + 1) * per) && lane < NB && r < n && c >= r - kl && c <= r + ku && c < n)
+                    const int c = cbase + (s < cb0 ? s - cb0 + CWp : s - cb0);
+                    v[u] = (s < send && lane < NB && r < n && c >= r - kl && c <= r + ku && c < n)
                                ? ab[(int64_t)r * ldab + (c - r + kl)]
                                : mk(0.0f, 0.0f);
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     const int s = s0 + u;
-                    if (s < min(CWp, (warp + 1) * per)) W[(int64_t)(r % RWp) + (int64_t)RWp * s] = v[u];
+                    if (s < send) W[rslot + RWp * s] = v[u];
                 }
             }
         }
-        __syncthreads();
+        csync();
     }
     // wind down: copies and products in flight finish (bounded) before the memory is released
     if (tid == 0) {
@@ -522,7 +678,7 @@ __global__ void __launch_bounds__(512, 1)
         tc::tc_fence_after();
         tc::tmem_dealloc(tmem, TMEM_COLS);
     }
-    if (tid == 0) *info_out = *abort_v ? n + 1 : info_s;
+    if (tid == 0 && part == 0) *info_out = *abort_v ? n + 1 : info_s;
 }
 
 // ------------------------------------------------------------------ host side
@@ -547,6 +703,42 @@ bool lu_tc_enabled() {
     return on;
 }
 
+// CTAs per point: two where the device then still holds every CTA at once
+static int lu_tc_split(int npts) {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 152;
+    }();
+    return 2 * npts <= sms ? 2 : 1;
+}
+// the largest kl with the scratch
+static int lu_tc_scratch_max_kl() {
+    static const int v = [] {
+        int kl = 0;
+        while (lu_tc_scratch(kl + 1)) ++kl;
+        return kl;
+    }();
+    return v;
+}
+template <typename... Args>
+static cudaError_t lu_tc_start(int npts, int nsplit, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(npts * nsplit);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = nsplit;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, lu_tc_kernel, args...);
+}
+
 bool band_lu_tc_can(int kl) { return kl >= NB && lu_tc_smem(kl) <= 227 * 1024; }
 
 bool band_lu_tc_fits(int kl) { return kl > 64 && band_lu_tc_can(kl); }
@@ -563,19 +755,19 @@ int launch_band_lu_tc(const SplitDev& s, int npts, zf* ab, int* ipiv, int* info,
     const int kv = s.kl + s.ku;
     const int rwp = (s.kl + NB + NB - 1) / NB * NB, cwp = (kv + NB + NB - 1) / NB * NB;
     const size_t smem = lu_tc_smem(s.kl);
-    const int nmt_max = (s.kl + MT - 1) / MT;
+    const int nmt_max = (s.kl + MT - 1) / MT, nsplit = lu_tc_split(npts);
     zf* win = nullptr;
     float* aimg = nullptr;
     int* err = nullptr;
     NEP_CUDA(cudaMallocAsync((void**)&win, sizeof(zf) * (size_t)rwp * cwp * npts, st));
-    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * npts, st);
+    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * npts * nsplit, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&err, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
     CUtensorMap tmap;
     if (e == cudaSuccess) {
         // the operand images as a 3-D array of floats: 64 per image row (256 B), 256 image rows per
         // tile, nmt_max tiles per point, npts points; one box = one tile (64 KB)
-        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)npts};
+        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)npts * nsplit};
         const cuuint64_t strides[2] = {256, (cuuint64_t)nmt_max * TILE_BYTES};
         const cuuint32_t box[3] = {64, 256, 1};
         const cuuint32_t estr[3] = {1, 1, 1};
@@ -592,10 +784,9 @@ int launch_band_lu_tc(const SplitDev& s, int npts, zf* ab, int* ipiv, int* info,
     }
     if (e == cudaSuccess) e = allow_max_dynamic_smem(lu_tc_kernel);
     if (e == cudaSuccess) {
-        lu_tc_kernel<<<npts, 512, smem, st>>>(s.n, s.kl, s.ku, s.ldab, ab, ipiv, info, active, win, rwp, cwp, aimg,
-                                              nmt_max, tmap, err, nullptr, passes);
+        e = lu_tc_start(npts, nsplit, smem, st, s.n, s.kl, s.ku, s.ldab, ab, ipiv, info, active, win, rwp, cwp, aimg,
+                        nmt_max, tmap, err, (const PointDesc*)nullptr, passes, nsplit, lu_tc_scratch_max_kl());
         count_launch();
-        e = cudaGetLastError();
     }
     int herr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -624,6 +815,7 @@ int launch_band_lu_tc_batch(const std::vector<PointDesc>& items_in, cudaStream_t
     std::vector<PointDesc> items(items_in);
     size_t smem = 0, win_elems = 0;
     int nmt_max = 1;
+    const int nsplit = lu_tc_split(count);
     for (auto& d : items) {
         if (!band_lu_tc_can(d.kl)) return NEP_ERR_UNSUPPORTED;
         const int kv = d.kl + d.ku;
@@ -638,7 +830,7 @@ int launch_band_lu_tc_batch(const std::vector<PointDesc>& items_in, cudaStream_t
     int* err = nullptr;
     PointDesc* pd = nullptr;
     NEP_CUDA(cudaMallocAsync((void**)&win, sizeof(zf) * win_elems, st));
-    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * count, st);
+    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * count * nsplit, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&err, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&pd, sizeof(PointDesc) * count, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
@@ -650,7 +842,7 @@ int launch_band_lu_tc_batch(const std::vector<PointDesc>& items_in, cudaStream_t
     if (e == cudaSuccess) e = cudaMemcpyAsync(pd, items.data(), sizeof(PointDesc) * count, cudaMemcpyHostToDevice, st);
     CUtensorMap tmap;
     if (e == cudaSuccess) {
-        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)count};
+        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)count * nsplit};
         const cuuint64_t strides[2] = {256, (cuuint64_t)nmt_max * TILE_BYTES};
         const cuuint32_t box[3] = {64, 256, 1};
         const cuuint32_t estr[3] = {1, 1, 1};
@@ -661,10 +853,10 @@ int launch_band_lu_tc_batch(const std::vector<PointDesc>& items_in, cudaStream_t
     }
     if (e == cudaSuccess) e = allow_max_dynamic_smem(lu_tc_kernel);
     if (e == cudaSuccess) {
-        lu_tc_kernel<<<count, 512, smem, st>>>(0, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0, aimg,
-                                               nmt_max, tmap, err, pd, passes);
+        e = lu_tc_start(count, nsplit, smem, st, 0, 0, 0, 0, (zf*)nullptr, (int*)nullptr, (int*)nullptr, (const int*)nullptr,
+                        (zf*)nullptr, 0, 0, aimg, nmt_max, tmap, err, (const PointDesc*)pd, passes, nsplit,
+                        lu_tc_scratch_max_kl());
         count_launch();
-        e = cudaGetLastError();
     }
     int herr = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, st);
