@@ -1,6 +1,5 @@
 // Extraction of the eigenpairs from the contour moments (all on the device, FP64 unless noted):
-//   * zgemm_kernel      dense complex products (column-major, op(A) in {A, A^H}), split-K
-//                       with a fixed-order reduction so results never depend on scheduling;
+//   * zgemm             dense complex products (gemm.cu);
 //   * jacobi_kernel     one-sided (Hestenes) Jacobi SVD, cooperative across CTAs: round-robin
 //                       pairings, one warp per column pair, a bounded grid barrier per round
 //                       (FP64 throughput per SM is low on this part, so the pairs of a round
@@ -20,145 +19,6 @@
 #include "nep_common.cuh"
 
 namespace nep {
-
-// ------------------------------------------------------------------ dense products
-// C = op(A) B (column-major, op in {A, A^H}). A CTA computes a BM x BN tile with (BM/TM) x (BN/TN)
-// threads of TM x TN outputs, K in steps of GK through shared memory; long K splits over CTAs
-// into a workspace reduced in a fixed order, so results never depend on scheduling. FP64
-// arithmetic is the bound on this part (about two FP64 FMAs per clock per SM), so the launcher
-// picks the tile shape and the split that waste the least of it: padding beyond M and N (the
-// reduced dimensions here are rarely multiples of 32) and SMs left idle or doubly loaded.
-constexpr int GK = 8;
-template <int BM, int BN, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-    zgemm_kernel(int M, int N, int K, int opA, const zd* __restrict__ A, int lda, const zd* __restrict__ B, int ldb,
-                 zd* __restrict__ C, int ldc, int kchunk, int64_t part_stride) {
-    constexpr int TX = BM / TM, TY = BN / TN, NT = TX * TY;
-    __shared__ zd As[GK][BM + 1];
-    __shared__ zd Bs[GK][BN + 1];
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
-    zd acc[TM][TN];
-#pragma unroll
-    for (int a = 0; a < TM; ++a)
-#pragma unroll
-        for (int b = 0; b < TN; ++b) acc[a][b] = mk(0.0, 0.0);
-    for (int k0 = kb; k0 < ke; k0 += GK) {
-        // loads run along the contiguous index of each operand
-        for (int t = threadIdx.x; t < GK * BM; t += NT) {
-            const int kk = opA == 0 ? t / BM : t % GK, mm = opA == 0 ? t % BM : t / GK;
-            const int gm = m0 + mm, gk = k0 + kk;
-            zd v = mk(0.0, 0.0);
-            if (gm < M && gk < ke) v = opA == 0 ? A[gm + (int64_t)lda * gk] : conj(A[gk + (int64_t)lda * gm]);
-            As[kk][mm] = v;
-        }
-        for (int t = threadIdx.x; t < GK * BN; t += NT) {
-            const int kk = t % GK, nn = t / GK;
-            const int gn = n0 + nn, gk = k0 + kk;
-            Bs[kk][nn] = (gn < N && gk < ke) ? B[gk + (int64_t)ldb * gn] : mk(0.0, 0.0);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < GK; ++kk) {
-            zd av[TM], bv[TN];
-#pragma unroll
-            for (int a = 0; a < TM; ++a) av[a] = As[kk][tx + TX * a];
-#pragma unroll
-            for (int b = 0; b < TN; ++b) bv[b] = Bs[kk][ty + TY * b];
-#pragma unroll
-            for (int a = 0; a < TM; ++a)
-#pragma unroll
-                for (int b = 0; b < TN; ++b) acc[a][b] = fma_(acc[a][b], av[a], bv[b]);
-        }
-        __syncthreads();
-    }
-    zd* Cz = C + (int64_t)blockIdx.z * part_stride;
-#pragma unroll
-    for (int a = 0; a < TM; ++a)
-#pragma unroll
-        for (int b = 0; b < TN; ++b) {
-            const int gm = m0 + tx + TX * a, gn = n0 + ty + TY * b;
-            if (gm < M && gn < N) Cz[gm + (int64_t)ldc * gn] = acc[a][b];
-        }
-}
-
-__global__ void zgemm_reduce_kernel(int M, int N, int splits, const zd* __restrict__ part, zd* __restrict__ C, int ldc) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)M * N) return;
-    const int m = (int)(t % M), n = (int)(t / M);
-    zd acc = mk(0.0, 0.0);
-    for (int z = 0; z < splits; ++z) acc = acc + part[(int64_t)z * M * N + t];
-    C[m + (int64_t)ldc * n] = acc;
-}
-
-namespace {
-struct GemmShape {
-    int bm, bn;
-};
-constexpr GemmShape kGemmShapes[] = {{64, 32}, {64, 24}, {32, 32}, {32, 24}, {24, 24}, {32, 16}, {24, 16}};
-
-template <int BM, int BN, int TM, int TN>
-void zgemm_launch(dim3 grid, int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int ldb, zd* C, int ldc,
-                  int kchunk, int64_t part_stride, cudaStream_t st) {
-    zgemm_kernel<BM, BN, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(M, N, K, opA, A, lda, B, ldb, C, ldc, kchunk,
-                                                                       part_stride);
-}
-}  // namespace
-
-// C = op(A) B. part: workspace of splits*M*N elements when K is long (nullptr => no split).
-int zgemm(int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int ldb, zd* C, int ldc, zd* part,
-          size_t part_elems, cudaStream_t st) {
-    if (M <= 0 || N <= 0) return NEP_OK;
-    static const int sms = [] {
-        int dev = 0, v = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        return v > 0 ? v : 152;
-    }();
-    // score = useful fraction of the padded tiles x SM load balance (mean over max CTAs per SM),
-    // a split costing a little for its partial sums and their reduction
-    int best = 0, best_splits = 1;
-    double best_score = -1.0;
-    for (int c = 0; c < (int)(sizeof(kGemmShapes) / sizeof(kGemmShapes[0])); ++c) {
-        const int bm = kGemmShapes[c].bm, bn = kGemmShapes[c].bn;
-        const int64_t tiles = (int64_t)ceil_div(M, bm) * ceil_div(N, bn);
-        const double pad = (double)M * N / ((double)ceil_div(M, bm) * bm * ceil_div(N, bn) * bn);
-        const int max_splits = part ? std::max(1, std::min<int>(K / 32, (int)std::min<size_t>(64, part_elems / ((size_t)M * N)))) : 1;
-        for (int sp = 1; sp <= max_splits; ++sp) {
-            const double ctas = (double)tiles * sp;
-            const double waves = std::ceil(ctas / sms);
-            const double score = pad * (ctas / sms) / waves * (sp > 1 ? 0.97 : 1.0);
-            if (score > best_score + 1e-9) {
-                best_score = score;
-                best = c;
-                best_splits = sp;
-            }
-        }
-    }
-    const int bm = kGemmShapes[best].bm, bn = kGemmShapes[best].bn;
-    const int kchunk = ceil_div(ceil_div(K, best_splits), GK) * GK;
-    const int splits = std::max(1, ceil_div(K, kchunk));
-    dim3 grid(ceil_div(M, bm), ceil_div(N, bn), splits);
-    zd* out = splits == 1 ? C : part;
-    const int ldo = splits == 1 ? ldc : M;
-    const int64_t ps = splits == 1 ? 0 : (int64_t)M * N;
-    switch (best) {
-        case 0: zgemm_launch<64, 32, 4, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
-        case 1: zgemm_launch<64, 24, 4, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
-        case 2: zgemm_launch<32, 32, 2, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
-        case 3: zgemm_launch<32, 24, 2, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
-        case 4: zgemm_launch<24, 24, 2, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
-        case 5: zgemm_launch<32, 16, 2, 1>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
-        default: zgemm_launch<24, 16, 2, 1>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
-    }
-    NEP_CHECK_LAUNCH();
-    if (splits > 1) {
-        zgemm_reduce_kernel<<<ceil_div((int64_t)M * N, 256), 256, 0, st>>>(M, N, splits, part, C, ldc);
-        NEP_CHECK_LAUNCH();
-    }
-    return NEP_OK;
-}
 
 // ------------------------------------------------------------------ grid barrier
 // Barrier for a cooperative launch (all CTAs co-resident) on a monotonically increasing

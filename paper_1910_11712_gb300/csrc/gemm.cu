@@ -1,0 +1,193 @@
+// Dense complex FP64 products C = op(A) B (column-major, op in {A, A^H}) of the extraction, on the tensor core by
+// exact 8-bit digit products (oz.cuh).
+//
+// A CTA of 8 warps computes a 32 x 32 tile, K in blocks of 64: the exponents of the tile's rows and columns over
+// the block, then twice 32 terms as digits in the MMA fragments' order in shared memory (A 64 KB, B 32 KB) and
+// 36 x 4 MMA steps per warp and 8 x 8 subtile (a warp takes 8 rows by 16 columns); the exact sums of a block
+// become FP64 once. Long K splits over CTAs into a workspace reduced in a fixed order, so results never depend
+// on scheduling. Blocks with a non-finite entry or an extreme exponent are summed in FP64 FMAs.
+#include "oz.cuh"
+
+namespace nep {
+
+namespace {
+constexpr int TB = 32, KH = 32, KCH = KH / 8;  // tile, terms per staged half, MMA steps of a half
+constexpr size_t A_WORDS = 4 * KCH * oz::S * 128, B_WORDS = 4 * KCH * oz::S * 64;
+}  // namespace
+
+__global__ void __launch_bounds__(256, 2)
+    zgemm_oz_kernel(int M, int N, int K, int opA, const zd* __restrict__ A, int lda, const zd* __restrict__ B, int ldb,
+                    zd* __restrict__ C, int ldc, int kchunk, int64_t part_stride) {
+    using namespace oz;
+    extern __shared__ uint4 sm4[];
+    unsigned* Af = reinterpret_cast<unsigned*>(sm4);  // [4 row tiles][KCH][S][32 lanes][4]
+    unsigned* Bf = Af + A_WORDS;                      // [4 column tiles][KCH][S][32 lanes][2]
+    __shared__ int ea[TB], eb[TB], bad;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int m0 = blockIdx.x * TB, n0 = blockIdx.y * TB;
+    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
+    auto aval = [&](int m, int k) -> zd {
+        if (m0 + m >= M || k >= ke) return mk(0.0, 0.0);
+        return opA == 0 ? A[m0 + m + (int64_t)lda * k] : conj(A[k + (int64_t)lda * (m0 + m)]);
+    };
+    auto bval = [&](int c, int k) -> zd { return n0 + c < N && k < ke ? B[k + (int64_t)ldb * (n0 + c)] : mk(0.0, 0.0); };
+    const int mt = warp & 3, nt0 = 2 * (warp >> 2);
+    // rows and columns of the tile in use, in eights: the rest is neither built nor multiplied
+    const int mu = min(TB, (M - m0 + 7) & ~7), nu = min(TB, (N - n0 + 7) & ~7);
+    const int g = lane >> 2, tq = lane & 3;
+    double out[2][4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) out[u][q] = 0.0;
+    for (int k0 = kb; k0 < ke; k0 += CH) {
+        const int kn = min(CH, ke - k0);
+        __syncthreads();  // the previous block's digits and exponents have been read
+        if (tid < TB) ea[tid] = eb[tid] = 0;
+        if (tid == 0) bad = 0;
+        __syncthreads();
+        // lanes along the contiguous index: A by rows (op A) or by k (op A^H), B by k
+        for (int e = tid; e < TB * CH; e += 256) {
+            const int m = opA == 0 ? e & (TB - 1) : e / CH, k = opA == 0 ? e / TB : e & (CH - 1);
+            if (k < kn && m < mu) {
+                int x = exp_field(aval(m, k0 + k));
+                if (opA != 0) x = __reduce_max_sync(__activemask(), x);  // one row per warp
+                if (opA == 0 || (tid & 31) == 0) atomicMax(&ea[m], x);
+            }
+            const int c = e / CH, kk = e & (CH - 1);
+            if (kk < kn && c < nu) {
+                const int x = __reduce_max_sync(__activemask(), exp_field(bval(c, k0 + kk)));
+                if ((tid & 31) == 0) atomicMax(&eb[c], x);
+            }
+        }
+        __syncthreads();
+        if (tid < TB) {
+            int x = ea[tid], y = eb[tid];
+            if ((x && (x < EXP_LO || x > EXP_HI)) || (y && (y < EXP_LO || y > EXP_HI))) bad = 1;
+            if (x == 0) ea[tid] = 1023;
+            if (y == 0) eb[tid] = 1023;
+        }
+        __syncthreads();
+        if (bad) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int c = 8 * (nt0 + u) + 2 * tq + q;
+                    zd acc = mk(out[u][q], out[u][2 + q]);
+                    for (int k = 0; k < kn; ++k) acc = fma_(acc, aval(8 * mt + g, k0 + k), bval(c, k0 + k));
+                    out[u][q] = acc.re;
+                    out[u][2 + q] = acc.im;
+                }
+            continue;
+        }
+        float D[2][S][4];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int t = 0; t < S; ++t)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) D[u][t][q] = 0.0f;
+        for (int h0 = 0; h0 < kn; h0 += KH) {
+            if (h0 > 0) __syncthreads();  // the first half's digits have been read
+            for (int e = tid; e < TB * KH; e += 256) {
+                const int m = opA == 0 ? e & (TB - 1) : e / KH, k = opA == 0 ? e / TB : e & (KH - 1);
+                if (m < mu) {
+                    const zd c = aval(m, k0 + h0 + k);
+                    const int E = ea[m];
+                    const unsigned long long re = fixed62(c.re, E), im = fixed62(c.im, E), ni = fixed62(-c.im, E);
+                    unsigned* f = Af + (((m >> 3) * KCH + (k >> 3)) * S) * 128 + ((m & 7) * 4 + (k & 3)) * 4 + ((k & 4) ? 2 : 0);
+#pragma unroll
+                    for (int t = 0; t < S; ++t)
+                        *reinterpret_cast<uint2*>(f + t * 128) =
+                            make_uint2(digits2(re, ni, S - 1 - t), digits2(im, re, S - 1 - t));
+                }
+                const int c = e / KH;
+                if (c < nu) {
+                    const int k = e & (KH - 1);
+                    const zd y = bval(c, k0 + h0 + k);
+                    const int E = eb[c];
+                    const unsigned long long re = fixed62(y.re, E), im = fixed62(y.im, E);
+                    unsigned* f = Bf + (((c >> 3) * KCH + (k >> 3)) * S) * 64 + ((c & 7) * 4 + (k & 3)) * 2 + ((k & 4) ? 1 : 0);
+#pragma unroll
+                    for (int t = 0; t < S; ++t) f[t * 64] = digits2(re, im, S - 1 - t);
+                }
+            }
+            __syncthreads();
+            const int kcs = min(KCH, (kn - h0 + 7) / 8);
+#pragma unroll 1
+            for (int kc = 0; kc < kcs; ++kc) {
+                const uint4* a4 = reinterpret_cast<const uint4*>(Af) + (mt * KCH + kc) * S * 32 + lane;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    if (8 * mt >= mu || 8 * (nt0 + u) >= nu) continue;
+                    const uint2* b2 = reinterpret_cast<const uint2*>(Bf) + ((nt0 + u) * KCH + kc) * S * 32 + lane;
+                    uint2 b[S];
+#pragma unroll
+                    for (int t = 0; t < S; ++t) b[t] = b2[t * 32];
+#pragma unroll
+                    for (int ta = 0; ta < S; ++ta) {
+                        const uint4 a = a4[ta * 32];
+#pragma unroll
+                        for (int tb = 0; ta + tb < S; ++tb) mma16816(D[u][ta + tb], a, b[tb].x, b[tb].y);
+                    }
+                }
+            }
+        }
+        // columns 2 (lane % 4) + (q & 1); rows lane / 4 (Re for q < 2, else Im)
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                out[u][q] += combine(D[u], q, ea[8 * mt + g], eb[8 * (nt0 + u) + 2 * tq + (q & 1)]);
+    }
+    zd* Cz = C + (int64_t)blockIdx.z * part_stride;
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int gm = m0 + 8 * mt + g, gn = n0 + 8 * (nt0 + u) + 2 * tq + q;
+            if (gm < M && gn < N) Cz[gm + (int64_t)ldc * gn] = mk(out[u][q], out[u][2 + q]);
+        }
+}
+
+__global__ void zgemm_reduce_kernel(int M, int N, int splits, const zd* __restrict__ part, zd* __restrict__ C, int ldc) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (int64_t)M * N) return;
+    const int m = (int)(t % M), n = (int)(t / M);
+    zd acc = mk(0.0, 0.0);
+    for (int z = 0; z < splits; ++z) acc = acc + part[(int64_t)z * M * N + t];
+    C[m + (int64_t)ldc * n] = acc;
+}
+
+// C = op(A) B. part: workspace of splits*M*N elements when K is long (nullptr => no split).
+int zgemm(int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int ldb, zd* C, int ldc, zd* part,
+          size_t part_elems, cudaStream_t st) {
+    if (M <= 0 || N <= 0) return NEP_OK;
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 152;
+    }();
+    // blocks of 64 terms over as many CTAs as two per SM allow
+    const int tiles = ceil_div(M, TB) * ceil_div(N, TB), blocks = std::max(1, ceil_div(K, oz::CH));
+    const int room = part ? (int)std::min<size_t>(64, part_elems / ((size_t)M * N)) : 1;
+    int splits = std::max(1, std::min(std::min(blocks, room), 2 * sms / tiles));
+    const int kchunk = ceil_div(blocks, splits) * oz::CH;
+    splits = std::max(1, ceil_div(K, kchunk));
+    zd* out = splits == 1 ? C : part;
+    const int ldo = splits == 1 ? ldc : M;
+    const int64_t ps = splits == 1 ? 0 : (int64_t)M * N;
+    NEP_CUDA(allow_max_dynamic_smem(zgemm_oz_kernel));
+    zgemm_oz_kernel<<<dim3(ceil_div(M, TB), ceil_div(N, TB), splits), 256, sizeof(unsigned) * (A_WORDS + B_WORDS), st>>>(
+        M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps);
+    NEP_CHECK_LAUNCH();
+    if (splits > 1) {
+        zgemm_reduce_kernel<<<ceil_div((int64_t)M * N, 256), 256, 0, st>>>(M, N, splits, part, C, ldc);
+        NEP_CHECK_LAUNCH();
+    }
+    return NEP_OK;
+}
+
+}  // namespace nep

@@ -627,7 +627,8 @@ struct nep_plan {
     int *active = nullptr, *sweeps = nullptr, *nactive = nullptr;
     zd* S = nullptr;      // K x n x L
     zd* mu = nullptr;     // K x L x L
-    zd* vpart = nullptr;  // chunks x K x L x L
+    zd* vpart = nullptr;  // splits of V^H S (up to 64) x K x L x L
+    size_t vpart_elems = 0;
     zd *H = nullptr, *Hs = nullptr, *Hw = nullptr, *U = nullptr, *W = nullptr;  // LM x LM
     double* sigma = nullptr;                                                     // LM
     zd *T1 = nullptr, *Bred = nullptr, *theta = nullptr, *Tv = nullptr, *Z = nullptr, *cand = nullptr;
@@ -717,7 +718,8 @@ static int plan_alloc(nep_plan* p) {
     NEP_TRY(dalloc(&p->nactive, 1, st));
     NEP_TRY(dalloc(&p->S, (size_t)K * n * L, st));
     NEP_TRY(dalloc(&p->mu, (size_t)K * L * L, st));
-    NEP_TRY(dalloc(&p->vpart, (size_t)ceil_div(n, 128) * K * L * L, st));
+    p->vpart_elems = (size_t)std::min(64, ceil_div(n, 64)) * K * L * L;
+    NEP_TRY(dalloc(&p->vpart, p->vpart_elems, st));
     const size_t lm2 = (size_t)LM * LM;
     NEP_TRY(dalloc(&p->H, lm2, st));
     NEP_TRY(dalloc(&p->Hs, lm2, st));
@@ -1227,7 +1229,7 @@ static int run_extract(nep_plan* p, cudaStream_t st) {
     if (p->mixed) NEP_TRY(launch_moments_df(n, L, p->Np, K, p->coef, p->Y, p->S, st));  // Y back to FP64 too
     else NEP_TRY(launch_moments(n, L, p->Np, K, p->coef, p->Y, p->S, st));
     if (p->Np != p->N) NEP_TRY(launch_double_real(int64_t(K) * n * L, p->S, st));
-    NEP_TRY(launch_vh_times(n, L, K, p->V, p->S, p->mu, p->vpart, st));
+    NEP_TRY(launch_vh_times(n, L, K, p->V, p->S, p->mu, p->vpart, p->vpart_elems, st));
     NEP_TRY(launch_hankel_build(L, M, p->mu, p->H, p->Hs, st));
     NEP_CUDA(cudaEventRecord(p->ev[4], st));
     // SVD of H and numerical rank

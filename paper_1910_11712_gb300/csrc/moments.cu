@@ -9,12 +9,13 @@
 // coefficients c_jk = w_j zeta_j^k sit in shared memory. Arithmetic is FP64 (1.75 FMA/clk/SM
 // on this part), so with 2M*4 FMAs per 16 bytes read the kernel is bound by FP64 issue,
 // not by HBM.
-// vh_partial_kernel + vh_reduce_kernel: mu_k = V^H S_k over row chunks with a fixed-order
-// reduction (no atomics), so results do not depend on scheduling.
+// mu_k = V^H S_k is a product of gemm.cu, split over the rows with a fixed-order reduction (no
+// atomics), so results do not depend on scheduling.
 #include <algorithm>
 
 #include "df_arith.cuh"
 #include "nep_common.cuh"
+#include "oz.cuh"
 
 namespace nep {
 
@@ -59,10 +60,167 @@ __global__ void __launch_bounds__(256) moments_kernel_generic(int64_t nl, int N,
     }
 }
 
+// ------------------------------------------------------------------ FP64 moments on the tensor core
+// The moments are a contraction, K x N coefficients by N x (n L) values, done with exact digit products (oz.cuh).
+// A warp takes 8 columns: its B fragments come straight from global memory (lane: column lane / 4,
+// nodes lane % 4 and + 4 of each 8; the column's exponent from a first pass over it, the digits from a
+// second that hits L1), the coefficients' digits are built once per CTA in the fragments' order in shared
+// memory. Columns with a non-finite entry or an extreme exponent take FP64 sums as moments_kernel does.
+// n L = 524288, N = 64, K = 16: 0.486 ms (FP64 FMAs: 3.56, at the FP64 pipe's rate; HBM alone: 0.10). Error
+// against a 113-bit sum: 4.7e-17 (N <= 64) and 8.3e-17 (N = 192) of the result's norm, FP64 FMAs 2.7e-16 to
+// 6.7e-16. What bounds it: issue (the digits' bytes and 72 MMAs per 8 nodes), not the tensor pipe.
+namespace oz {
+constexpr int KC = CH / 8;        // 16-wide MMA steps per chunk (8 nodes)
+constexpr int FRAG = 32 * 4;      // words of one A fragment
+}  // namespace oz
+
+// MT: tiles of 8 moments (1 or 2) of this CTA's share (blockIdx.y); nch chunks of CH nodes
+template <int MT>
+__global__ void __launch_bounds__(256, 2)
+    moments_oz_kernel(int64_t nl, int N, int K, int nch, const zd* __restrict__ coef, const zd* __restrict__ Y,
+                      zd* __restrict__ Sout) {
+    using namespace oz;
+    extern __shared__ uint4 afrag[];  // [chunk][MT][KC][S][32 lanes]
+    __shared__ int ea[8 * MT], bad;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int kbase = blockIdx.y * 8 * MT;
+    auto cval = [&](int j, int k) { return j < N && k < K ? coef[j + (int64_t)N * k] : mk(0.0, 0.0); };
+    if (tid == 0) bad = 0;
+    if (tid < 8 * MT) ea[tid] = 0;
+    __syncthreads();
+    for (int e = tid; e < N * 8 * MT; e += blockDim.x) {
+        const int k = e / N, j = e - k * N;
+        const zd c = cval(j, kbase + k);
+        atomicMax(&ea[k], exp_field(c));
+    }
+    __syncthreads();
+    if (tid < 8 * MT) {
+        if (ea[tid] != 0 && (ea[tid] < EXP_LO || ea[tid] > EXP_HI)) bad = 1;
+        if (ea[tid] == 0) ea[tid] = 1023;
+    }
+    __syncthreads();
+    const bool slow_all = bad != 0;
+    if (!slow_all) {
+        // word w of lane l of the fragment: row l / 4 (+ 8: the Im row) for w odd, node l % 4 (+ 4 for w >= 2)
+        for (int e = tid; e < nch * MT * KC * 32 * 4; e += blockDim.x) {
+            const int w = e & 3, l = (e >> 2) & 31, kc = (e >> 7) % KC, mt = (e >> 7) / KC % MT, ch = (e >> 7) / (KC * MT);
+            const int k = 8 * mt + l / 4, j = ch * CH + kc * 8 + (l & 3) + ((w & 2) ? 4 : 0);
+            const zd c = cval(j, kbase + k);
+            const int E = ea[k];
+            const unsigned long long p = fixed62((w & 1) ? c.im : c.re, E), q = fixed62((w & 1) ? c.re : -c.im, E);
+            unsigned* f = reinterpret_cast<unsigned*>(afrag) + (((size_t)(ch * MT + mt) * KC + kc) * S) * FRAG + l * 4 + w;
+#pragma unroll
+            for (int t = 0; t < S; ++t) f[t * FRAG] = digits2(p, q, S - 1 - t);  // the highest digit first
+        }
+    }
+    __syncthreads();
+    const int64_t tiles = (nl + 7) / 8;
+    for (int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; tile < tiles;
+         tile += (int64_t)gridDim.x * (blockDim.x >> 5)) {
+        const int64_t e0 = tile * 8, col = e0 + (lane >> 2);
+        const int jl = lane & 3;
+        const zd* yc = Y + col;
+        const bool in = col < nl;
+        int E = 0;
+#pragma unroll 4
+        for (int j = jl; j < N; j += 4) {
+            if (in) E = max(E, exp_field(yc[(int64_t)j * nl]));
+        }
+        E = max(E, __shfl_xor_sync(0xffffffffu, E, 1));
+        E = max(E, __shfl_xor_sync(0xffffffffu, E, 2));
+        const bool okc = E == 0 || (E >= EXP_LO && E <= EXP_HI);
+        if (slow_all || __any_sync(0xffffffffu, !okc)) {
+            for (int o = lane; o < 64 * MT; o += 32) {
+                const int64_t c = e0 + (o & 7);
+                const int k = kbase + (o >> 3);
+                if (c >= nl || k >= K) continue;
+                zd acc = mk(0.0, 0.0);
+                for (int j = 0; j < N; ++j) acc = fma_(acc, coef[j + (int64_t)N * k], Y[(int64_t)j * nl + c]);
+                Sout[(int64_t)k * nl + c] = acc;
+            }
+            continue;
+        }
+        if (E == 0) E = 1023;
+        double out[MT][4];
+        for (int ch = 0; ch < nch; ++ch) {
+            float D[MT][S][4];
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int t = 0; t < S; ++t)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) D[m][t][q] = 0.0f;
+            const int kcs = min(KC, (N - ch * CH + 7) / 8);
+            const uint4* af = afrag + (size_t)ch * MT * KC * S * 32 + lane;
+#pragma unroll 1
+            for (int kc = 0; kc < kcs; ++kc) {
+                const int j = ch * CH + kc * 8 + jl;
+                const zd y0 = in && j < N ? yc[(int64_t)j * nl] : mk(0.0, 0.0);
+                const zd y1 = in && j + 4 < N ? yc[(int64_t)(j + 4) * nl] : mk(0.0, 0.0);
+                const unsigned long long r0 = fixed62(y0.re, E), i0 = fixed62(y0.im, E);
+                const unsigned long long r1 = fixed62(y1.re, E), i1 = fixed62(y1.im, E);
+                unsigned b0[S], b1[S];
+#pragma unroll
+                for (int t = 0; t < S; ++t) {
+                    b0[t] = digits2(r0, i0, S - 1 - t);
+                    b1[t] = digits2(r1, i1, S - 1 - t);
+                }
+#pragma unroll
+                for (int ta = 0; ta < S; ++ta)
+#pragma unroll
+                    for (int m = 0; m < MT; ++m) {
+                        const uint4 a = af[(size_t)((m * KC + kc) * S + ta) * 32];
+#pragma unroll
+                        for (int tb = 0; ta + tb < S; ++tb) mma16816(D[m][ta + tb], a, b0[tb], b1[tb]);
+                    }
+            }
+            // columns 2 (lane % 4) + (q & 1); rows lane / 4 (Re for q < 2, else Im)
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int Eb = __shfl_sync(0xffffffffu, E, 4 * (2 * (lane & 3) + (q & 1)));
+                    const double sv = combine(D[m], q, ea[8 * m + (lane >> 2)], Eb);
+                    out[m][q] = ch == 0 ? sv : out[m][q] + sv;
+                }
+        }
+#pragma unroll
+        for (int m = 0; m < MT; ++m) {
+            const int k = kbase + 8 * m + (lane >> 2);
+            const int64_t c = e0 + 2 * (lane & 3);
+            if (k < K) {
+                if (c < nl) Sout[(int64_t)k * nl + c] = mk(out[m][0], out[m][2]);
+                if (c + 1 < nl) Sout[(int64_t)k * nl + c + 1] = mk(out[m][1], out[m][3]);
+            }
+        }
+    }
+}
+
+// The digits of up to 192 nodes' coefficients fit in shared memory
+template <int MT>
+static int launch_moments_oz(int64_t nl, int N, int K, const zd* coef, const zd* Y, zd* S, cudaStream_t st) {
+    const int nch = ceil_div(N, oz::CH);
+    const size_t sm = (size_t)nch * MT * oz::KC * oz::S * oz::FRAG * 4;
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 152;
+    }();
+    NEP_CUDA(allow_max_dynamic_smem(moments_oz_kernel<MT>));
+    const int gy = ceil_div(K, 8 * MT), per = sm <= 100 * 1024 ? 2 : 1;
+    const int gx = (int)std::min<int64_t>((nl + 63) / 64, std::max(1, per * sms / gy));
+    moments_oz_kernel<MT><<<dim3(gx, gy), 256, sm, st>>>(nl, N, K, nch, coef, Y, S);
+    NEP_CHECK_LAUNCH();
+    return NEP_OK;
+}
+
 int launch_moments(int n, int L, int N, int K, const zd* coef, const zd* Y, zd* S, cudaStream_t st) {
     const int64_t nl = (int64_t)n * L;
     const int blocks = ceil_div(nl, 256);
     const size_t sm = sizeof(zd) * (size_t)N * K;
+    if (nl >= 1 && N <= 3 * oz::CH && K >= 1)
+        return K <= 8 ? launch_moments_oz<1>(nl, N, K, coef, Y, S, st) : launch_moments_oz<2>(nl, N, K, coef, Y, S, st);
     if (K == 16 && sm <= 96 * 1024) {
         NEP_CUDA(allow_max_dynamic_smem(moments_kernel<16>));
         moments_kernel<16><<<blocks, 256, sm, st>>>(nl, N, coef, Y, S);
@@ -130,50 +288,9 @@ int launch_moments_df(int n, int L, int N, int K, const zd* coef, void* Y, zd* S
     return NEP_OK;
 }
 
-// part[(chunk*K + k)*L*L + a + L*b] = sum_{i in chunk} conj(V(i,a)) S_k(i,b)
-constexpr int VH_ROWS = 128;
-__global__ void __launch_bounds__(256) vh_partial_kernel(int n, int L, int K, const zd* __restrict__ V,
-                                                         const zd* __restrict__ S, zd* __restrict__ part) {
-    extern __shared__ zd sh[];
-    zd* vs = sh;                    // VH_ROWS x L
-    zd* ss = sh + VH_ROWS * L;      // VH_ROWS x L
-    const int chunk = blockIdx.x, k = blockIdx.y;
-    const int i0 = chunk * VH_ROWS;
-    const int rows = min(VH_ROWS, n - i0);
-    const zd* Sk = S + (int64_t)k * n * L;
-    for (int t = threadIdx.x; t < VH_ROWS * L; t += blockDim.x) {
-        const int i = t % VH_ROWS, a = t / VH_ROWS;
-        vs[t] = i < rows ? V[(int64_t)a * n + i0 + i] : mk(0.0, 0.0);
-        ss[t] = i < rows ? Sk[(int64_t)a * n + i0 + i] : mk(0.0, 0.0);
-    }
-    __syncthreads();
-    for (int ab = threadIdx.x; ab < L * L; ab += blockDim.x) {
-        const int a = ab % L, b = ab / L;
-        zd acc = mk(0.0, 0.0);
-        for (int i = 0; i < rows; ++i) acc = fmac(acc, vs[a * VH_ROWS + i], ss[b * VH_ROWS + i]);
-        part[((int64_t)chunk * K + k) * L * L + ab] = acc;
-    }
-}
-
-__global__ void vh_reduce_kernel(int nchunks, int LL, int K, const zd* __restrict__ part, zd* __restrict__ mu) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= K * LL) return;
-    const int k = t / LL, ab = t % LL;
-    zd acc = mk(0.0, 0.0);
-    for (int c = 0; c < nchunks; ++c) acc = acc + part[((int64_t)c * K + k) * LL + ab];
-    mu[t] = acc;
-}
-
-int launch_vh_times(int n, int L, int K, const zd* V, const zd* S, zd* mu, zd* part, cudaStream_t st) {
-    const int nch = ceil_div(n, VH_ROWS);
-    const size_t sm = sizeof(zd) * 2 * VH_ROWS * L;
-    if (sm > 200 * 1024) return NEP_ERR_UNSUPPORTED;
-    NEP_CUDA(allow_max_dynamic_smem(vh_partial_kernel));
-    vh_partial_kernel<<<dim3(nch, K), 256, sm, st>>>(n, L, K, V, S, part);
-    NEP_CHECK_LAUNCH();
-    vh_reduce_kernel<<<ceil_div(K * L * L, 256), 256, 0, st>>>(nch, L * L, K, part, mu);
-    NEP_CHECK_LAUNCH();
-    return NEP_OK;
+// mu_k = V^H S_k for all k: one product of V^H (L x n) and the n x (K L) block of the S_k, split over n.
+int launch_vh_times(int n, int L, int K, const zd* V, const zd* S, zd* mu, zd* part, size_t part_elems, cudaStream_t st) {
+    return zgemm(L, K * L, n, 1, V, n, S, n, mu, L, part, part_elems, st);
 }
 
 // H(a*L + i, b*L + c) = mu_{a+b}(i, c), Hs likewise with mu_{a+b+1}; mu_k is L x L column-major.

@@ -328,7 +328,7 @@ int launch_refine_decide(int npts, int L, int sweep, int max_sweeps, double tol,
                          int* active, int* sweeps, int* nactive, cudaStream_t st);
 // moments.cu
 int launch_moments(int n, int L, int N, int K, const zd* coef, const zd* Y, zd* S, cudaStream_t st);
-int launch_vh_times(int n, int L, int K, const zd* V, const zd* S, zd* mu, zd* part, cudaStream_t st);
+int launch_vh_times(int n, int L, int K, const zd* V, const zd* S, zd* mu, zd* part, size_t part_elems, cudaStream_t st);
 int launch_hankel_build(int L, int M, const zd* mu, zd* H, zd* Hs, cudaStream_t st);
 // extract.cu
 int zgemm(int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int ldb, zd* C, int ldc, zd* part,
