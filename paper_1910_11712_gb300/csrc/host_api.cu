@@ -611,7 +611,8 @@ struct nep_plan {
     zd* F = nullptr;      // nterms x N
     zd* coef = nullptr;   // N x K (column k: w_j zeta_j^k)
     void* ab = nullptr;   // N x n x ldab of complex64/complex128
-    void* ut = nullptr;   // N x n x (kl+ku+1): U by columns for the narrow-band sweeps (else unused)
+    void* ut = nullptr;     // N x n x (kl+ku+1): U by columns, for the sweeps or once nep_plan_buffer was asked for it
+    bool ut_asked = false;  // then every execution fills it
     int* ipiv = nullptr;  // N x n
     int* info = nullptr;  // N
     double* tnorm = nullptr;
@@ -694,7 +695,9 @@ static int plan_alloc(nep_plan* p) {
     NEP_TRY(dalloc(&p->F, (size_t)nt * N, st));
     NEP_TRY(dalloc(&p->coef, (size_t)N * K, st));
     NEP_TRY(dalloc_raw(&p->ab, esz * (size_t)N * n * h->ldab, st));
-    if (band_sweeps_fit(h->kl, h->ku)) NEP_TRY(dalloc_raw(&p->ut, esz * (size_t)N * n * (h->kl + h->ku + 1), st));
+    const bool needs_ut =
+        p->mixed ? band_solve_needs_ut<float>(h->kl, h->ku, N, L) : band_solve_needs_ut<double>(h->kl, h->ku, N, L);
+    if (needs_ut) NEP_TRY(dalloc_raw(&p->ut, esz * (size_t)N * n * (h->kl + h->ku + 1), st));
     NEP_TRY(dalloc(&p->ipiv, (size_t)N * n, st));
     NEP_TRY(dalloc(&p->info, N, st));
     NEP_TRY(dalloc(&p->tnorm, N, st));
@@ -972,7 +975,7 @@ static int run_solves(nep_plan* p, cudaStream_t st) {
     NEP_CUDA(cudaEventRecord(p->ev[1], st));
     NEP_TRY(launch_band_lu<T>(s, N, ab, p->ipiv, p->info, nullptr, st, p->lu_kernel));
     cx<T>* ut = reinterpret_cast<cx<T>*>(p->ut);
-    if (ut) NEP_TRY(band_transpose_u<T>(s, N, ab, ut, st));
+    if (ut && (p->ut_asked || band_solve_needs_ut<T>(s.kl, s.ku, N, L))) NEP_TRY(band_transpose_u<T>(s, N, ab, ut, st));
     NEP_CUDA(cudaEventRecord(p->ev[2], st));
     constexpr bool df = sizeof(T) == 4;  // complex64 factors: double-float refinement
     zdf* Ydf = reinterpret_cast<zdf*>(p->Y);
@@ -1128,16 +1131,28 @@ static int run_solves_batch(const std::vector<nep_plan*>& ps, cudaStream_t st) {
     if (!tc[1].empty()) NEP_TRY(launch_band_lu_tc_batch(tc[1], st, 1));
     for (nep_plan* p : ps) {
         const SplitDev s = p->h->dev();
-        if (p->ut) NEP_TRY(band_transpose_u<T>(s, p->Np, reinterpret_cast<cx<T>*>(p->ab), reinterpret_cast<cx<T>*>(p->ut), st));
+        if (p->ut && (p->ut_asked || band_solve_needs_ut<T>(s.kl, s.ku, p->Np, p->L)))
+            NEP_TRY(band_transpose_u<T>(s, p->Np, reinterpret_cast<cx<T>*>(p->ab), reinterpret_cast<cx<T>*>(p->ut), st));
         NEP_CUDA(cudaEventRecord(p->ev[2], st));
     }
-    // one solve of every live plan's points: register-window sweeps in shared launches per shape key
+    // one solve of every live plan's points in shared launches: the blocked substitution per right-hand
+    // sides a CTA and whether two CTAs share an SM, the register-window sweeps per shape key
     auto solve_all = [&](const std::vector<nep_plan*>& live, bool masked) -> int {
         std::map<std::tuple<int, int, int>, std::vector<PointDesc>> groups;
         std::map<std::tuple<int, int, int>, int> maxL;
+        std::map<std::pair<int, bool>, std::vector<PointDesc>> sgroups;
+        std::map<std::pair<int, bool>, int> smaxL;
+        std::map<std::pair<int, bool>, size_t> ssmem;
         for (nep_plan* p : live) {
             const SplitDev s = p->h->dev();
-            if (p->ut) {
+            if (band_subst_chosen<T>(s.kl, s.ku, p->Np, p->L)) {
+                const int rt = band_subst_rt<T>(s.kl, s.ku, p->Np, p->L, p->solve_rh);
+                const size_t bytes = band_subst_smem<T>(s.kl, s.ku, rt);
+                const auto key = std::make_pair(rt, bytes > 113 * 1024);
+                ssmem[key] = std::max(ssmem[key], bytes);
+                for (int j = 0; j < p->Np; ++j) sgroups[key].push_back(point(p, j, p->D, masked ? p->active : nullptr));
+                smaxL[key] = std::max(smaxL[key], p->L);
+            } else if (p->ut) {
                 int a, b, r;
                 sweep_key<T>(s.kl, s.ku, p->Np, p->L, &a, &b, &r, p->solve_rh);
                 const auto key = std::make_tuple(a, b, r);
@@ -1148,6 +1163,11 @@ static int run_solves_batch(const std::vector<nep_plan*>& ps, cudaStream_t st) {
                                              reinterpret_cast<cx<T>*>(p->D), masked ? p->active : nullptr, st,
                                              p->solve_rh));
             }
+        }
+        for (auto& g : sgroups) {
+            PointDesc* pd = nullptr;
+            NEP_TRY(upload(g.second, &pd));
+            NEP_TRY(band_subst_batch<T>(g.first.first, ssmem[g.first], (int)g.second.size(), smaxL[g.first], pd, st));
         }
         for (auto& g : groups) {
             PointDesc* pd = nullptr;
@@ -1463,6 +1483,16 @@ extern "C" int nep_plan_buffer(nep_plan_t p, const char* name, void** dev_ptr, s
     const nep_split* h = p->h;
     const size_t n = h->n, N = p->Np, L = p->L, K = p->K;
     const size_t esz = p->mixed ? sizeof(zf) : sizeof(zd);
+    if (!strcmp(name, "ut") && !p->ut_asked && band_sweeps_fit(h->kl, h->ku)) {
+        // a plan whose solves read U from the band makes the column copy when first asked for it, from the
+        // factors as they stand, and at every later execution
+        if (!p->ut) NEP_CUDA(cudaMallocAsync(&p->ut, esz * p->N * n * (h->kl + h->ku + 1), p->alloc_stream));
+        p->ut_asked = true;
+        NEP_CUDA(cudaDeviceSynchronize());  // the last execution may be on any stream
+        if (p->mixed) NEP_TRY(band_transpose_u<float>(h->dev(), p->Np, (const zf*)p->ab, (zf*)p->ut, p->alloc_stream));
+        else NEP_TRY(band_transpose_u<double>(h->dev(), p->Np, (const zd*)p->ab, (zd*)p->ut, p->alloc_stream));
+        NEP_CUDA(cudaStreamSynchronize(p->alloc_stream));
+    }
     struct B { const char* nm; void* ptr; size_t bytes; } tab[] = {
         {"F", p->F, sizeof(zd) * h->nterms * N},   {"coef", p->coef, sizeof(zd) * N * K},
         {"ab", p->ab, esz * N * n * h->ldab},       {"ipiv", p->ipiv, sizeof(int) * N * n},
@@ -2134,7 +2164,7 @@ extern "C" int nep_band_factor(nep_split_t h, int32_t npts, int32_t precision, v
 template <typename T>
 static int band_solve_step(const SplitDev& s, int npts, const cx<T>* ab, const int* ipiv, int L, cx<T>* B,
                            cudaStream_t st) {
-    if (!band_sweeps_fit(s.kl, s.ku) || npts <= 0 || L <= 0)
+    if (npts <= 0 || L <= 0 || !band_solve_needs_ut<T>(s.kl, s.ku, npts, L))
         return launch_band_solve<T>(s, npts, ab, nullptr, ipiv, L, B, nullptr, st);
     cx<T>* ut = nullptr;
     NEP_CUDA(cudaMallocAsync((void**)&ut, sizeof(cx<T>) * (size_t)npts * s.n * (s.kl + s.ku + 1), st));

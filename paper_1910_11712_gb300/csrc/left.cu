@@ -507,7 +507,7 @@ static int left_route(const SplitDev& s, bool adjoint, int P, const zd* lam, con
     NEP_TRY(w.get(&F, (size_t)nt * P));
     NEP_TRY(w.get(&Fd, (size_t)nt * P));
     NEP_TRY(w.get(&ab, (size_t)P * n * sh.ldab));
-    if (!adjoint && band_sweeps_fit(sh.kl, sh.ku)) NEP_TRY(w.get(&ut, (size_t)P * n * (sh.kl + sh.ku + 1)));
+    if (!adjoint && band_solve_needs_ut<T>(sh.kl, sh.ku, P, 1)) NEP_TRY(w.get(&ut, (size_t)P * n * (sh.kl + sh.ku + 1)));
     NEP_TRY(w.get(&ipiv, (size_t)P * n));
     NEP_TRY(w.get(&info, (size_t)P));
     NEP_TRY(w.get(&B, (size_t)P * n));

@@ -289,6 +289,19 @@ bool lu_tc_enabled();
 template <typename T>
 int launch_band_lu(const SplitDev& s, int npts, cx<T>* ab, int* ipiv, int* info, const int* active, cudaStream_t st,
                    int lu_kernel = LU_AUTO);
+// band_subst.cuh: the blocked substitution, reading U from the band; NEP_ERR_UNSUPPORTED when its windows
+// do not fit in shared memory. Its results are those of the sweeps, bit for bit.
+template <typename T>
+int band_subst_rt(int kl, int ku, int npts, int L, int rh_force = 0);  // right-hand sides per CTA, 0: none fit
+template <typename T>
+size_t band_subst_smem(int kl, int ku, int rt);
+template <typename T>
+int band_subst(const SplitDev& s, int npts, const cx<T>* ab, const int* ipiv, int L, cx<T>* B, const int* active,
+               cudaStream_t st, int rh_force = 0);
+template <typename T>
+int band_subst_batch(int rt, size_t smem, int count, int maxL, const PointDesc* pd, cudaStream_t st);
+template <typename T>
+bool band_subst_chosen(int kl, int ku, int npts, int L);  // band_lu.cu: this solve takes it
 // Narrow-band substitution sweeps (register windows of kl+1 and kl+ku+1 rows, up to 288).
 inline bool band_sweeps_fit(int kl, int ku) { return kl >= 1 && kl + 1 <= 288 && kl + ku + 1 <= 288; }
 // band_solve_blocked.cu: the blocked substitution for complex64 factors of wider bands (NB-step
@@ -296,6 +309,11 @@ inline bool band_sweeps_fit(int kl, int ku) { return kl >= 1 && kl + 1 <= 288 &&
 int band_solve_blocked_rhs(int kl, int ku, int L);
 int launch_band_solve_blocked(const SplitDev& s, int npts, const zf* ab, const int* ipiv, int L, zf* B,
                               const int* active, cudaStream_t st);
+// Whether a solve needs the column copy of U (ut) that the sweeps read.
+template <typename T>
+inline bool band_solve_needs_ut(int kl, int ku, int npts, int L) {
+    return band_sweeps_fit(kl, ku) && !band_subst_chosen<T>(kl, ku, npts, L);
+}
 // ut (npts x n x (kl+ku+1)): the U factor by columns, written by band_transpose_u after the LU.
 template <typename T>
 int band_sweeps(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, const int* ipiv, int L, cx<T>* B,

@@ -963,7 +963,7 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
     NEP_TRY(w.get(&tnorm, 1));
     NEP_TRY(w.get(&ipiv, (size_t)n));
     NEP_TRY(w.get(&info, 1));
-    if (band_sweeps_fit(s.kl, s.ku)) NEP_TRY(w.get(&ut, (size_t)n * (kv + 1)));
+    if (band_solve_needs_ut<float>(s.kl, s.ku, 1, 1)) NEP_TRY(w.get(&ut, (size_t)n * (kv + 1)));
     NEP_TRY(w.get(&V, (size_t)N * (lin.toar ? 1 : kmax + 1)));
     NEP_TRY(w.get(&C, (size_t)nt * n));
     NEP_TRY(w.get(&rhs, (size_t)n));

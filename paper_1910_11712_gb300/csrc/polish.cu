@@ -183,7 +183,7 @@ int rii_polish(const SplitDev& s, int P, zd* lam, zd* X, double* eta, int* its, 
     NEP_TRY(w.get(&c, (size_t)P * nc));
     NEP_TRY(w.get(&active, (size_t)P));
     NEP_TRY(w.get(&cnt, 1));
-    if (band_sweeps_fit(s.kl, s.ku)) NEP_TRY(w.get(&ut, (size_t)P * n * (kv + 1)));
+    if (band_solve_needs_ut<T>(s.kl, s.ku, P, nc)) NEP_TRY(w.get(&ut, (size_t)P * n * (kv + 1)));
     // T(sigma_p) at the starting eigenvalues, factored once
     rii_coeffs_kernel<<<ceil_div(P * nt, 128), 128, 0, st>>>(s, P, lam, F);
     NEP_CHECK_LAUNCH();
