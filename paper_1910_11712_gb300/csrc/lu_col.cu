@@ -289,6 +289,11 @@ __global__ void __launch_bounds__(512, 1)
     // Step cc on this warp's columns: publish the pivot row (row Pc; the entering row when
     // Pc = cc+kl), the pivot's slot takes the entering row, a(r, k) -= l(r) u(k), U(cc, k) to
     // the band, and the slot of column cc+1 (if this warp holds it) empties for column cc+1+CS.
+    // Columns beyond the step's reach (the farthest pivot row so far + ku) are zero in the pivot row: the
+    // complex128 update, bound by the FP64 units, leaves them out (half the window without interchanges:
+    // 64 points at bandwidth 64, n = 4096, 42.8 -> 23.0 ms). The complex64 one, bound by the chain of pivots,
+    // lost more to the test than it saved (3.92 -> 4.41 ms).
+    int reach = 0;
     auto run_step = [&](int cc, int Pc, const bool(&ispc)[RPL]) __attribute__((always_inline)) {
         const int e = cc % RING, lb = cc % 3;
         // the pivot row's lane publishes its registers, then takes the entering row into them
@@ -346,6 +351,7 @@ __global__ void __launch_bounds__(512, 1)
             for (int q = 0; q < RPL; ++q) lqc[q] = vr[q] ? lvec[lb][lane + 32 * q] : mk<T>(0, 0);
 #pragma unroll
             for (int p = 0; p < CPW; ++p) {
+                if (toff(p, cc) > reach - cc) continue;
                 const cx<T> u = xrow[warp][p];
 #pragma unroll
                 for (int q = 0; q < RPL; ++q) a[q][p] = fms(a[q][p], lqc[q], u);
@@ -409,6 +415,7 @@ __global__ void __launch_bounds__(512, 1)
         }
         const int cb = c % 3, re = c + kl;
         const int P = piv_s[cb];
+        if constexpr (!PAIRED) reach = max(reach, P + ku);
         bool isp[RPL];
 #pragma unroll
         for (int q = 0; q < RPL; ++q) {

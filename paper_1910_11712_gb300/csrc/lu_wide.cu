@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(512, 1)
     int* src = reinterpret_cast<int*>(Us + (int64_t)NB * CHW);  // RW: row permutation of the panel
     int* plist = src + RW;                                      // partner rows (local, >= nbc)
     __shared__ int piv_sh[NB];
-    __shared__ int info_s, npart_s;
+    __shared__ int info_s, npart_s, far_s;
     if (tid == 0) info_s = 0;
 
     // window: zero, then rows 0 .. RW-1 of the band
@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(512, 1)
     load_rows(0, min(RW, n));
     __syncthreads();
 
+    int reach = 0;  // last column that a row of U so far can reach: max over the pivots of their row + ku
     for (int p0 = 0; p0 < n; p0 += NB) {
         const int nbc = min(NB, n - p0);
         const int pr = min(RW, n - p0);  // panel rows (local 0 .. pr-1)
@@ -146,9 +147,10 @@ __global__ void __launch_bounds__(512, 1)
         for (int l = tid; l < RW; l += nthr) src[l] = l;
         __syncthreads();
         if (tid == 0) {
-            int np = 0;
+            int np = 0, far = 0;
             for (int k = 0; k < nbc; ++k) {
                 const int b = piv_sh[k] - p0;
+                far = max(far, b);
                 if (b != k) {
                     const int t = src[k];
                     src[k] = src[b];
@@ -161,12 +163,15 @@ __global__ void __launch_bounds__(512, 1)
                 }
             }
             npart_s = np;
+            far_s = far;
         }
         __syncthreads();
         const int npart = npart_s;
 
         // ---- 2, 3. trailing columns [p0+nbc, cend) in chunks, rows [p0+nbc, rend)
-        const int cend = min(p0 + nbc + kv, n), rend = min(p0 + nbc + kl, n);
+        // columns beyond the reach are zero in the panel's rows of U: the trailing update ends there
+        reach = max(reach, p0 + far_s + ku);
+        const int cend = min(reach + 1, n), rend = min(p0 + nbc + kl, n);
         const int mr = rend - (p0 + nbc);
         for (int c0 = p0 + nbc; c0 < cend; c0 += CHW) {
             const int cw = min(CHW, cend - c0);
