@@ -419,7 +419,8 @@ __global__ void __launch_bounds__(512)
 // Whether a solve takes the blocked substitution (band_subst.cuh) rather than the register-window sweeps.
 // Its chain from step to step is shorter (bandwidth 64: 114 ns against 162 with one right-hand side) and it
 // needs no column copy of U, but its arithmetic costs more instructions per right-hand side: measured, ms
-// per solve, sweeps (without the copy of U) against substitution, points x right-hand sides:
+// per solve, sweeps (without the copy of U) against substitution, points x right-hand sides, both with
+// backward windows of kl + ku rows:
 //   complex64, bandwidth 64: 1 x 1 .661 / .463, 9 x 4 .680 / .549, 64 x 16 .820 / .673, 128 x 16 1.11 / 2.34
 //   (64 of its 256 CTAs in a last wave or 16 right-hand sides a CTA); bandwidth 24: 32 x 8 .090 / .065;
 //   bandwidth 40: 64 x 16 .324 / .238, 128 x 32 .562 / .735; bandwidth 97: 64 x 16 2.40 / 2.62;

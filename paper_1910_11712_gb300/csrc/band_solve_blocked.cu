@@ -15,7 +15,8 @@
 //     thread per row with the R right-hand sides in registers.
 // Backward, block of rows top .. c1 from the bottom, on the window [top - kl - ku, c1]:
 //   * the upper nb x nb triangle gives x (one warp per right-hand side);
-//   * the rows above take w -= U(rows, top .. c1) x, U read straight from the band rows.
+//   * the rows above take w -= U(rows, top .. c1) x, U read straight from the band rows; a point without
+//     interchanges has ku rows there, not kl + ku.
 // The windows are rings of rows in shared memory; rows enter by asynchronous copies into the slots
 // the finished block frees, and the next block's L columns and pivots are copied while the current
 // block runs. Results equal the sweeps' up to the order of the FP32 roundings.
@@ -203,6 +204,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
 
     // ===================================================================== backward
     {
+        const int kv = u_reach(n, ku, ipiv);  // this point's U is no wider
         const int PB = NB + kv;
         zf* W = sm;                                  // PB x RS: row r at slot r mod PB
         zf* U0 = W + (size_t)PB * RS;                // 2 x NB x (NB+1): U(top+i, top+k) at i (NB+1) + k

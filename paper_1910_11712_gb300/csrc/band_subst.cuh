@@ -3,7 +3,8 @@
 // parallel.
 //
 // One CTA per (point, RT right-hand sides) runs the forward sweep (row interchanges and unit lower L,
-// window of kl rows) and then the backward sweep (U, window of kl + ku rows). Both are written in steps
+// window of kl rows) and then the backward sweep (U, window of the rows it can reach, ku without
+// interchanges and kl + ku at most). Both are written in steps
 // s: row s forward, row n-1-s backward; local row i of a block is step s0 + i. A block's coefficients
 // form a panel P(i, k), k < 16:
 //   forward   P(i, k) = L(c0+i, c0+k), 0 < i - k <= kl, read from ab[(c0+k) ldab + kv + i - k];
@@ -35,9 +36,9 @@
 // What bounds it: the chain from block to block (two barriers' worth of shuffles and 16 dependent
 // multiply-adds, 1.8 us a block at bandwidth 64) up to one CTA per SM; beyond that the staging and
 // shared-memory instructions of the update, which is why many columns of complex64 keep the sweeps.
-// n = 4096, bandwidth 64, complex64: one right-hand side 0.463 ms (sweeps .661), 64 points x 16 0.673
-// (.820); complex128: 9 x 1 3.62 ms (10.6), bandwidth 40 at 128 x 32 9.1 (11.1); bandwidth 200, n = 3000,
-// 16 x 16 9.8 (12.5, one step at a time).
+// n = 4096, bandwidth 64, complex64: one right-hand side 0.461 ms (sweeps .661), 64 points x 16 0.612
+// (.820); complex128: 9 x 1 3.62 ms (10.6), 64 x 16 8.5 (10.7), bandwidth 40 at 128 x 32 7.5 (11.1);
+// bandwidth 200 with interchanges throughout, n = 3000, 16 x 16 9.8 (12.5, one step at a time).
 #pragma once
 #include <algorithm>
 #include <cstdlib>
@@ -471,7 +472,7 @@ __global__ void __launch_bounds__(subst::threads(RT), 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cx<T>* smem = reinterpret_cast<cx<T>*>(smem_raw);
     subst_sweep<T, RT, false>(n, kl, kl + ku, ldab, ab, ipiv, nr, B, smem, smem_bytes);
-    subst_sweep<T, RT, true>(n, kl, kl + ku, ldab, ab, ipiv, nr, B, smem, smem_bytes);
+    subst_sweep<T, RT, true>(n, kl, u_reach(n, ku, ipiv), ldab, ab, ipiv, nr, B, smem, smem_bytes);
 }
 
 // Shared memory of a launch: what three stages of both sweeps take if two CTAs then share an SM, else

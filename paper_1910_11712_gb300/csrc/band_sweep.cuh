@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(256)
     band_sweep_kernel(int n, int kl, int ku, int ldab, const cx<T>* __restrict__ ab_all,
                       const cx<T>* __restrict__ ut_all, const int* __restrict__ ipiv_all, int L,
                       cx<T>* __restrict__ B_all, const int* __restrict__ active, int CH,
-                      const PointDesc* __restrict__ pd) {
+                      const PointDesc* __restrict__ pd, int rpl_done) {
     int j = blockIdx.x;
     if (pd) {  // a point of one of several problems sharing the launch (the grid covers the largest L)
         const PointDesc d = pd[blockIdx.x];
@@ -53,7 +53,6 @@ __global__ void __launch_bounds__(256)
     if (active && !active[j]) return;
     constexpr int RS = 32 * RPL, RPLP = RPL | 1, RSP = 32 * RPLP + 1;
     const int kv = kl + ku;
-    const int W = BWD ? kv : kl;  // window width: rows updated per step
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nwarps = (blockDim.x >> 5) / 2;  // compute warps; warps nwarps .. 2 nwarps-1 produce
     const bool producer = warp >= nwarps;
@@ -62,6 +61,11 @@ __global__ void __launch_bounds__(256)
     const int64_t cstride = BWD ? kv + 1 : ldab;
     const cx<T>* colbase = BWD ? ut_all + (int64_t)j * n * (kv + 1) : ab_all + (int64_t)j * n * ldab + kv;
     const int* ipiv = ipiv_all + (int64_t)j * n;
+    // Window width: rows updated per step. Backward it is what this point's U can reach (ku without
+    // interchanges); the points that need no more than rpl_done registers a lane belong to another
+    // launch of the sweep, those that need more than RPL to a third.
+    const int W = BWD ? u_reach(n, ku, ipiv) : kl;
+    if (BWD && (W >= RS || W < 32 * rpl_done)) return;
     bool has[RH];
     cx<T>* bh[RH];
 #pragma unroll
@@ -236,7 +240,7 @@ __global__ void band_transpose_u_kernel(int n, int kv, int ldab, const cx<T>* __
 
 template <typename T, int RPL, bool BWD, int RH>
 static int run_sweep(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, const int* ipiv, int L,
-                     cx<T>* B, const int* active, cudaStream_t st) {
+                     cx<T>* B, const int* active, cudaStream_t st, int rpl_done) {
     constexpr int RSP = 32 * (RPL | 1) + 1;
     const int warps = (L + RH - 1) / RH;
     // four compute warps per CTA (those beyond the right-hand sides idle), and as many producer
@@ -254,7 +258,7 @@ static int run_sweep(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* 
     if (smem > 227 * 1024) return NEP_ERR_UNSUPPORTED;
     NEP_CUDA(allow_max_dynamic_smem(band_sweep_kernel<T, RPL, BWD, RH>));
     band_sweep_kernel<T, RPL, BWD, RH><<<dim3(npts, gy), 2 * wpb * 32, smem, st>>>(s.n, s.kl, s.ku, s.ldab, ab, ut,
-                                                                             ipiv, L, B, active, CH, nullptr);
+                                                                             ipiv, L, B, active, CH, nullptr, rpl_done);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
 }
@@ -262,7 +266,7 @@ static int run_sweep(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* 
 // The same sweep over points of several problems (descriptors pd_dev[count]; maxL the most
 // right-hand sides of any of them): the launch shape of run_sweep, per-point arithmetic unchanged.
 template <typename T, int RPL, bool BWD, int RH>
-static int run_sweep_batch(int count, int maxL, const PointDesc* pd_dev, cudaStream_t st) {
+static int run_sweep_batch(int count, int maxL, const PointDesc* pd_dev, cudaStream_t st, int rpl_done) {
     constexpr int RSP = 32 * (RPL | 1) + 1;
     const int warps = (maxL + RH - 1) / RH;
     const int wpb = 4;
@@ -278,33 +282,34 @@ static int run_sweep_batch(int count, int maxL, const PointDesc* pd_dev, cudaStr
     NEP_CUDA(allow_max_dynamic_smem(band_sweep_kernel<T, RPL, BWD, RH>));
     band_sweep_kernel<T, RPL, BWD, RH><<<dim3(count, gy), 2 * wpb * 32, smem, st>>>(0, 0, 0, 0, nullptr, nullptr,
                                                                               nullptr, maxL, nullptr, nullptr, CH,
-                                                                              pd_dev);
+                                                                              pd_dev, rpl_done);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
 }
 
 template <typename T, bool BWD, int RH>
-static int sweep_batch_rpl(int rpl, int count, int maxL, const PointDesc* pd, cudaStream_t st) {
+static int sweep_batch_rpl(int rpl, int count, int maxL, const PointDesc* pd, cudaStream_t st, int done) {
     switch (rpl) {
-        case 1: return run_sweep_batch<T, 1, BWD, RH>(count, maxL, pd, st);
-        case 2: return run_sweep_batch<T, 2, BWD, RH>(count, maxL, pd, st);
-        case 3: return run_sweep_batch<T, 3, BWD, RH>(count, maxL, pd, st);
-        case 4: return run_sweep_batch<T, 4, BWD, RH>(count, maxL, pd, st);
-        case 5: return run_sweep_batch<T, 5, BWD, RH>(count, maxL, pd, st);
-        case 6: return run_sweep_batch<T, 6, BWD, RH>(count, maxL, pd, st);
-        case 7: return run_sweep_batch<T, 7, BWD, RH>(count, maxL, pd, st);
-        case 8: return run_sweep_batch<T, 8, BWD, RH>(count, maxL, pd, st);
-        case 9: return run_sweep_batch<T, 9, BWD, RH>(count, maxL, pd, st);
+        case 1: return run_sweep_batch<T, 1, BWD, RH>(count, maxL, pd, st, done);
+        case 2: return run_sweep_batch<T, 2, BWD, RH>(count, maxL, pd, st, done);
+        case 3: return run_sweep_batch<T, 3, BWD, RH>(count, maxL, pd, st, done);
+        case 4: return run_sweep_batch<T, 4, BWD, RH>(count, maxL, pd, st, done);
+        case 5: return run_sweep_batch<T, 5, BWD, RH>(count, maxL, pd, st, done);
+        case 6: return run_sweep_batch<T, 6, BWD, RH>(count, maxL, pd, st, done);
+        case 7: return run_sweep_batch<T, 7, BWD, RH>(count, maxL, pd, st, done);
+        case 8: return run_sweep_batch<T, 8, BWD, RH>(count, maxL, pd, st, done);
+        case 9: return run_sweep_batch<T, 9, BWD, RH>(count, maxL, pd, st, done);
     }
     return NEP_ERR_UNSUPPORTED;
 }
 
 template <typename T, bool BWD>
-static int sweep_batch_dispatch(int rpl, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st) {
+static int sweep_batch_dispatch(int rpl, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st,
+                                int done) {
     switch (rh) {
-        case 1: return sweep_batch_rpl<T, BWD, 1>(rpl, count, maxL, pd, st);
-        case 4: return sweep_batch_rpl<T, BWD, 4>(rpl, count, maxL, pd, st);
-        default: return sweep_batch_rpl<T, BWD, 2>(rpl, count, maxL, pd, st);
+        case 1: return sweep_batch_rpl<T, BWD, 1>(rpl, count, maxL, pd, st, done);
+        case 4: return sweep_batch_rpl<T, BWD, 4>(rpl, count, maxL, pd, st, done);
+        default: return sweep_batch_rpl<T, BWD, 2>(rpl, count, maxL, pd, st, done);
     }
 }
 
@@ -336,53 +341,61 @@ static int sweep_rh(int chains) {
 
 template <typename T, bool BWD, int RH>
 static int sweep_rpl(int rpl, const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, const int* ipiv, int L,
-                     cx<T>* B, const int* active, cudaStream_t st) {
+                     cx<T>* B, const int* active, cudaStream_t st, int done) {
     switch (rpl) {
-        case 1: return run_sweep<T, 1, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 2: return run_sweep<T, 2, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 3: return run_sweep<T, 3, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 4: return run_sweep<T, 4, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 5: return run_sweep<T, 5, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 6: return run_sweep<T, 6, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 7: return run_sweep<T, 7, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 8: return run_sweep<T, 8, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
-        case 9: return run_sweep<T, 9, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st);
+        case 1: return run_sweep<T, 1, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 2: return run_sweep<T, 2, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 3: return run_sweep<T, 3, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 4: return run_sweep<T, 4, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 5: return run_sweep<T, 5, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 6: return run_sweep<T, 6, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 7: return run_sweep<T, 7, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 8: return run_sweep<T, 8, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 9: return run_sweep<T, 9, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
     }
     return NEP_ERR_UNSUPPORTED;
 }
 
 template <typename T, bool BWD>
 static int sweep_dispatch(int rpl, const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, const int* ipiv,
-                          int L, cx<T>* B, const int* active, cudaStream_t st, int rh_force) {
+                          int L, cx<T>* B, const int* active, cudaStream_t st, int rh_force, int done) {
     switch (rh_force == 1 || rh_force == 2 || rh_force == 4 ? rh_force : sweep_rh<T>(npts * L)) {
-        case 1: return sweep_rpl<T, BWD, 1>(rpl, s, npts, ab, ut, ipiv, L, B, active, st);
-        case 4: return sweep_rpl<T, BWD, 4>(rpl, s, npts, ab, ut, ipiv, L, B, active, st);
-        default: return sweep_rpl<T, BWD, 2>(rpl, s, npts, ab, ut, ipiv, L, B, active, st);
+        case 1: return sweep_rpl<T, BWD, 1>(rpl, s, npts, ab, ut, ipiv, L, B, active, st, done);
+        case 4: return sweep_rpl<T, BWD, 4>(rpl, s, npts, ab, ut, ipiv, L, B, active, st, done);
+        default: return sweep_rpl<T, BWD, 2>(rpl, s, npts, ab, ut, ipiv, L, B, active, st, done);
     }
 }
 
+// The backward sweep runs in up to two launches: points whose U stayed within ku rounded up to whole
+// registers, then the rest (kl + ku registers; a point that has run returns at once). Without interchanges
+// the first does all the work with about half the registers and staged coefficients. Solve, ms before ->
+// after: bandwidth 128, 128 points x 16: 7.13 -> 5.06; bandwidth 97, 64 x 32: 3.23 -> 2.85; bandwidth 64,
+// 128 x 32: 1.80 -> 1.66; the blocked kernel at bandwidth 576, 64 x 16: 13.6 -> 10.5.
 // Registers per lane of a sweep's window for window width W: RS = 32 RPL > W. (A variant with
 // RS = W, the entering row moved ahead of the step's update, executed fewer instructions on
 // bandwidth 64 but ran no faster: 0.349 + 0.506 ms per solve against 0.345 + 0.476; each step is
 // bound by its dependency chain rather than by issue.)
 inline int sweep_rpl_of(int W) { return (W + 1 + 31) / 32; }
 
-// Sweep launch shape of a problem: rows per lane of the forward and backward windows and right-hand
+// Sweep launch shape of a problem: rows per lane of the forward window and of the backward one (without
+// interchanges and at most) and right-hand
 // sides per warp (from the problem's own chain count N L). Points of problems with equal keys share
 // batched launches.
 template <typename T>
-void sweep_key(int kl, int ku, int npts, int L, int* rplf, int* rplb, int* rh, int rh_force) {
+void sweep_key(int kl, int ku, int npts, int L, int* rplf, int* rplu, int* rplb, int* rh, int rh_force) {
     *rplf = sweep_rpl_of(kl);
+    *rplu = sweep_rpl_of(ku);
     *rplb = sweep_rpl_of(kl + ku);
     *rh = rh_force == 1 || rh_force == 2 || rh_force == 4 ? rh_force : sweep_rh<T>(npts * L);
 }
 
 template <typename T>
-int band_sweeps_batch(int rplf, int rplb, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st) {
+int band_sweeps_batch(int rplf, int rplu, int rplb, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st) {
     if (count <= 0 || maxL <= 0) return NEP_OK;
-    const int rc = sweep_batch_dispatch<T, false>(rplf, rh, count, maxL, pd, st);
+    int rc = sweep_batch_dispatch<T, false>(rplf, rh, count, maxL, pd, st, 0);
+    if (rc == NEP_OK && rplu < rplb) rc = sweep_batch_dispatch<T, true>(rplu, rh, count, maxL, pd, st, 0);
     if (rc != NEP_OK) return rc;
-    return sweep_batch_dispatch<T, true>(rplb, rh, count, maxL, pd, st);
+    return sweep_batch_dispatch<T, true>(rplb, rh, count, maxL, pd, st, rplu < rplb ? rplu : 0);
 }
 
 template <typename T>
@@ -390,10 +403,12 @@ int band_sweeps(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, c
                 const int* active, cudaStream_t st, int rh_force) {
     if (npts <= 0 || L <= 0) return NEP_OK;
     if (!band_sweeps_fit(s.kl, s.ku) || !ut) return NEP_ERR_UNSUPPORTED;
-    const int rplf = sweep_rpl_of(s.kl), rplb = sweep_rpl_of(s.kl + s.ku);
-    const int rc = sweep_dispatch<T, false>(rplf, s, npts, ab, ut, ipiv, L, B, active, st, rh_force);
+    const int rplf = sweep_rpl_of(s.kl), rplu = sweep_rpl_of(s.ku), rplb = sweep_rpl_of(s.kl + s.ku);
+    int rc = sweep_dispatch<T, false>(rplf, s, npts, ab, ut, ipiv, L, B, active, st, rh_force, 0);
+    // backward: points whose U the interchanges left within rplu registers a lane, then the others
+    if (rc == NEP_OK && rplu < rplb) rc = sweep_dispatch<T, true>(rplu, s, npts, ab, ut, ipiv, L, B, active, st, rh_force, 0);
     if (rc != NEP_OK) return rc;
-    return sweep_dispatch<T, true>(rplb, s, npts, ab, ut, ipiv, L, B, active, st, rh_force);
+    return sweep_dispatch<T, true>(rplb, s, npts, ab, ut, ipiv, L, B, active, st, rh_force, rplu < rplb ? rplu : 0);
 }
 
 template <typename T>

@@ -73,4 +73,28 @@ __device__ __forceinline__ void set_reg(cx<T> (&a)[RPL], int q, cx<T> v) {
         if (t == q) a[t] = v;
 }
 
+// Columns beyond the diagonal that U can reach: ku + the farthest pivot row below its step (kl + ku at
+// most), from the interchanges. Run by the whole CTA; ends with a barrier. Without interchanges the
+// backward substitution then reads and multiplies ku columns of U, not kl + ku.
+__device__ __forceinline__ int u_reach(int n, int ku, const int* __restrict__ ipiv) {
+    __shared__ int far_s;
+    if (threadIdx.x == 0) far_s = 0;
+    __syncthreads();
+    int far = 0;
+    for (int c0 = threadIdx.x; c0 < n; c0 += 8 * blockDim.x) {
+        int p[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int c = c0 + u * blockDim.x;
+            p[u] = c < n ? ipiv[c] - c : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) far = max(far, p[u]);
+    }
+    far = __reduce_max_sync(0xffffffffu, far);
+    if ((threadIdx.x & 31) == 0 && far > 0) atomicMax(&far_s, far);
+    __syncthreads();
+    return ku + far_s;
+}
+
 }  // namespace nep

@@ -1138,8 +1138,8 @@ static int run_solves_batch(const std::vector<nep_plan*>& ps, cudaStream_t st) {
     // one solve of every live plan's points in shared launches: the blocked substitution per right-hand
     // sides a CTA and whether two CTAs share an SM, the register-window sweeps per shape key
     auto solve_all = [&](const std::vector<nep_plan*>& live, bool masked) -> int {
-        std::map<std::tuple<int, int, int>, std::vector<PointDesc>> groups;
-        std::map<std::tuple<int, int, int>, int> maxL;
+        std::map<std::tuple<int, int, int, int>, std::vector<PointDesc>> groups;
+        std::map<std::tuple<int, int, int, int>, int> maxL;
         std::map<std::pair<int, bool>, std::vector<PointDesc>> sgroups;
         std::map<std::pair<int, bool>, int> smaxL;
         std::map<std::pair<int, bool>, size_t> ssmem;
@@ -1153,9 +1153,9 @@ static int run_solves_batch(const std::vector<nep_plan*>& ps, cudaStream_t st) {
                 for (int j = 0; j < p->Np; ++j) sgroups[key].push_back(point(p, j, p->D, masked ? p->active : nullptr));
                 smaxL[key] = std::max(smaxL[key], p->L);
             } else if (p->ut) {
-                int a, b, r;
-                sweep_key<T>(s.kl, s.ku, p->Np, p->L, &a, &b, &r, p->solve_rh);
-                const auto key = std::make_tuple(a, b, r);
+                int a, u, b, r;
+                sweep_key<T>(s.kl, s.ku, p->Np, p->L, &a, &u, &b, &r, p->solve_rh);
+                const auto key = std::make_tuple(a, u, b, r);
                 for (int j = 0; j < p->Np; ++j) groups[key].push_back(point(p, j, p->D, masked ? p->active : nullptr));
                 maxL[key] = std::max(maxL[key], p->L);
             } else {
@@ -1172,7 +1172,7 @@ static int run_solves_batch(const std::vector<nep_plan*>& ps, cudaStream_t st) {
         for (auto& g : groups) {
             PointDesc* pd = nullptr;
             NEP_TRY(upload(g.second, &pd));
-            NEP_TRY(band_sweeps_batch<T>(std::get<0>(g.first), std::get<1>(g.first), std::get<2>(g.first),
+            NEP_TRY(band_sweeps_batch<T>(std::get<0>(g.first), std::get<1>(g.first), std::get<2>(g.first), std::get<3>(g.first),
                                          (int)g.second.size(), maxL[g.first], pd, st));
         }
         return NEP_OK;
