@@ -1,5 +1,6 @@
 // Kernel (b) for wide bands in complex64: the blocked banded LU of lu_wide.cu with its trailing
-// update A22 -= L~21 U12 on the fifth-generation tensor core. One CTA per quadrature point.
+// update A22 -= L~21 U12 on the fifth-generation tensor core. One CTA per quadrature point, or a cluster of
+// two that share the trailing columns and the operand image.
 //
 // Elimination, pivot rule and stored factors are those of lu_wide.cu (the unblocked LU's order of
 // operations per element); only the trailing product changes arithmetic: it runs as TF32 tensor-
@@ -22,7 +23,7 @@
 //        shared-memory layout, 64 complex rows (128 MMA rows) per tile, hi part then lo part;
 //   4.   per tile of 128 trailing columns: B (from U12) written to shared memory by the threads;
 //        per tile of 64 trailing rows: its A tile staged by a TMA tensor copy (double-buffered),
-//        24 MMAs (M = 128, N = 128, K = 8) into one of two tensor-memory accumulators, and the
+//        24 MMAs (M = 128, N <= 128, K = 8) into one of two tensor-memory accumulators, and the
 //        accumulator drained by all 16 warps (tcgen05.ld), which subtract it from the window.
 // The shared memory of steps 0-3 (the panel) and of step 4 (B, two A buffers) is shared.
 #include <cuda.h>
@@ -231,9 +232,9 @@ __global__ void __launch_bounds__(512, 1)
                  int CWp, float* __restrict__ aimg_all, int nmt_max, const __grid_constant__ CUtensorMap tmap,
                  int* __restrict__ err, const PointDesc* __restrict__ pd, int passes, int nsplit, int scratch_max_kl) {
     // nsplit CTAs (a cluster) per point: each factors the panel itself and takes its share of the
-    // trailing columns; CTA 0 writes the panel's outputs. Each CTA has an operand image of its own.
+    // trailing columns; CTA 0 writes the panel's outputs. They build half of the point's operand image each.
     const int j = blockIdx.x / nsplit, part = blockIdx.x - j * nsplit;
-    const int img = blockIdx.x;  // operand image and its TMA coordinate
+    const int img = j;  // operand image and its TMA coordinate
     zf* ab = ab_all + (int64_t)j * n * ldab;
     int* ipiv = ipiv_all + (int64_t)j * n;
     int* info_out = info_all + j;
@@ -274,10 +275,12 @@ __global__ void __launch_bounds__(512, 1)
     __shared__ int wlab[2][PW16], wphys[2][PW16], diag_s[2];
     __shared__ uint32_t tmem_s;
     __shared__ __align__(8) uint64_t full_b[2], done_b[2], free_b[2];
+    __shared__ int tma_seen[2];
 
     if (tid == 0) {
         info_s = 0;
         abort_s = 0;
+        tma_seen[0] = tma_seen[1] = 0;
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(&full_b[b], 1);
             tc::mbar_init(&done_b[b], 1);
@@ -309,8 +312,8 @@ __global__ void __launch_bounds__(512, 1)
         }
         return true;
     };
-    // TMA loads issued into each A buffer and awaited by the MMA issuer (thread 0 only)
-    int tma_issued[2] = {0, 0}, tma_seen[2] = {0, 0};
+    // TMA loads issued into each A buffer (thread 0) and awaited by the MMA issuers
+    int tma_issued[2] = {0, 0};
     long long g = 0;  // tiles processed so far: accumulator / A buffer g & 1, phase (g >> 1) & 1
 
     auto load_rows = [&](int r0, int r1) {
@@ -476,9 +479,10 @@ __global__ void __launch_bounds__(512, 1)
         // ---- 3. A operand image of L~21 (global, the tensor core's layout), tiles of 64 rows
         const int nmt = mr > 0 ? (mr + MT - 1) / MT : 0;
         const int ntn = (chi > clo && mr > 0) ? (chi - clo + NT - 1) / NT : 0;
-        if (ntn > 0) {
-            for (int e = tid; e < nmt * PART; e += nthr) {
-                const int mt = e / PART, f = e - mt * PART;
+        if (ctot > 0 && nmt > 0) {
+            const int mine = (nmt - part + nsplit - 1) / nsplit;  // tiles part, part + nsplit, ...
+            for (int e = tid; e < mine * PART; e += nthr) {
+                const int mt = e / PART * nsplit + part, f = e % PART;
                 int r, k;
                 tile_rk(f, r, k);
                 const int i = mt * MT + (r >> 1), cc = k & (NB - 1);
@@ -496,7 +500,8 @@ __global__ void __launch_bounds__(512, 1)
             }
             tc::fence_async_global();
         }
-        __syncthreads();
+        csync();
+        if (nsplit > 1) tc::fence_async_global();  // the other CTA's half, before this one's copies read it
 
         // ---- 4. A22 -= L~21 U12 on the tensor core
         for (int nt = 0; nt < ntn; ++nt) {
@@ -541,25 +546,31 @@ __global__ void __launch_bounds__(512, 1)
             tc::fence_async_shared();
             __syncthreads();
 
-            // MMA issue for tile t of this column tile (thread 0)
+            // MMA issue for tile t of this column tile: one lane, of another warp for every tile, since it
+            // comes to its part of the window about 1.5 us later than the rest (bandwidth 576, 64 points: the
+            // update 126 -> 86 us a panel, the factorisation 117 -> 97 ms; with thread 0 issuing every
+            // product, each tile waited for its warp)
             auto issue = [&](int t) {
                 const long long gt = g + t;
                 const int b = (int)(gt & 1);
                 if (!wait(&full_b[b], (uint32_t)((gt >> 1) & 1))) return;
-                ++tma_seen[b];
+                atomicAdd(&tma_seen[b], 1);
                 if (gt >= 2 && !wait(&free_b[b], (uint32_t)(((gt >> 1) - 1) & 1))) return;
                 tc::tc_fence_after();
                 const uint32_t d = tmem + (uint32_t)(b * NT);
                 const uint32_t abase = tc::smem_u32(b ? Abuf1 : Abuf0), bbase = tc::smem_u32(Bimg);
-                const int pa[3] = {0, 0, 1}, pb[3] = {0, 1, 0};  // hi*hi, hi*lo, lo*hi
-                // passes = 3: hi*hi + hi*lo + lo*hi (~FP32); passes = 1: hi*hi alone (TF32 operands)
-                for (int ps = 0; ps < passes; ++ps)
+                // passes = 3: hi*hi + hi*lo + lo*hi (~FP32); passes = 1: hi*hi alone (TF32 operands).
+                // (the start address is the descriptor's low field, in 16 bytes: steps add to it)
+                const uint64_t ad = tc::smem_desc(abase, LBO, SBO), bd = tc::smem_desc(bbase, LBO, SBO);
+                constexpr uint64_t step = 2 * LBO / 16, lo = PART * 4 / 16;
 #pragma unroll
-                    for (int s = 0; s < KR / 8; ++s) {
-                        const uint64_t ad = tc::smem_desc(abase + (uint32_t)(pa[ps] * PART * 4) + s * 2 * LBO, LBO, SBO);
-                        const uint64_t bd = tc::smem_desc(bbase + (uint32_t)(pb[ps] * PART * 4) + s * 2 * LBO, LBO, SBO);
-                        tc::mma_tf32(d, ad, bd, idesc, (ps | s) != 0);
-                    }
+                for (int s = 0; s < KR / 8; ++s) tc::mma_tf32(d, ad + s * step, bd + s * step, idesc, s != 0);
+                if (passes == 3) {
+#pragma unroll
+                    for (int s = 0; s < KR / 8; ++s) tc::mma_tf32(d, ad + s * step, bd + lo + s * step, idesc, 1);
+#pragma unroll
+                    for (int s = 0; s < KR / 8; ++s) tc::mma_tf32(d, ad + lo + s * step, bd + s * step, idesc, 1);
+                }
                 tc::mma_commit(&done_b[b]);
             };
             for (int t = 0; t < nmt; ++t) {
@@ -573,10 +584,8 @@ __global__ void __launch_bounds__(512, 1)
                     if (i < mr)
                         tc::prefetch_l2(W + wi(nbc + i, c0 - p0 + cb + lane));
                 }
-                if (tid == 0) {
-                    if (t == 0) issue(0);
-                    if (t + 1 < nmt) issue(t + 1);
-                }
+                if (tid == 0 && t == 0) issue(0);
+                if (lane == 0 && t + 1 < nmt && warp == (int)((gt + 1) & 15)) issue(t + 1);
                 __syncwarp();
                 const bool ok = __all_sync(0xffffffffu, wait(&done_b[b], ph));
                 // MMA t is done: its A buffer takes tile t + 2 (the copy runs during this epilogue)
@@ -771,14 +780,14 @@ int launch_band_lu_tc(const SplitDev& s, int npts, zf* ab, int* ipiv, int* info,
     float* aimg = nullptr;
     int* err = nullptr;
     NEP_CUDA(cudaMallocAsync((void**)&win, sizeof(zf) * (size_t)rwp * cwp * npts, st));
-    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * npts * nsplit, st);
+    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * npts, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&err, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
     CUtensorMap tmap;
     if (e == cudaSuccess) {
         // the operand images as a 3-D array of floats: 64 per image row (256 B), 256 image rows per
         // tile, nmt_max tiles per point, npts points; one box = one tile (64 KB)
-        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)npts * nsplit};
+        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)npts};
         const cuuint64_t strides[2] = {256, (cuuint64_t)nmt_max * TILE_BYTES};
         const cuuint32_t box[3] = {64, 256, 1};
         const cuuint32_t estr[3] = {1, 1, 1};
@@ -841,7 +850,7 @@ int launch_band_lu_tc_batch(const std::vector<PointDesc>& items_in, cudaStream_t
     int* err = nullptr;
     PointDesc* pd = nullptr;
     NEP_CUDA(cudaMallocAsync((void**)&win, sizeof(zf) * win_elems, st));
-    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * count * nsplit, st);
+    cudaError_t e = cudaMallocAsync((void**)&aimg, (size_t)TILE_BYTES * nmt_max * count, st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&err, sizeof(int), st);
     if (e == cudaSuccess) e = cudaMallocAsync((void**)&pd, sizeof(PointDesc) * count, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(err, 0, sizeof(int), st);
@@ -853,7 +862,7 @@ int launch_band_lu_tc_batch(const std::vector<PointDesc>& items_in, cudaStream_t
     if (e == cudaSuccess) e = cudaMemcpyAsync(pd, items.data(), sizeof(PointDesc) * count, cudaMemcpyHostToDevice, st);
     CUtensorMap tmap;
     if (e == cudaSuccess) {
-        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)count * nsplit};
+        const cuuint64_t dims[3] = {64, (cuuint64_t)nmt_max * 256, (cuuint64_t)count};
         const cuuint64_t strides[2] = {256, (cuuint64_t)nmt_max * TILE_BYTES};
         const cuuint32_t box[3] = {64, 256, 1};
         const cuuint32_t estr[3] = {1, 1, 1};
