@@ -4,8 +4,8 @@
 // T(z_j) is applied on the union sparsity pattern with the FP64 values the assembly kernel
 // produced (the split sum sum_i f_i(z_j) A_i of Sec. 2 Eq. (split), evaluated once per point);
 // this is the residual r = sum_i f_i(lambda) A_i x of Sec. 5 (one SpMV per term in the
-// paper's implementation, one fused pass here). One CTA handles 256 rows of one
-// (point, right-hand side) pair so that the infinity norms of R, Y and V it produces reduce
+// paper's implementation, one fused pass here). One CTA handles 256 rows of one to four
+// right-hand sides of a point, so that the infinity norms of R, Y and V it produces reduce
 // inside the CTA to one atomic maximum each.
 //
 // Refinement sweep per point (all points in one launch each, points that have converged
@@ -35,46 +35,99 @@ __device__ __forceinline__ double block_max(double v, double* red) {
     return v;
 }
 
+// Bits of a maximum's candidate: values that are not below 0 order like their bits; NaN counts as none.
+__device__ __forceinline__ unsigned long long max_bits(double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    return b > 0x7ff0000000000000ull ? 0ull : b;
+}
+__device__ __forceinline__ unsigned max_bits(float v) {
+    const unsigned b = __float_as_uint(v);
+    return b > 0x7f800000u ? 0u : b;
+}
+__device__ __forceinline__ unsigned long long warp_max_bits(unsigned long long b) {
+    for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+    return b;
+}
+__device__ __forceinline__ unsigned warp_max_bits(unsigned b) { return __reduce_max_sync(0xffffffffu, b); }
+
+// Bits of the maxima over the CTA of Q values a thread: thread q < Q returns the q-th. red holds 8 Q.
+template <int Q, typename T, typename B>
+__device__ __forceinline__ B block_maxima(const T (&v)[Q], B* red) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const B b = warp_max_bits(max_bits(v[q]));
+        if (lane == 0) red[w * Q + q] = b;
+    }
+    __syncthreads();
+    B b = 0;
+    if (threadIdx.x < Q)
+        for (int u = 0; u < (int)(blockDim.x >> 5); ++u) b = max(b, red[u * Q + threadIdx.x]);
+    return b;
+}
+
+// RL right-hand sides of a point per thread: the pattern, T's values and their loads are shared.
 // nrm[(j*L + l)*3 + {0,1,2}] = max |R|, max |Y|, max |V| of column l of point j.
+template <int RL>
 __global__ void __launch_bounds__(256) split_residual_kernel(const int64_t* __restrict__ rowptr,
                                                              const int32_t* __restrict__ col, int64_t nnz, int n,
                                                              int L, const zd* __restrict__ tval,
                                                              const zd* __restrict__ V, const zd* __restrict__ Y,
                                                              zd* __restrict__ R, double* __restrict__ nrm,
                                                              const int* __restrict__ active) {
-    __shared__ double red[32];
-    const int jl = blockIdx.y;
-    const int j = jl / L, l = jl % L;
+    __shared__ unsigned long long red[24 * RL];
+    const int groups = (L + RL - 1) / RL;
+    const int j = blockIdx.y / groups, l0 = (blockIdx.y - j * groups) * RL, nl = min(RL, L - l0);
     if (active && !active[j]) return;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    const zd* y = Y + (int64_t)jl * n;
+    const zd* y = Y + ((int64_t)j * L + l0) * n;
     const zd* tv = tval + (int64_t)j * nnz;
-    double mr = 0.0, my = 0.0, mv = 0.0;
+    double m[3 * RL];
+#pragma unroll
+    for (int q = 0; q < 3 * RL; ++q) m[q] = 0.0;
     if (r < n) {
-        const zd v = V[(int64_t)l * n + r];
-        zd acc = v;
-        for (int64_t e = rowptr[r]; e < rowptr[r + 1]; ++e) acc = fms(acc, tv[e], y[col[e]]);
-        R[(int64_t)jl * n + r] = acc;
-        // squared moduli: the maxima are taken first and rooted once (FP64 issue is scarce)
-        mr = norm2(acc);
-        my = norm2(y[r]);
-        mv = norm2(v);
+        zd acc[RL];
+#pragma unroll
+        for (int q = 0; q < RL; ++q) acc[q] = q < nl ? V[(int64_t)(l0 + q) * n + r] : mk(0.0, 0.0);
+        if (nrm)  // squared moduli: the maxima are taken first and rooted once (FP64 issue is scarce)
+#pragma unroll
+            for (int q = 0; q < RL; ++q)
+                if (q < nl) m[3 * q + 1] = norm2(y[(int64_t)q * n + r]), m[3 * q + 2] = norm2(acc[q]);
+        for (int64_t e = rowptr[r]; e < rowptr[r + 1]; ++e) {
+            const zd t = tv[e];
+            const zd* ye = y + col[e];
+#pragma unroll
+            for (int q = 0; q < RL; ++q)
+                if (q < nl) acc[q] = fms(acc[q], t, ye[(int64_t)q * n]);
+        }
+#pragma unroll
+        for (int q = 0; q < RL; ++q)
+            if (q < nl) {
+                R[((int64_t)j * L + l0 + q) * n + r] = acc[q];
+                if (nrm) m[3 * q] = norm2(acc[q]);
+            }
     }
     if (!nrm) return;
-    mr = block_max(mr, red);
-    if (threadIdx.x == 0) atomic_max_nonneg_d(nrm + (int64_t)jl * 3 + 0, sqrt(mr));
-    my = block_max(my, red);
-    if (threadIdx.x == 0) atomic_max_nonneg_d(nrm + (int64_t)jl * 3 + 1, sqrt(my));
-    mv = block_max(mv, red);
-    if (threadIdx.x == 0) atomic_max_nonneg_d(nrm + (int64_t)jl * 3 + 2, sqrt(mv));
+    const double top = __longlong_as_double((long long)block_maxima<3 * RL>(m, red));
+    if (threadIdx.x < 3 * nl) atomic_max_nonneg_d(nrm + ((int64_t)j * L + l0) * 3 + threadIdx.x, sqrt(top));
+}
+
+// Right-hand sides per thread of the residual kernels: four where the blocks still fill the device.
+// n = 16384, five-point, 128 points x 32, double-float: 1.28 ms with one (T's values read 32 times a point
+// through L2), 0.68 with four; FP64 residual of 128 points x 16 with its assembly: 3.42 -> 1.23 ms, then
+// bound by the FP64 units.
+static int residual_rl(int n, int npts, int L) {
+    return L >= 4 && (int64_t)ceil_div(n, 256) * npts * ((L + 3) / 4) >= 608 ? 4 : 1;
 }
 
 int launch_split_residual(const SplitDev& s, int npts, const zd* tval, int L, const zd* V, const zd* Y, zd* R,
                           double* nrm, const int* active, cudaStream_t st) {
     if (npts <= 0 || L <= 0) return NEP_OK;
     if (nrm) NEP_CUDA(cudaMemsetAsync(nrm, 0, sizeof(double) * 3 * npts * L, st));
-    dim3 grid(ceil_div(s.n, 256), npts * L);
-    split_residual_kernel<<<grid, 256, 0, st>>>(s.rowptr, s.col, s.nnz, s.n, L, tval, V, Y, R, nrm, active);
+    const int rl = residual_rl(s.n, npts, L);
+    dim3 grid(ceil_div(s.n, 256), npts * ((L + rl - 1) / rl));
+    if (rl == 4) split_residual_kernel<4><<<grid, 256, 0, st>>>(s.rowptr, s.col, s.nnz, s.n, L, tval, V, Y, R, nrm, active);
+    else split_residual_kernel<1><<<grid, 256, 0, st>>>(s.rowptr, s.col, s.nnz, s.n, L, tval, V, Y, R, nrm, active);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
 }
@@ -276,43 +329,55 @@ __global__ void widen_df_kernel(int64_t total, const zf* __restrict__ B, zdf* __
 
 // D_j = V - T(z_j) Y_j rounded to complex64 (the next correction's right-hand side), and the maxima
 // of |R|, |Y|, |V| per (point, column) as split_residual_kernel gives them
+template <int RL>
 __global__ void __launch_bounds__(256) split_residual_df_kernel(const int64_t* __restrict__ rowptr,
                                                                 const int32_t* __restrict__ col, int64_t nnz, int n,
                                                                 int L, const zdf* __restrict__ tval,
                                                                 const zdf* __restrict__ V, const zdf* __restrict__ Y,
                                                                 zf* __restrict__ D, double* __restrict__ nrm,
                                                                 const int* __restrict__ active) {
-    __shared__ float red[32];
-    const int jl = blockIdx.y;
-    const int j = jl / L, l = jl % L;
+    __shared__ unsigned red[24 * RL];
+    const int groups = (L + RL - 1) / RL;
+    const int j = blockIdx.y / groups, l0 = (blockIdx.y - j * groups) * RL, nl = min(RL, L - l0);
     if (active && !active[j]) return;
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    const zdf* y = Y + (int64_t)jl * n;
+    const zdf* y = Y + ((int64_t)j * L + l0) * n;
     const zdf* tv = tval + (int64_t)j * nnz;
-    float mr = 0.0f, my = 0.0f, mv = 0.0f;
+    float m[3 * RL];
+#pragma unroll
+    for (int q = 0; q < 3 * RL; ++q) m[q] = 0.0f;
     if (r < n) {
-        const zdf v = V[(int64_t)l * n + r];
-        float rh = v.hr, rl = v.lr, ih = v.hi, il = v.li;
-        for (int64_t e = rowptr[r]; e < rowptr[r + 1]; ++e) {
-            const zdf t = tv[e], x = y[col[e]];
-            df_fms(rh, rl, t.hr, t.lr, x.hr, x.lr);    // re -= t.re x.re
-            df_fms(rh, rl, -t.hi, -t.li, x.hi, x.li);  // re += t.im x.im
-            df_fms(ih, il, t.hr, t.lr, x.hi, x.li);    // im -= t.re x.im
-            df_fms(ih, il, t.hi, t.li, x.hr, x.lr);    // im -= t.im x.re
+        zdf acc[RL];
+#pragma unroll
+        for (int q = 0; q < RL; ++q) {
+            acc[q] = q < nl ? V[(int64_t)(l0 + q) * n + r] : zdf{0.0f, 0.0f, 0.0f, 0.0f};
+            if (q < nl) m[3 * q + 2] = hypotf(acc[q].hr, acc[q].hi);
         }
-        D[(int64_t)jl * n + r] = mk(rh + rl, ih + il);
-        const zdf yr = y[r];
-        mr = hypotf(rh, ih);
-        my = hypotf(yr.hr, yr.hi);
-        mv = hypotf(v.hr, v.hi);
+        for (int64_t e = rowptr[r]; e < rowptr[r + 1]; ++e) {
+            const zdf t = tv[e];
+            const zdf* ye = y + col[e];
+#pragma unroll
+            for (int q = 0; q < RL; ++q)
+                if (q < nl) {
+                    const zdf x = ye[(int64_t)q * n];
+                    df_fms(acc[q].hr, acc[q].lr, t.hr, t.lr, x.hr, x.lr);    // re -= t.re x.re
+                    df_fms(acc[q].hr, acc[q].lr, -t.hi, -t.li, x.hi, x.li);  // re += t.im x.im
+                    df_fms(acc[q].hi, acc[q].li, t.hr, t.lr, x.hi, x.li);    // im -= t.re x.im
+                    df_fms(acc[q].hi, acc[q].li, t.hi, t.li, x.hr, x.lr);    // im -= t.im x.re
+                }
+        }
+#pragma unroll
+        for (int q = 0; q < RL; ++q)
+            if (q < nl) {
+                D[((int64_t)j * L + l0 + q) * n + r] = mk(acc[q].hr + acc[q].lr, acc[q].hi + acc[q].li);
+                const zdf yr = y[(int64_t)q * n + r];
+                m[3 * q] = hypotf(acc[q].hr, acc[q].hi);
+                m[3 * q + 1] = hypotf(yr.hr, yr.hi);
+            }
     }
     if (!nrm) return;
-    mr = block_max_f(mr, red);
-    if (threadIdx.x == 0) atomic_max_nonneg_d(nrm + (int64_t)jl * 3 + 0, (double)mr);
-    my = block_max_f(my, red);
-    if (threadIdx.x == 0) atomic_max_nonneg_d(nrm + (int64_t)jl * 3 + 1, (double)my);
-    mv = block_max_f(mv, red);
-    if (threadIdx.x == 0) atomic_max_nonneg_d(nrm + (int64_t)jl * 3 + 2, (double)mv);
+    const float top = __uint_as_float(block_maxima<3 * RL>(m, red));
+    if (threadIdx.x < 3 * nl) atomic_max_nonneg_d(nrm + ((int64_t)j * L + l0) * 3 + threadIdx.x, (double)top);
 }
 
 // Y += D in double-float; dmax[j] = max |D|, ymax[j] = max |Y| over the point's block
@@ -364,8 +429,10 @@ int launch_split_residual_df(const SplitDev& s, int npts, const zdf* tval, int L
                              double* nrm, const int* active, cudaStream_t st) {
     if (npts <= 0 || L <= 0) return NEP_OK;
     if (nrm) NEP_CUDA(cudaMemsetAsync(nrm, 0, sizeof(double) * 3 * npts * L, st));
-    dim3 grid(ceil_div(s.n, 256), npts * L);
-    split_residual_df_kernel<<<grid, 256, 0, st>>>(s.rowptr, s.col, s.nnz, s.n, L, tval, V, Y, D, nrm, active);
+    const int rl = residual_rl(s.n, npts, L);
+    dim3 grid(ceil_div(s.n, 256), npts * ((L + rl - 1) / rl));
+    if (rl == 4) split_residual_df_kernel<4><<<grid, 256, 0, st>>>(s.rowptr, s.col, s.nnz, s.n, L, tval, V, Y, D, nrm, active);
+    else split_residual_df_kernel<1><<<grid, 256, 0, st>>>(s.rowptr, s.col, s.nnz, s.n, L, tval, V, Y, D, nrm, active);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
 }
