@@ -10,6 +10,21 @@
 
 namespace nep {
 
+// Launch shape of a sweep for window width W: RPL = registers per lane, RS = 32 RPL > W, or for widths of
+// exactly 64, 96 and 128 and two or more right-hand sides a warp kFullWindow + W / 32: RS = W, the entering
+// row taking its slot ahead of the step's update. That saves a register a lane and its staged coefficients
+// where the sweep is bound by issue (bandwidth 64, 128 points x 32: 1.66 -> 1.44 ms a solve; bandwidth 128,
+// 128 x 16: 5.06 -> 4.83). With one right-hand side a warp the chain bounds the sweep and the
+// extra select costs 4 %.
+constexpr int kFullWindow = 16;
+template <typename T>
+inline int sweep_shape(int W, int rh) {
+    return sizeof(T) == 4 && rh >= 2 && W >= 64 && W <= 128 && W % 32 == 0 ? kFullWindow + W / 32 : W / 32 + 1;
+}
+__host__ __device__ inline bool sweep_covers(int shape, int W) {
+    return shape > kFullWindow ? W == 32 * (shape - kFullWindow) : W < 32 * shape;
+}
+
 // One substitution sweep (forward with L and the row interchanges, or backward with U) for
 // narrow bands; each warp carries RH right-hand sides. Step k handles row c = k (forward) or
 // c = n-1-k (backward); the row with step index k' lives in window slot s = k' mod RS,
@@ -17,7 +32,7 @@ namespace nep {
 // through the registers in a fixed order, so with the step loop unrolled by RPL every
 // register index is a compile-time constant. The row leaving the window at step k (row c
 // itself) is replaced in the same register by the row with step index k + RS, which needs
-// its first update only later (RS > window width).
+// its first update only later (RS > window width), or at once where RS is the window width.
 //
 // The coefficients of step k form one contiguous column col(k)[d], d in [1, W]:
 //   forward  (W = kl):    col(k)[d] = ab[c*ldab + kv + d] = L(c+d, c)
@@ -35,12 +50,12 @@ namespace nep {
 // while the compute warps (one or more right-hand sides each) run chunk c, so the staging's index
 // work and copy issue stay off the compute warps' dependency chains. One CTA barrier per chunk:
 // each producer arrives once its copies have landed, the compute warps once the chunk is done.
-template <typename T, int RPL, bool BWD, int RH>
+template <typename T, int RPL, bool BWD, int RH, bool FULL>
 __global__ void __launch_bounds__(256)
     band_sweep_kernel(int n, int kl, int ku, int ldab, const cx<T>* __restrict__ ab_all,
                       const cx<T>* __restrict__ ut_all, const int* __restrict__ ipiv_all, int L,
                       cx<T>* __restrict__ B_all, const int* __restrict__ active, int CH,
-                      const PointDesc* __restrict__ pd, int rpl_done) {
+                      const PointDesc* __restrict__ pd, int done) {
     int j = blockIdx.x;
     if (pd) {  // a point of one of several problems sharing the launch (the grid covers the largest L)
         const PointDesc d = pd[blockIdx.x];
@@ -62,10 +77,9 @@ __global__ void __launch_bounds__(256)
     const cx<T>* colbase = BWD ? ut_all + (int64_t)j * n * (kv + 1) : ab_all + (int64_t)j * n * ldab + kv;
     const int* ipiv = ipiv_all + (int64_t)j * n;
     // Window width: rows updated per step. Backward it is what this point's U can reach (ku without
-    // interchanges); the points that need no more than rpl_done registers a lane belong to another
-    // launch of the sweep, those that need more than RPL to a third.
+    // interchanges); the points whose width another launch of the sweep has covered (done) are not this one's.
     const int W = BWD ? u_reach(n, ku, ipiv) : kl;
-    if (BWD && (W >= RS || W < 32 * rpl_done)) return;
+    if (BWD && (!sweep_covers(FULL ? RPL + kFullWindow : RPL, W) || (done > 0 && sweep_covers(done, W)))) return;
     bool has[RH];
     cx<T>* bh[RH];
 #pragma unroll
@@ -147,9 +161,14 @@ __global__ void __launch_bounds__(256)
                     cx<T> x[RH];
 #pragma unroll
                     for (int h = 0; h < RH; ++h) x[h] = shfl_cx(a[h][u], lane_k);
+                    bool entered = false;  // the entering row has become row c, its slot holds the old row c
                     if constexpr (SWAPS) {
                         const int p = pv[cc] - (k0 + cc);
-                        if (p != 0) {
+                        if (FULL && p == RS) {
+                            entered = true;
+#pragma unroll
+                            for (int h = 0; h < RH; ++h) x[h] = nb[h * CH + cc];
+                        } else if (p != 0) {
                             // interchange rows c and c+p: slot of c+p is (lane_k*RPL + u + p) mod RS
                             int sp = lane_k * RPL + u + p;
                             if (sp >= RS) sp -= RS;
@@ -167,6 +186,10 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
                         for (int h = 0; h < RH; ++h) x[h] = x[h] * rd;
                     }
+                    if (FULL && !entered && lane == lane_k) {  // the entering row takes this step's update too
+#pragma unroll
+                        for (int h = 0; h < RH; ++h) a[h][u] = nb[h * CH + cc];
+                    }
                     const cx<T>* c1 = cf + (int64_t)cc * RSP;
 #pragma unroll
                     for (int q = 0; q < RPL; ++q) {
@@ -174,7 +197,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
                         for (int h = 0; h < RH; ++h) a[h][q] = fms(a[h][q], cq, x[h]);
                     }
-                    if (lane == lane_k) {
+                    if (!FULL && lane == lane_k) {
 #pragma unroll
                         for (int h = 0; h < RH; ++h) a[h][u] = nb[h * CH + cc];
                     }
@@ -238,9 +261,9 @@ __global__ void band_transpose_u_kernel(int n, int kv, int ldab, const cx<T>* __
     }
 }
 
-template <typename T, int RPL, bool BWD, int RH>
+template <typename T, int RPL, bool BWD, int RH, bool FULL = false>
 static int run_sweep(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, const int* ipiv, int L,
-                     cx<T>* B, const int* active, cudaStream_t st, int rpl_done) {
+                     cx<T>* B, const int* active, cudaStream_t st, int done) {
     constexpr int RSP = 32 * (RPL | 1) + 1;
     const int warps = (L + RH - 1) / RH;
     // four compute warps per CTA (those beyond the right-hand sides idle), and as many producer
@@ -256,17 +279,17 @@ static int run_sweep(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* 
     while (CH > RPL && bytes(CH) > 200 * 1024) CH -= RPL;
     const size_t smem = bytes(CH);
     if (smem > 227 * 1024) return NEP_ERR_UNSUPPORTED;
-    NEP_CUDA(allow_max_dynamic_smem(band_sweep_kernel<T, RPL, BWD, RH>));
-    band_sweep_kernel<T, RPL, BWD, RH><<<dim3(npts, gy), 2 * wpb * 32, smem, st>>>(s.n, s.kl, s.ku, s.ldab, ab, ut,
-                                                                             ipiv, L, B, active, CH, nullptr, rpl_done);
+    NEP_CUDA(allow_max_dynamic_smem(band_sweep_kernel<T, RPL, BWD, RH, FULL>));
+    band_sweep_kernel<T, RPL, BWD, RH, FULL><<<dim3(npts, gy), 2 * wpb * 32, smem, st>>>(s.n, s.kl, s.ku, s.ldab, ab, ut,
+                                                                             ipiv, L, B, active, CH, nullptr, done);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
 }
 
 // The same sweep over points of several problems (descriptors pd_dev[count]; maxL the most
 // right-hand sides of any of them): the launch shape of run_sweep, per-point arithmetic unchanged.
-template <typename T, int RPL, bool BWD, int RH>
-static int run_sweep_batch(int count, int maxL, const PointDesc* pd_dev, cudaStream_t st, int rpl_done) {
+template <typename T, int RPL, bool BWD, int RH, bool FULL = false>
+static int run_sweep_batch(int count, int maxL, const PointDesc* pd_dev, cudaStream_t st, int done) {
     constexpr int RSP = 32 * (RPL | 1) + 1;
     const int warps = (maxL + RH - 1) / RH;
     const int wpb = 4;
@@ -279,10 +302,10 @@ static int run_sweep_batch(int count, int maxL, const PointDesc* pd_dev, cudaStr
     while (CH > RPL && bytes(CH) > 200 * 1024) CH -= RPL;
     const size_t smem = bytes(CH);
     if (smem > 227 * 1024) return NEP_ERR_UNSUPPORTED;
-    NEP_CUDA(allow_max_dynamic_smem(band_sweep_kernel<T, RPL, BWD, RH>));
-    band_sweep_kernel<T, RPL, BWD, RH><<<dim3(count, gy), 2 * wpb * 32, smem, st>>>(0, 0, 0, 0, nullptr, nullptr,
+    NEP_CUDA(allow_max_dynamic_smem(band_sweep_kernel<T, RPL, BWD, RH, FULL>));
+    band_sweep_kernel<T, RPL, BWD, RH, FULL><<<dim3(count, gy), 2 * wpb * 32, smem, st>>>(0, 0, 0, 0, nullptr, nullptr,
                                                                               nullptr, maxL, nullptr, nullptr, CH,
-                                                                              pd_dev, rpl_done);
+                                                                              pd_dev, done);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
 }
@@ -300,6 +323,12 @@ static int sweep_batch_rpl(int rpl, int count, int maxL, const PointDesc* pd, cu
         case 8: return run_sweep_batch<T, 8, BWD, RH>(count, maxL, pd, st, done);
         case 9: return run_sweep_batch<T, 9, BWD, RH>(count, maxL, pd, st, done);
     }
+    if constexpr (sizeof(T) == 4 && RH >= 2)
+        switch (rpl) {
+            case kFullWindow + 2: return run_sweep_batch<T, 2, BWD, RH, true>(count, maxL, pd, st, done);
+            case kFullWindow + 3: return run_sweep_batch<T, 3, BWD, RH, true>(count, maxL, pd, st, done);
+            case kFullWindow + 4: return run_sweep_batch<T, 4, BWD, RH, true>(count, maxL, pd, st, done);
+        }
     return NEP_ERR_UNSUPPORTED;
 }
 
@@ -353,49 +382,49 @@ static int sweep_rpl(int rpl, const SplitDev& s, int npts, const cx<T>* ab, cons
         case 8: return run_sweep<T, 8, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
         case 9: return run_sweep<T, 9, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
     }
+    if constexpr (sizeof(T) == 4 && RH >= 2)
+        switch (rpl) {
+            case kFullWindow + 2: return run_sweep<T, 2, BWD, RH, true>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+            case kFullWindow + 3: return run_sweep<T, 3, BWD, RH, true>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+            case kFullWindow + 4: return run_sweep<T, 4, BWD, RH, true>(s, npts, ab, ut, ipiv, L, B, active, st, done);
+        }
     return NEP_ERR_UNSUPPORTED;
 }
 
 template <typename T, bool BWD>
 static int sweep_dispatch(int rpl, const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, const int* ipiv,
-                          int L, cx<T>* B, const int* active, cudaStream_t st, int rh_force, int done) {
-    switch (rh_force == 1 || rh_force == 2 || rh_force == 4 ? rh_force : sweep_rh<T>(npts * L)) {
+                          int L, cx<T>* B, const int* active, cudaStream_t st, int rh, int done) {
+    switch (rh) {
         case 1: return sweep_rpl<T, BWD, 1>(rpl, s, npts, ab, ut, ipiv, L, B, active, st, done);
         case 4: return sweep_rpl<T, BWD, 4>(rpl, s, npts, ab, ut, ipiv, L, B, active, st, done);
         default: return sweep_rpl<T, BWD, 2>(rpl, s, npts, ab, ut, ipiv, L, B, active, st, done);
     }
 }
 
-// The backward sweep runs in up to two launches: points whose U stayed within ku rounded up to whole
-// registers, then the rest (kl + ku registers; a point that has run returns at once). Without interchanges
+// The backward sweep runs in up to two launches: points whose U the shape for ku covers, then the rest
+// (kl + ku rows; a point that has run returns at once). Without interchanges
 // the first does all the work with about half the registers and staged coefficients. Solve, ms before ->
 // after: bandwidth 128, 128 points x 16: 7.13 -> 5.06; bandwidth 97, 64 x 32: 3.23 -> 2.85; bandwidth 64,
 // 128 x 32: 1.80 -> 1.66; the blocked kernel at bandwidth 576, 64 x 16: 13.6 -> 10.5.
-// Registers per lane of a sweep's window for window width W: RS = 32 RPL > W. (A variant with
-// RS = W, the entering row moved ahead of the step's update, executed fewer instructions on
-// bandwidth 64 but ran no faster: 0.349 + 0.506 ms per solve against 0.345 + 0.476; each step is
-// bound by its dependency chain rather than by issue.)
-inline int sweep_rpl_of(int W) { return (W + 1 + 31) / 32; }
-
-// Sweep launch shape of a problem: rows per lane of the forward window and of the backward one (without
-// interchanges and at most) and right-hand
-// sides per warp (from the problem's own chain count N L). Points of problems with equal keys share
+//
+// Sweep launch shapes of a problem, forward, backward and backward for points with more interchanges, and
+// right-hand sides per warp (from the problem's own chain count N L). Points of problems with equal keys share
 // batched launches.
 template <typename T>
-void sweep_key(int kl, int ku, int npts, int L, int* rplf, int* rplu, int* rplb, int* rh, int rh_force) {
-    *rplf = sweep_rpl_of(kl);
-    *rplu = sweep_rpl_of(ku);
-    *rplb = sweep_rpl_of(kl + ku);
+void sweep_key(int kl, int ku, int npts, int L, int* fwd, int* bwd, int* wide, int* rh, int rh_force) {
     *rh = rh_force == 1 || rh_force == 2 || rh_force == 4 ? rh_force : sweep_rh<T>(npts * L);
+    *fwd = sweep_shape<T>(kl, *rh);
+    *bwd = sweep_shape<T>(ku, *rh);
+    *wide = (kl + ku) / 32 + 1;
 }
 
 template <typename T>
-int band_sweeps_batch(int rplf, int rplu, int rplb, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st) {
+int band_sweeps_batch(int fwd, int bwd, int wide, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st) {
     if (count <= 0 || maxL <= 0) return NEP_OK;
-    int rc = sweep_batch_dispatch<T, false>(rplf, rh, count, maxL, pd, st, 0);
-    if (rc == NEP_OK && rplu < rplb) rc = sweep_batch_dispatch<T, true>(rplu, rh, count, maxL, pd, st, 0);
-    if (rc != NEP_OK) return rc;
-    return sweep_batch_dispatch<T, true>(rplb, rh, count, maxL, pd, st, rplu < rplb ? rplu : 0);
+    int rc = sweep_batch_dispatch<T, false>(fwd, rh, count, maxL, pd, st, 0);
+    if (rc == NEP_OK) rc = sweep_batch_dispatch<T, true>(bwd, rh, count, maxL, pd, st, 0);
+    if (rc != NEP_OK || bwd == wide) return rc;
+    return sweep_batch_dispatch<T, true>(wide, rh, count, maxL, pd, st, bwd);
 }
 
 template <typename T>
@@ -403,12 +432,13 @@ int band_sweeps(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, c
                 const int* active, cudaStream_t st, int rh_force) {
     if (npts <= 0 || L <= 0) return NEP_OK;
     if (!band_sweeps_fit(s.kl, s.ku) || !ut) return NEP_ERR_UNSUPPORTED;
-    const int rplf = sweep_rpl_of(s.kl), rplu = sweep_rpl_of(s.ku), rplb = sweep_rpl_of(s.kl + s.ku);
-    int rc = sweep_dispatch<T, false>(rplf, s, npts, ab, ut, ipiv, L, B, active, st, rh_force, 0);
-    // backward: points whose U the interchanges left within rplu registers a lane, then the others
-    if (rc == NEP_OK && rplu < rplb) rc = sweep_dispatch<T, true>(rplu, s, npts, ab, ut, ipiv, L, B, active, st, rh_force, 0);
-    if (rc != NEP_OK) return rc;
-    return sweep_dispatch<T, true>(rplb, s, npts, ab, ut, ipiv, L, B, active, st, rh_force, rplu < rplb ? rplu : 0);
+    int fwd, bwd, wide, rh;
+    sweep_key<T>(s.kl, s.ku, npts, L, &fwd, &bwd, &wide, &rh, rh_force);
+    int rc = sweep_dispatch<T, false>(fwd, s, npts, ab, ut, ipiv, L, B, active, st, rh, 0);
+    // backward: points whose U the interchanges left at ku, then the others
+    if (rc == NEP_OK) rc = sweep_dispatch<T, true>(bwd, s, npts, ab, ut, ipiv, L, B, active, st, rh, 0);
+    if (rc != NEP_OK || bwd == wide) return rc;
+    return sweep_dispatch<T, true>(wide, s, npts, ab, ut, ipiv, L, B, active, st, rh, bwd);
 }
 
 template <typename T>

@@ -266,9 +266,9 @@ template <typename T>
 int launch_band_lu_col_batch(int instance, int count, const PointDesc* pd_dev, cudaStream_t st);
 // the narrow-band sweeps' launch shape of a problem, and the sweeps over points of equal shape
 template <typename T>
-void sweep_key(int kl, int ku, int npts, int L, int* rplf, int* rplu, int* rplb, int* rh, int rh_force = 0);
+void sweep_key(int kl, int ku, int npts, int L, int* fwd, int* bwd, int* wide, int* rh, int rh_force = 0);
 template <typename T>
-int band_sweeps_batch(int rplf, int rplu, int rplb, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st);
+int band_sweeps_batch(int fwd, int bwd, int wide, int rh, int count, int maxL, const PointDesc* pd, cudaStream_t st);
 // the tensor-core LU over points of several complex64 problems (each kl > 64)
 int launch_band_lu_tc_batch(const std::vector<PointDesc>& items, cudaStream_t st, int passes = 3);
 
