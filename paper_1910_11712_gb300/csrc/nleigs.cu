@@ -470,8 +470,11 @@ __global__ void nleigs_combine_kernel(int n, int d, const zd* __restrict__ u, zd
 }
 
 // h = sqrt(Re nr); H sub-diagonal entry (or hlast) = h; w /= h (w = 0 after a breakdown)
-__global__ void nleigs_scale_kernel(int64_t N, zd* __restrict__ w, const zd* __restrict__ nr, zd* __restrict__ hsub) {
-    const double h = sqrt(fmax(nr->re, 0.0));
+__global__ void nleigs_scale_kernel(int64_t N, zd* __restrict__ w, int nch, const zd* __restrict__ nr,
+                                    zd* __restrict__ hsub) {
+    double sq = 0.0;  // Re of the total of nr's nch partial sums, in their order
+    for (int c = 0; c < nch; ++c) sq += nr[c].re;
+    const double h = sqrt(fmax(sq, 0.0));
     const double sc = h > 1e-300 ? 1.0 / h : 0.0;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < N) w[t] = sc * w[t];
@@ -747,6 +750,7 @@ __global__ void __launch_bounds__(256) nleigs_dots_kernel(int64_t N, int64_t chu
     const int64_t r0 = (int64_t)c * chunk, r1 = min(N, r0 + chunk);
     const zd* v = V + (int64_t)j * N;
     zd acc = mk(0.0, 0.0);
+#pragma unroll 4
     for (int64_t r = r0 + threadIdx.x; r < r1; r += blockDim.x) acc = fmac(acc, v[r], w[r]);
     for (int o = 16; o > 0; o >>= 1) {
         acc.re += __shfl_xor_sync(0xffffffffu, acc.re, o);
@@ -771,22 +775,51 @@ __global__ void nleigs_dots_reduce_kernel(int nchunks, int K, const zd* __restri
     h[j] = t;
 }
 
-// w[r] -= sum_{j<K} V[r + N j] h[j]; Hcol[j] += h[j] (block 0)
-__global__ void __launch_bounds__(256) nleigs_sub_kernel(int64_t N, int K, const zd* __restrict__ V,
-                                                         const zd* __restrict__ h, zd* __restrict__ w,
-                                                         zd* __restrict__ Hcol) {
+// The sums of a dot product, given as nch partial sums (1: the sum itself), in their fixed order.
+__device__ __forceinline__ zd nleigs_total(int nch, const zd* __restrict__ part) {
+    zd t = mk(0.0, 0.0);
+    for (int c = 0; c < nch; ++c) t = t + part[c];
+    return t;
+}
+
+// w[r] -= sum_{j<K} V[r + N j] h[j], h[j] = the total of part[.. + nch j]; Hcol[j] += h[j] (block 0).
+// 64 rows a block, the columns in four shares of eight loads in flight: at N = 4096 blocks of 256 rows filled
+// 16 SMs, each thread waiting for one or two loads at a time (29 us a call at K = 70; 18 with blocks of 64 and
+// eight loads, 9 in shares).
+constexpr int kSubRows = 64, kSubShares = 4;
+__global__ void __launch_bounds__(kSubRows * kSubShares)
+    nleigs_sub_kernel(int64_t N, int K, const zd* __restrict__ V, int nch, const zd* __restrict__ part,
+                      zd* __restrict__ w, zd* __restrict__ Hcol) {
     extern __shared__ zd hs[];
-    for (int j = threadIdx.x; j < K; j += blockDim.x) hs[j] = h[j];
+    __shared__ zd sums[kSubShares - 1][kSubRows];
+    for (int j = threadIdx.x; j < K; j += blockDim.x) hs[j] = nleigs_total(nch, part + (int64_t)nch * j);
     __syncthreads();
     if (blockIdx.x == 0 && Hcol)
         for (int j = threadIdx.x; j < K; j += blockDim.x) Hcol[j] = Hcol[j] + hs[j];
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= N) return;
-    zd acc = w[r];
-    for (int j = 0; j < K; ++j) acc = fms(acc, V[r + (int64_t)j * N], hs[j]);
-    w[r] = acc;
+    const int row = threadIdx.x % kSubRows, share = threadIdx.x / kSubRows;
+    const int64_t r = (int64_t)blockIdx.x * kSubRows + row;
+    const int per = (K + kSubShares - 1) / kSubShares, j1 = min(K, (share + 1) * per);
+    zd acc = mk(0.0, 0.0);
+    if (r < N) {
+        int j = share * per;
+        const zd* v = V + r + j * N;
+        for (; j + 8 <= j1; j += 8, v += 8 * N) {
+            zd x[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = v[q * N];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) acc = fma_(acc, x[q], hs[j + q]);
+        }
+        for (; j < j1; ++j, v += N) acc = fma_(acc, *v, hs[j]);
+    }
+    if (share > 0) sums[share - 1][row] = acc;
+    __syncthreads();
+    if (share == 0 && r < N) {
+#pragma unroll
+        for (int q = 0; q < kSubShares - 1; ++q) acc = acc + sums[q][row];
+        w[r] = w[r] - acc;
+    }
 }
-
 
 // ---- the compact (TOAR) basis of Sec. 4.5.3: Krylov vectors (I_d (x) U) g with U (n x m) orthonormal,
 // growing by one column per step, and coefficient blocks g^i in C^m. Coefficient vectors are stored
@@ -796,31 +829,42 @@ __global__ void __launch_bounds__(256) nleigs_sub_kernel(int64_t N, int K, const
 // (j = d-1 .. 1: the recurrence of nleigs_expand_kernel, acting on U's coordinates), and the per-term
 // combinations Cc[t Mx + q] = sum_{j<=d-2} ddc[t, j] pt^j_q + ddc[t, d] g^{d-1}_q, whose images U Cc_t
 // enter the split SpMV of Eq. (nleigs-toar2). One thread per coordinate q < m.
-__global__ void toar_coef_kernel(int d, int m, int Mx, int nt, const zd* __restrict__ g, zd* __restrict__ pt,
-                                 zd* __restrict__ Cc, const ExpandCoef* __restrict__ ec,
-                                 const zd* __restrict__ ddc) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= m) return;
-    zd acc[kNleigsMaxTerms];
-    zd gj = g[(int64_t)(d - 1) * Mx + q];
-#pragma unroll
-    for (int i = 0; i < kNleigsMaxTerms; ++i) acc[i] = i < nt ? ddc[i + (int64_t)nt * d] * gj : mk(0.0, 0.0);
-    pt[(int64_t)(d - 1) * Mx + q] = mk(0.0, 0.0);
-    zd pj = mk(0.0, 0.0);
-    for (int j = d - 1; j >= 1; --j) {
-        const zd gjm = g[(int64_t)(j - 1) * Mx + q];
-        const zd z = fma_(gjm, ec->g[j], gj);
-        const zd pv = (z - ec->e[j] * pj) * ec->inv_ds[j];
-        pt[(int64_t)(j - 1) * Mx + q] = pv;
-#pragma unroll
-        for (int i = 0; i < kNleigsMaxTerms; ++i)
-            if (i < nt) acc[i] = fma_(acc[i], ddc[i + (int64_t)nt * (j - 1)], pv);
-        pj = pv;
-        gj = gjm;
+// A block takes 32 coordinates. The recurrence is a chain over j whose FP64 instructions each hold a quarter of
+// the SM's FP64 unit for 64 cycles, so only one multiply-add per step stays in it,
+// pt^{j-1} = z_j inv_ds_j - (e_j inv_ds_j) pt^j with z_j = g^{j-1} + g_j g^j; the four warps form the z_j before
+// and the terms' sums after. d = 64: 53 us a call with one thread per coordinate and all of it in the chain,
+// 14 us now.
+constexpr int kToarWarps = 4;
+__global__ void __launch_bounds__(32 * kToarWarps)
+    toar_coef_kernel(int d, int m, int Mx, int nt, const zd* __restrict__ g, zd* __restrict__ pt,
+                     zd* __restrict__ Cc, const ExpandCoef* __restrict__ ec, const zd* __restrict__ ddc) {
+    extern __shared__ zd tab[];  // e inv_ds (d), ddc (nt x (d + 1)), then z inv_ds, later pt (d x 32)
+    zd *te = tab, *td = te + d, *p = td + nt * (d + 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int q = blockIdx.x * 32 + lane, qc = min(q, m - 1);
+    for (int j = threadIdx.x; j < d; j += blockDim.x) te[j] = j > 0 ? ec->e[j] * ec->inv_ds[j] : mk(0.0, 0.0);
+    for (int j = threadIdx.x; j < nt * (d + 1); j += blockDim.x) td[j] = ddc[j];
+#pragma unroll 4
+    for (int j = 1 + warp; j < d; j += kToarWarps)
+        p[(j - 1) * 32 + lane] = fma_(g[(int64_t)(j - 1) * Mx + qc], ec->g[j], g[(int64_t)j * Mx + qc]) * ec->inv_ds[j];
+    __syncthreads();
+    if (warp == 0) {
+        zd pj = mk(0.0, 0.0);
+        p[(d - 1) * 32 + lane] = pj;
+#pragma unroll 4
+        for (int j = d - 1; j >= 1; --j) {
+            pj = fms(p[(j - 1) * 32 + lane], te[j], pj);
+            p[(j - 1) * 32 + lane] = pj;
+        }
     }
-#pragma unroll
-    for (int i = 0; i < kNleigsMaxTerms; ++i)
-        if (i < nt) Cc[(int64_t)i * Mx + q] = acc[i];
+    __syncthreads();
+    if (q >= m) return;
+    for (int j = warp; j < d; j += kToarWarps) pt[(int64_t)j * Mx + q] = p[j * 32 + lane];
+    for (int i = warp; i < nt; i += kToarWarps) {
+        zd acc = td[i + nt * d] * g[(int64_t)(d - 1) * Mx + q];
+        for (int j = d - 1; j >= 1; --j) acc = fma_(acc, td[i + nt * (j - 1)], p[(j - 1) * 32 + lane]);
+        Cc[(int64_t)i * Mx + q] = acc;
+    }
 }
 
 // Eq. (nleigs-toar4): the coefficients of S v in the (possibly extended) basis,
@@ -953,8 +997,10 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
     double *tnorm = nullptr, *dmax = nullptr, *ymax = nullptr;
     int *ipiv = nullptr, *info = nullptr;
     const int kv = s.kl + s.ku;
-    const int64_t chunk = 4096;
-    const int nchunks = (int)((N + chunk - 1) / chunk);
+    // rows per block of a dot product: short vectors in more blocks; their few partial sums (kDirectSums at
+    // most) are added up by the kernels that use them, longer ones by a kernel of their own
+    auto chunk_of = [](int64_t len) -> int64_t { return len <= 16384 ? 1024 : 4096; };
+    constexpr int kDirectSums = 16;
     NEP_TRY(w.get(&d_ec, 1));
     NEP_TRY(w.get(&d_ddc, (size_t)nt * (d + 1)));
     NEP_TRY(w.get(&d_F, (size_t)nt));
@@ -976,7 +1022,8 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
     NEP_TRY(w.get(&Hf, (size_t)ldh * kmax));
     NEP_TRY(w.get(&hv, (size_t)kmax + 1));
     NEP_TRY(w.get(&nr, 1));
-    NEP_TRY(w.get(&part, (size_t)std::max<int64_t>(nchunks, ((int64_t)d * (d + kmax) + chunk - 1) / chunk) * (kmax + 1)));
+    auto chunks = [&](int64_t len) { return (size_t)((len + chunk_of(len) - 1) / chunk_of(len)); };
+    NEP_TRY(w.get(&part, std::max(chunks(N), chunks((int64_t)d * (d + kmax))) * (kmax + 1)));
     NEP_CUDA(cudaMemcpyAsync(d_ec, &ec, sizeof(ec), cudaMemcpyHostToDevice, st));
     NEP_CUDA(cudaMemcpyAsync(d_ddc, ddc.data(), sizeof(zd) * ddc.size(), cudaMemcpyHostToDevice, st));
     NEP_CUDA(cudaMemcpyAsync(d_F, Fs.data(), sizeof(zd) * nt, cudaMemcpyHostToDevice, st));
@@ -985,11 +1032,47 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
     NEP_TRY(launch_assemble<float>(s, 1, d_F, ab, tnorm, tval, st));
     NEP_TRY(launch_band_lu<float>(s, 1, ab, ipiv, info, nullptr, st));
     if (ut) NEP_TRY(band_transpose_u<float>(s, 1, ab, ut, st));
-    // ||x||^2 or x^H y over N entries into out (K = 1)
-    auto dots = [&](const zd* Vb, int K, const zd* x, zd* out) -> int {
-        nleigs_dots_kernel<<<dim3(nchunks, K), 256, 0, st>>>(N, chunk, Vb, x, part);
+    // V_j^H x of K vectors over len entries, as sums that the kernels below finish (Sums::nch each), and as
+    // numbers in out
+    struct Sums {
+        int nch;
+        const zd* part;
+    };
+    auto dot_parts = [&](const zd* Vb, int K, const zd* x, int64_t len, zd* parts, int* nch) -> int {
+        const int64_t ch = chunk_of(len);
+        *nch = (int)((len + ch - 1) / ch);
+        nleigs_dots_kernel<<<dim3(*nch, K), 256, 0, st>>>(len, ch, Vb, x, parts);
         NEP_CHECK_LAUNCH();
-        nleigs_dots_reduce_kernel<<<ceil_div(K, 128), 128, 0, st>>>(nchunks, K, part, out);
+        return NEP_OK;
+    };
+    auto dots = [&](const zd* Vb, int K, const zd* x, int64_t len, zd* parts, zd* out) -> int {
+        int nch = 0;
+        NEP_TRY(dot_parts(Vb, K, x, len, parts, &nch));
+        nleigs_dots_reduce_kernel<<<ceil_div(K, 128), 128, 0, st>>>(nch, K, parts, out);
+        NEP_CHECK_LAUNCH();
+        return NEP_OK;
+    };
+    auto dots_sums = [&](const zd* Vb, int K, const zd* x, int64_t len, zd* parts, zd* out, Sums* s2) -> int {
+        int nch = 0;
+        NEP_TRY(dot_parts(Vb, K, x, len, parts, &nch));
+        *s2 = Sums{nch, parts};
+        if (nch > kDirectSums) {
+            nleigs_dots_reduce_kernel<<<ceil_div(K, 128), 128, 0, st>>>(nch, K, parts, out);
+            NEP_CHECK_LAUNCH();
+            *s2 = Sums{1, out};
+        }
+        return NEP_OK;
+    };
+    // x -= V (V^H x), twice (classical Gram-Schmidt), the coefficients added to Hcol; then x /= |x| and *hsub = |x|
+    auto orthogonalise = [&](const zd* Vb, int K, zd* x, int64_t len, zd* parts, zd* h, zd* nrm, zd* Hcol, zd* hsub) -> int {
+        Sums sm;
+        for (int pass = 0; pass < 2 && K > 0; ++pass) {
+            NEP_TRY(dots_sums(Vb, K, x, len, parts, h, &sm));
+            nleigs_sub_kernel<<<ceil_div(len, kSubRows), kSubRows * kSubShares, sizeof(zd) * K, st>>>(len, K, Vb, sm.nch, sm.part, x, Hcol);
+            NEP_CHECK_LAUNCH();
+        }
+        NEP_TRY(dots_sums(x, 1, x, len, parts, nrm, &sm));
+        nleigs_scale_kernel<<<ceil_div(len, 256), 256, 0, st>>>(len, x, sm.nch, sm.part, hsub);
         NEP_CHECK_LAUNCH();
         return NEP_OK;
     };
@@ -1011,23 +1094,7 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
     zd *U = nullptr, *Gc = nullptr, *pt = nullptr, *Cc = nullptr, *hacc = nullptr, *hv2 = nullptr, *partn = nullptr;
     zd *rho = nullptr, *nr0 = nullptr;
     int m_cur = 0;
-    const int nchunks_n = (int)((n + chunk - 1) / chunk);
     const int64_t NG = (int64_t)d * Mx;
-    const int nchunks_g = (int)((NG + chunk - 1) / chunk);
-    auto dots_n = [&](const zd* Vb, int K, const zd* x, zd* out) -> int {  // over n entries
-        nleigs_dots_kernel<<<dim3(nchunks_n, K), 256, 0, st>>>(n, chunk, Vb, x, partn);
-        NEP_CHECK_LAUNCH();
-        nleigs_dots_reduce_kernel<<<ceil_div(K, 128), 128, 0, st>>>(nchunks_n, K, partn, out);
-        NEP_CHECK_LAUNCH();
-        return NEP_OK;
-    };
-    auto dots_g = [&](const zd* Vb, int K, const zd* x, zd* out) -> int {  // over d Mx coefficient entries
-        nleigs_dots_kernel<<<dim3(nchunks_g, K), 256, 0, st>>>(NG, chunk, Vb, x, part);
-        NEP_CHECK_LAUNCH();
-        nleigs_dots_reduce_kernel<<<ceil_div(K, 128), 128, 0, st>>>(nchunks_g, K, part, out);
-        NEP_CHECK_LAUNCH();
-        return NEP_OK;
-    };
     // u (n) orthogonalised against the m columns of U twice into the column slot m of U; the
     // coefficients accumulate in hacc, rho = its remaining norm; returns whether U grew (not a breakdown)
     std::vector<double> hp(4, 0.0);
@@ -1035,16 +1102,9 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
         zd* col = U + (int64_t)m * n;
         toar_copy_kernel<<<ceil_div(n, 256), 256, 0, st>>>(n, u, col);
         NEP_CHECK_LAUNCH();
-        NEP_TRY(dots_n(col, 1, col, nr0));
+        NEP_TRY(dots(col, 1, col, n, partn, nr0));
         NEP_CUDA(cudaMemsetAsync(hacc, 0, sizeof(zd) * Mx, st));
-        for (int pass = 0; pass < 2 && m > 0; ++pass) {
-            NEP_TRY(dots_n(U, m, col, hv2));
-            nleigs_sub_kernel<<<ceil_div(n, 256), 256, sizeof(zd) * m, st>>>(n, m, U, hv2, col, hacc);
-            NEP_CHECK_LAUNCH();
-        }
-        NEP_TRY(dots_n(col, 1, col, nr));
-        nleigs_scale_kernel<<<ceil_div(n, 256), 256, 0, st>>>(n, col, nr, rho);
-        NEP_CHECK_LAUNCH();
+        NEP_TRY(orthogonalise(U, m, col, n, partn, hv2, nr, hacc, rho));
         NEP_CUDA(cudaMemcpyAsync(hp.data(), nr0, sizeof(double), cudaMemcpyDeviceToHost, st));
         NEP_CUDA(cudaMemcpyAsync(hp.data() + 2, rho, sizeof(double), cudaMemcpyDeviceToHost, st));
         NEP_CUDA(cudaStreamSynchronize(st));
@@ -1058,7 +1118,7 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
         NEP_TRY(w.get(&Cc, (size_t)nt * Mx));
         NEP_TRY(w.get(&hacc, (size_t)Mx));
         NEP_TRY(w.get(&hv2, (size_t)Mx));
-        NEP_TRY(w.get(&partn, (size_t)nchunks_n * (Mx + 1)));
+        NEP_TRY(w.get(&partn, chunks(n) * (Mx + 1)));
         NEP_TRY(w.get(&rho, 1));
         NEP_TRY(w.get(&nr0, 1));
         NEP_CUDA(cudaMemsetAsync(Gc, 0, sizeof(zd) * (size_t)NG * (kmax + 1), st));
@@ -1073,13 +1133,13 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
             NEP_CHECK_LAUNCH();
             ++m_cur;
         }
-        NEP_TRY(dots_g(Gc, 1, Gc, nr));
+        NEP_TRY(dots(Gc, 1, Gc, NG, part, nr));
         nleigs_normalize_start_kernel<<<ceil_div(NG, 256), 256, 0, st>>>(NG, Gc, nr);
         NEP_CHECK_LAUNCH();
     } else {
         // start vector, unit 2-norm
         NEP_CUDA(cudaMemcpyAsync(V, start_host, sizeof(zd) * (size_t)N, cudaMemcpyHostToDevice, st));
-        NEP_TRY(dots(V, 1, V, nr));
+        NEP_TRY(dots(V, 1, V, N, part, nr));
         nleigs_normalize_start_kernel<<<ceil_div(N, 256), 256, 0, st>>>(N, V, nr);
         NEP_CHECK_LAUNCH();
     }
@@ -1090,7 +1150,8 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
         if (lin.toar) {
             const zd* gk = Gc + (int64_t)k * NG;
             zd* gn = Gc + (int64_t)(k + 1) * NG;
-            toar_coef_kernel<<<ceil_div(m_cur, 128), 128, 0, st>>>(d, m_cur, Mx, nt, gk, pt, Cc, d_ec, d_ddc);
+            toar_coef_kernel<<<ceil_div(m_cur, 32), 32 * kToarWarps, sizeof(zd) * (d + nt * (d + 1) + 32 * d), st>>>(
+                d, m_cur, Mx, nt, gk, pt, Cc, d_ec, d_ddc);
             NEP_CHECK_LAUNCH();
             NEP_TRY(zgemm(n, nt, m_cur, 0, U, n, Cc, Mx, C, n, nullptr, 0, st));  // C_t = U Cc_t
             nleigs_spmv_kernel<<<ceil_div((int64_t)n * 32, 256), 256, 0, st>>>(s, C, rhs);
@@ -1102,15 +1163,8 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
             toar_next_kernel<<<ceil_div(NG, 256), 256, 0, st>>>(d, m_cur, mnew, Mx, pt, hacc, rho, d_ec, gn);
             NEP_CHECK_LAUNCH();
             m_cur = mnew;
-            // Arnoldi on the coefficient vectors, classical Gram-Schmidt twice
-            for (int pass = 0; pass < 2; ++pass) {
-                NEP_TRY(dots_g(Gc, k + 1, gn, hv));
-                nleigs_sub_kernel<<<ceil_div(NG, 256), 256, sizeof(zd) * (k + 1), st>>>(NG, k + 1, Gc, hv, gn, Hcol);
-                NEP_CHECK_LAUNCH();
-            }
-            NEP_TRY(dots_g(gn, 1, gn, nr));
-            nleigs_scale_kernel<<<ceil_div(NG, 256), 256, 0, st>>>(NG, gn, nr, Hcol + k + 1);
-            NEP_CHECK_LAUNCH();
+            // Arnoldi on the coefficient vectors
+            NEP_TRY(orthogonalise(Gc, k + 1, gn, NG, part, hv, nr, Hcol, Hcol + k + 1));
             return NEP_OK;
         }
         const zd* vk = V + (int64_t)k * N;
@@ -1125,14 +1179,7 @@ static int krylov_lin_run(const SplitDev& s, const KrylovLin& lin, int kmax, con
         NEP_TRY(solve());
         nleigs_combine_kernel<<<ceil_div(N, 256), 256, 0, st>>>(n, d, u, wk, d_ec);
         NEP_CHECK_LAUNCH();
-        for (int pass = 0; pass < 2; ++pass) {
-            NEP_TRY(dots(V, k + 1, wk, hv));
-            nleigs_sub_kernel<<<ceil_div(N, 256), 256, sizeof(zd) * (k + 1), st>>>(N, k + 1, V, hv, wk, Hcol);
-            NEP_CHECK_LAUNCH();
-        }
-        NEP_TRY(dots(wk, 1, wk, nr));
-        nleigs_scale_kernel<<<ceil_div(N, 256), 256, 0, st>>>(N, wk, nr, Hcol + k + 1);
-        NEP_CHECK_LAUNCH();
+        NEP_TRY(orthogonalise(V, k + 1, wk, N, part, hv, nr, Hcol, Hcol + k + 1));
         return NEP_OK;
     };
     // Ritz pairs of H = Hf[:m, :m] and the restart work arrays
