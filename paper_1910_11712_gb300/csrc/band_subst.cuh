@@ -37,7 +37,7 @@
 // multiply-adds, 1.8 us a block at bandwidth 64) up to one CTA per SM; beyond that the staging and
 // shared-memory instructions of the update, which is why many columns of complex64 keep the sweeps.
 // n = 4096, bandwidth 64, complex64: one right-hand side 0.461 ms (sweeps .661), 64 points x 16 0.612
-// (.820); complex128: 9 x 1 3.62 ms (10.6), 64 x 16 8.5 (10.7), bandwidth 40 at 128 x 32 7.5 (11.1);
+// (.820); complex128: 9 x 1 3.62 ms (10.6), 64 x 16 6.5 (10.7), bandwidth 40 at 128 x 32 7.5 (11.1);
 // bandwidth 200 with interchanges throughout, n = 3000, 16 x 16 9.8 (12.5, one step at a time).
 #pragma once
 #include <algorithm>
@@ -53,10 +53,15 @@ constexpr int HR = 32, HS = 33;   // rows of a head and its stride between colum
 constexpr int NHD = 6;            // heads held: blocks b-1 .. b+4
 constexpr int RCMAX = 256;        // rows of a staged piece of a backward body
 
-// right-hand sides per half warp of the triangle warps, and those warps
-__host__ __device__ constexpr int tri_rh(int RT) { return RT >= 8 ? 2 : 1; }
-__host__ __device__ constexpr int tri_warps(int RT) { return (RT + 2 * tri_rh(RT) - 1) / (2 * tri_rh(RT)); }
-__host__ __device__ constexpr int threads(int RT) { return 32 * (UW + tri_warps(RT)); }
+// Right-hand sides per half warp of the triangle warps, and those warps. Complex128: one warp on each of the
+// SM's four FP64 units where the registers allow (bandwidth 64, 64 points x 16: 8.47 -> 6.47 ms, 8 right-hand sides
+// having kept two units busy and two waiting).
+template <typename T>
+__host__ __device__ constexpr int tri_rh(int RT) { return RT >= (sizeof(T) == 8 ? 16 : 8) ? 2 : 1; }
+template <typename T>
+__host__ __device__ constexpr int tri_warps(int RT) { return (RT + 2 * tri_rh<T>(RT) - 1) / (2 * tri_rh<T>(RT)); }
+template <typename T>
+__host__ __device__ constexpr int threads(int RT) { return 32 * (UW + tri_warps<T>(RT)); }
 // Row stride of the window: RT elements, padded to 18 for RT = 16 (two rows x four column groups of 32
 // bytes then fall in distinct banks).
 __host__ __device__ constexpr int wstride(int RT) { return RT == 16 ? 18 : RT; }
@@ -88,6 +93,13 @@ __device__ __forceinline__ cx<T> shfl16(cx<T> v, int k) {
     r.re = __shfl_sync(0xffffffffu, v.re, k, 16);
     r.im = __shfl_sync(0xffffffffu, v.im, k, 16);
     return r;
+}
+
+// w times a reciprocal of U's diagonal. Complex128 with its rounding spelled out: the instances for different
+// RT give the same bits.
+__device__ __forceinline__ cx<float> mul_diag(cx<float> w, cx<float> rd) { return w * rd; }
+__device__ __forceinline__ cx<double> mul_diag(cx<double> w, cx<double> rd) {
+    return mk(__fma_rn(w.re, rd.re, -__dmul_rn(w.im, rd.im)), __fma_rn(w.re, rd.im, __dmul_rn(w.im, rd.re)));
 }
 
 // TQ consecutive elements from shared memory (pairs of complex64 as one 16-byte load)
@@ -163,7 +175,7 @@ __device__ __forceinline__ void subst_sweep(int n, int kl, int kv, int ldab, con
                                             const int* __restrict__ ipiv, int nr, cx<T>* B, cx<T>* smem,
                                             size_t smem_bytes) {
     using namespace subst;
-    constexpr int RTP = wstride(RT), NT = threads(RT), UT = 32 * UW;
+    constexpr int RTP = wstride(RT), NT = threads<T>(RT), UT = 32 * UW;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int width = BWD ? kv : kl;
     const int ns = stages(BWD, width, RT, (int)sizeof(cx<T>), smem_bytes);
@@ -357,7 +369,7 @@ __device__ __forceinline__ void subst_sweep(int n, int kl, int kv, int ldab, con
             hs = h1;
         }
     } else {
-        constexpr int RH = tri_rh(RT);
+        constexpr int RH = tri_rh<T>(RT);
         const int i = lane & (NB - 1);
         const int q0 = (2 * (warp - UW) + (lane >> 4)) * RH;  // this half warp's right-hand sides
         const bool live = q0 < RT;
@@ -413,7 +425,7 @@ __device__ __forceinline__ void subst_sweep(int n, int kl, int kv, int ldab, con
 #pragma unroll
                 for (int h = 0; h < RH; ++h) {
                     cx<T> v = w[h];
-                    if constexpr (BWD) v = w[h] * rd;
+                    if constexpr (BWD) v = mul_diag(w[h], rd);
                     const cx<T> xk = shfl16(v, k);
                     if (i == k) x[h] = xk;
                     w[h] = fms(w[h], pc[k], xk);
@@ -450,7 +462,7 @@ __device__ __forceinline__ void subst_sweep(int n, int kl, int kv, int ldab, con
 }
 
 template <typename T, int RT>
-__global__ void __launch_bounds__(subst::threads(RT), 1)
+__global__ void __launch_bounds__(subst::threads<T>(RT), 1)
     band_subst_kernel(int n, int kl, int ku, int ldab, const cx<T>* __restrict__ ab_all,
                       const int* __restrict__ ipiv_all, int L, cx<T>* __restrict__ B_all,
                       const int* __restrict__ active, size_t smem_bytes, const PointDesc* __restrict__ pd) {
@@ -522,7 +534,7 @@ template <typename T, int RT>
 static int run_subst(dim3 grid, size_t smem, int n, int kl, int ku, int ldab, const cx<T>* ab, const int* ipiv, int L,
                      cx<T>* B, const int* active, const PointDesc* pd, cudaStream_t st) {
     NEP_CUDA(allow_max_dynamic_smem(band_subst_kernel<T, RT>));
-    band_subst_kernel<T, RT><<<grid, subst::threads(RT), smem, st>>>(n, kl, ku, ldab, ab, ipiv, L, B, active, smem, pd);
+    band_subst_kernel<T, RT><<<grid, subst::threads<T>(RT), smem, st>>>(n, kl, ku, ldab, ab, ipiv, L, B, active, smem, pd);
     NEP_CHECK_LAUNCH();
     return NEP_OK;
 }
