@@ -37,15 +37,25 @@ constexpr int kBlkUS = kBlkNB + 1;          // staged U row stride (odd: rows fa
 
 // RT right-hand-side columns per CTA (a multiple of 4; columns beyond the point's L stay zero).
 // Shared memory: X (NB x RT, rows 16-byte aligned for paired loads) first, then the window ring
-// (odd row stride RT + 1), then the forward's two L panels and pivots, or the backward's two U
+// (see win), then the forward's two L panels and pivots, or the backward's two U
 // triangles and two staged chunks of U rows.
+// Element q of window row s: an odd row stride RT + 1, or for RT = 16 rows of 16 rotated by their number, so
+// that the lanes of an update (16 rows, both halves) fall in distinct bank pairs either way. Without the
+// padding 16 columns fit at bandwidth 576: 64 points x 32 columns are 128 CTAs of 16, one an SM, where 192 of
+// 12 ran in two waves (24.8 -> 13.7 ms).
+__host__ __device__ constexpr int win_stride(int RT) { return RT == 16 ? 16 : RT + 1; }
+template <int RT>
+__device__ __forceinline__ int win(int s, int q) {
+    return RT == 16 ? s * 16 + ((q + s) & 15) : s * (RT + 1) + q;
+}
+constexpr size_t kBlkSmemMax = 226 * 1024;
 __host__ __device__ inline size_t blk_smem_fwd(int kl, int RT) {
     const size_t PF = kBlkNB + kl;
-    return sizeof(zf) * ((size_t)kBlkNB * RT + PF * (RT + 1) + 2 * (size_t)kBlkNB * PF) + sizeof(int) * 2 * kBlkNB;
+    return sizeof(zf) * ((size_t)kBlkNB * RT + PF * win_stride(RT) + 2 * (size_t)kBlkNB * PF) + sizeof(int) * 2 * kBlkNB;
 }
 __host__ __device__ inline size_t blk_smem_bwd(int kv, int RT) {
     const size_t PB = kBlkNB + kv;
-    return sizeof(zf) * ((size_t)kBlkNB * RT + PB * (RT + 1) + 2 * (size_t)kBlkNB * (kBlkNB + 1) +
+    return sizeof(zf) * ((size_t)kBlkNB * RT + PB * win_stride(RT) + 2 * (size_t)kBlkNB * (kBlkNB + 1) +
                          2 * (size_t)kBlkChunk * kBlkUS);
 }
 
@@ -61,17 +71,17 @@ __device__ __forceinline__ void axpy_row(zf (&acc)[H], zf a, const zf* x) {
     }
 }
 
-// w[q] (q in one half of the RT columns, row stride of w: 1) -= sum_k a[k] X[k][q]
+// window row s -= sum_k a[k] X[k][..] on one half of the RT columns
 template <int RT>
-__device__ __forceinline__ void update_half(zf* w, const zf (&a)[kBlkNB], const zf* X1, int half) {
+__device__ __forceinline__ void update_half(zf* W, int s, const zf (&a)[kBlkNB], const zf* X1, int half) {
     constexpr int H = RT / 2;
     zf acc[H];
 #pragma unroll
-    for (int q = 0; q < H; ++q) acc[q] = w[q];
+    for (int q = 0; q < H; ++q) acc[q] = W[win<RT>(s, half * H + q)];
 #pragma unroll
     for (int k = 0; k < kBlkNB; ++k) axpy_row<H>(acc, a[k], X1 + k * RT + half * H);
 #pragma unroll
-    for (int q = 0; q < H; ++q) w[q] = acc[q];
+    for (int q = 0; q < H; ++q) W[win<RT>(s, half * H + q)] = acc[q];
 }
 
 template <int RT>
@@ -84,7 +94,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
     const int q0 = blockIdx.y * RT;
     const int nr = min(RT, L - q0);
     if (nr <= 0) return;
-    constexpr int NB = kBlkNB, RS = RT + 1, H = RT / 2;
+    constexpr int NB = kBlkNB;
     const int kv = kl + ku;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nthr = blockDim.x, nwarp = nthr >> 5;
@@ -100,13 +110,13 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
     // ===================================================================== forward
     {
         const int PF = NB + kl;
-        zf* W = sm;                                 // PF x RS: row r at slot r mod PF
-        zf* Lp0 = W + (size_t)PF * RS;              // 2 x (NB columns of PF local rows)
+        zf* W = sm;                                 // PF rows: row r at slot r mod PF
+        zf* Lp0 = W + (size_t)PF * win_stride(RT);              // 2 x (NB columns of PF local rows)
         int* pv0 = reinterpret_cast<int*>(Lp0 + 2 * (size_t)NB * PF);  // 2 x NB pivots
         auto Lp = [&](int b) { return Lp0 + (size_t)b * NB * PF; };
         for (int e = tid; e < 2 * NB * PF; e += nthr) Lp0[e] = zero;
         for (int q = 0; q < RT; ++q)
-            for (int r = tid; r < PF; r += nthr) W[r * RS + q] = (r < n && q < nr) ? B[(int64_t)q * n + r] : zero;
+            for (int r = tid; r < PF; r += nthr) W[win<RT>(r, q)] = (r < n && q < nr) ? B[(int64_t)q * n + r] : zero;
         __syncthreads();
         // column k of the panel at c0: local rows k+1 .. k+kl from the stored L column c0+k, rows
         // beyond k+kl zero (an earlier block's interchanges may have left values there); rows 0 .. k
@@ -154,9 +164,9 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                         int s1 = sbase + k, s2 = sbase + p;
                         if (s1 >= PF) s1 -= PF;
                         if (s2 >= PF) s2 -= PF;
-                        const zf t = W[s1 * RS + q];
-                        W[s1 * RS + q] = W[s2 * RS + q];
-                        W[s2 * RS + q] = t;
+                        const zf t = W[win<RT>(s1, q)];
+                        W[win<RT>(s1, q)] = W[win<RT>(s2, q)];
+                        W[win<RT>(s2, q)] = t;
                     }
                 }
             }
@@ -164,7 +174,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
             for (int q = warp; q < nr; q += nwarp) {  // unit lower triangle of the panel form
                 int s = sbase + lane;
                 if (s >= PF) s -= PF;
-                zf w = lane < nbc ? W[s * RS + q] : zero;
+                zf w = lane < nbc ? W[win<RT>(s, q)] : zero;
                 for (int k = 0; k + 1 < nbc; ++k) {
                     const zf xk = shfl_cx(w, k);
                     if (lane > k && lane < nbc) w = fms(w, P[(size_t)k * PF + lane], xk);
@@ -179,8 +189,8 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                 const int r = c0 + PF + i;
                 int s = sbase + i;
                 if (s >= PF) s -= PF;
-                if (r < n) cp_async_cx(&W[s * RS + q], B + (int64_t)q * n + r);
-                else W[s * RS + q] = zero;
+                if (r < n) cp_async_cx(&W[win<RT>(s, q)], B + (int64_t)q * n + r);
+                else W[win<RT>(s, q)] = zero;
             }
             cp_async_commit();
             // rows below the block: w -= L~21 x, two threads a row (one half of the columns each);
@@ -193,7 +203,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                 zf a[NB];
 #pragma unroll
                 for (int k = 0; k < NB; ++k) a[k] = P[(size_t)k * PF + lr];
-                update_half<RT>(W + s * RS + half * H, a, X1, half);
+                update_half<RT>(W, s, a, X1, half);
             }
             sbase += nbc;
             if (sbase >= PF) sbase -= PF;
@@ -206,8 +216,8 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
     {
         const int kv = u_reach(n, ku, ipiv);  // this point's U is no wider
         const int PB = NB + kv;
-        zf* W = sm;                                  // PB x RS: row r at slot r mod PB
-        zf* U0 = W + (size_t)PB * RS;                // 2 x NB x (NB+1): U(top+i, top+k) at i (NB+1) + k
+        zf* W = sm;                                  // PB rows: row r at slot r mod PB
+        zf* U0 = W + (size_t)PB * win_stride(RT);                // 2 x NB x (NB+1): U(top+i, top+k) at i (NB+1) + k
         zf* S0 = U0 + 2 * (size_t)NB * (NB + 1);     // 2 x kBlkChunk x kBlkUS staged U rows
         auto issue_u11 = [&](int c1, int b) {
             const int top = max(0, c1 - NB + 1), nbc = c1 - top + 1;
@@ -239,7 +249,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
             cp_async_commit();
         };
         for (int q = 0; q < RT; ++q)
-            for (int r = max(0, n - PB) + tid; r < n; r += nthr) W[(r % PB) * RS + q] = q < nr ? B[(int64_t)q * n + r] : zero;
+            for (int r = max(0, n - PB) + tid; r < n; r += nthr) W[win<RT>(r % PB, q)] = q < nr ? B[(int64_t)q * n + r] : zero;
         for (int e = tid; e < NB * RT; e += nthr) X1[e] = zero;
         issue_u11(n - 1, 0);
         issue_chunk(n - 1, 0, 0);
@@ -253,7 +263,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
             const zf* Ub = U0 + (size_t)b * NB * (NB + 1);
             for (int q = warp; q < nr; q += nwarp) {  // upper triangle, bottom row first
                 const zf rd = lane < nbc ? pivot_recip(Ub[lane * (NB + 1) + lane]) : zero;
-                zf w = lane < nbc ? W[((top + lane) % PB) * RS + q] : zero;
+                zf w = lane < nbc ? W[win<RT>((top + lane) % PB, q)] : zero;
                 for (int k = nbc - 1; k >= 0; --k) {
                     const zf xk = shfl_cx(w, k) * shfl_cx(rd, k);
                     if (lane == k) w = xk;
@@ -267,7 +277,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
             for (int e = tid; e < nbc * nr; e += nthr) {
                 const int i = e % nbc, q = e / nbc;
                 const int r = top - PB + i;
-                if (r >= 0) cp_async_cx(&W[((top + i) % PB) * RS + q], B + (int64_t)q * n + r);
+                if (r >= 0) cp_async_cx(&W[win<RT>((top + i) % PB, q)], B + (int64_t)q * n + r);
             }
             cp_async_commit();
             // rows above the block, a chunk of staged U rows at a time: w -= U(r, top .. c1) x
@@ -286,7 +296,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                     zf a[NB];
 #pragma unroll
                     for (int k = 0; k < NB; ++k) a[k] = S[l * kBlkUS + k];
-                    update_half<RT>(W + (r % PB) * RS + half * H, a, X1, half);
+                    update_half<RT>(W, r % PB, a, X1, half);
                 }
                 sb ^= 1;
             }
@@ -297,17 +307,26 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
 
 }  // namespace
 
-// Right-hand sides per CTA: the fewest CTAs per point with at most kBlkRMax columns each (rounded
-// up to a multiple of 4) whose windows fit in shared memory; 0 if none does
-int band_solve_blocked_rhs(int kl, int ku, int L) {
-    const int kv = kl + ku;
-    for (int groups = (L + kBlkRMax - 1) / kBlkRMax; groups <= L; ++groups) {
-        const int RT = (((L + groups - 1) / groups) + 3) / 4 * 4;
-        const size_t bytes = std::max(blk_smem_fwd(kl, RT), blk_smem_bwd(kv, RT));
-        if (bytes <= 220 * 1024) return RT;
-        if (RT == 4) break;
+// Right-hand sides per CTA (a multiple of 4 up to kBlkRMax whose windows fit in shared memory; 0 if none does):
+// the split of a point's columns with the least time, waves of one CTA per SM times 17.5 + columns (bandwidth
+// 576, 64 points, ms: 16 columns as 2 x 8 10.5, as 16 13.9; 32 as 2 x 16 13.7, as 3 x 12 in two waves 24.8).
+// The results do not depend on it.
+int band_solve_blocked_rhs(int kl, int ku, int npts, int L) {
+    static const int sms = [] {
+        int dev = 0, v = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        return v > 0 ? v : 152;
+    }();
+    int best = 0;
+    double least = 0;
+    for (int RT = kBlkRMax; RT >= 4; RT -= 4) {
+        if (std::max(blk_smem_fwd(kl, RT), blk_smem_bwd(kl + ku, RT)) > kBlkSmemMax) continue;
+        const int64_t groups = (L + RT - 1) / RT;
+        const double t = (double)(((int64_t)std::max(npts, 1) * groups + sms - 1) / sms) * (17.5 + RT);
+        if (best == 0 || t < least) best = RT, least = t;
     }
-    return 0;
+    return best;
 }
 
 template <int RT>
@@ -325,7 +344,7 @@ static int launch_blocked(const SplitDev& s, int npts, const zf* ab, const int* 
 int launch_band_solve_blocked(const SplitDev& s, int npts, const zf* ab, const int* ipiv, int L, zf* B,
                               const int* active, cudaStream_t st) {
     if (npts <= 0 || L <= 0) return NEP_OK;
-    switch (band_solve_blocked_rhs(s.kl, s.ku, L)) {
+    switch (band_solve_blocked_rhs(s.kl, s.ku, npts, L)) {
         case 4: return launch_blocked<4>(s, npts, ab, ipiv, L, B, active, st);
         case 8: return launch_blocked<8>(s, npts, ab, ipiv, L, B, active, st);
         case 12: return launch_blocked<12>(s, npts, ab, ipiv, L, B, active, st);

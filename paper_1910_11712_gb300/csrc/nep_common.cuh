@@ -306,7 +306,7 @@ bool band_subst_chosen(int kl, int ku, int npts, int L);  // band_lu.cu: this so
 inline bool band_sweeps_fit(int kl, int ku) { return kl >= 1 && kl + 1 <= 288 && kl + ku + 1 <= 288; }
 // band_solve_blocked.cu: the blocked substitution for complex64 factors of wider bands (NB-step
 // blocks, products for the rows beyond each block); NEP_ERR_UNSUPPORTED when its windows do not fit
-int band_solve_blocked_rhs(int kl, int ku, int L);
+int band_solve_blocked_rhs(int kl, int ku, int npts, int L);
 int launch_band_solve_blocked(const SplitDev& s, int npts, const zf* ab, const int* ipiv, int L, zf* B,
                               const int* active, cudaStream_t st);
 // Whether a solve needs the column copy of U (ut) that the sweeps read.
