@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(512)
 // needs no column copy of U, but its arithmetic costs more instructions per right-hand side: measured, ms
 // per solve, sweeps (without the copy of U) against substitution, points x right-hand sides, both with
 // backward windows of kl + ku rows:
-//   complex64, bandwidth 64: 1 x 1 .661 / .463, 9 x 4 .680 / .549, 64 x 16 .820 / .673, 128 x 16 1.11 / 2.34
-//   (64 of its 256 CTAs in a last wave or 16 right-hand sides a CTA); bandwidth 24: 32 x 8 .090 / .065;
+//   complex64, bandwidth 64: 1 x 1 .661 / .463, 9 x 4 .680 / .549, 64 x 16 .820 / .673, 128 x 16 1.11 / 2.34;
+//   bandwidth 24: 32 x 8 .090 / .065;
 //   bandwidth 40: 64 x 16 .324 / .238, 128 x 32 .562 / .735; bandwidth 97: 64 x 16 2.40 / 2.62;
 //   bandwidth 128: 1 x 1 3.05 / 2.23;
 //   complex128, bandwidth 64: 9 x 1 10.6 / 3.6, 64 x 16 10.7 / 10.5; bandwidth 40: 128 x 32 11.1 / 9.1;
@@ -444,7 +444,8 @@ int launch_band_solve(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>*
     // blocked substitution, or register windows for narrow bands (kl+1 <= 288 and kv+1 <= 288 rows): two sweeps with
     // slot-ordered coefficients
     if (band_subst_chosen<T>(s.kl, s.ku, npts, L)) return band_subst<T>(s, npts, ab, ipiv, L, B, active, st, rh_force);
-    if (band_sweeps_fit(s.kl, s.ku)) return band_sweeps<T>(s, npts, ab, ut, ipiv, L, B, active, st, rh_force);
+    if constexpr (sizeof(T) == 4)
+        if (band_sweeps_fit(s.kl, s.ku)) return band_sweeps<T>(s, npts, ab, ut, ipiv, L, B, active, st, rh_force);
     // complex64 factors: blocked substitution (NEP_SOLVE_UNBLOCKED=1 keeps the per-step sweeps below)
     if constexpr (sizeof(T) == 4) {
         static const bool unblocked = [] {

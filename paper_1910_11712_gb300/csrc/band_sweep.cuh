@@ -1,6 +1,5 @@
 // Banded forward/backward substitution sweeps for narrow bands (kernel (b), solve part).
-// Instantiated once per element type (band_sweep_f.cu, band_sweep_d.cu) so the two compile in
-// parallel.
+// Instantiated for complex64 in band_sweep_f.cu.
 #pragma once
 #include <algorithm>
 #include <cstdlib>
@@ -19,7 +18,7 @@ namespace nep {
 constexpr int kFullWindow = 16;
 template <typename T>
 inline int sweep_shape(int W, int rh) {
-    return sizeof(T) == 4 && rh >= 2 && W >= 64 && W <= 128 && W % 32 == 0 ? kFullWindow + W / 32 : W / 32 + 1;
+    return rh >= 2 && W >= 64 && W <= 128 && W % 32 == 0 ? kFullWindow + W / 32 : W / 32 + 1;
 }
 __host__ __device__ inline bool sweep_covers(int shape, int W) {
     return shape > kFullWindow ? W == 32 * (shape - kFullWindow) : W < 32 * shape;
@@ -323,7 +322,7 @@ static int sweep_batch_rpl(int rpl, int count, int maxL, const PointDesc* pd, cu
         case 8: return run_sweep_batch<T, 8, BWD, RH>(count, maxL, pd, st, done);
         case 9: return run_sweep_batch<T, 9, BWD, RH>(count, maxL, pd, st, done);
     }
-    if constexpr (sizeof(T) == 4 && RH >= 2)
+    if constexpr (RH >= 2)
         switch (rpl) {
             case kFullWindow + 2: return run_sweep_batch<T, 2, BWD, RH, true>(count, maxL, pd, st, done);
             case kFullWindow + 3: return run_sweep_batch<T, 3, BWD, RH, true>(count, maxL, pd, st, done);
@@ -363,9 +362,8 @@ static int sweep_rh(int chains) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         return 4 * (sms > 0 ? sms : 152);
     }();
-    // about one or two warps per sub-partition; complex FP64 (FP64-throughput-bound) takes at least two
-    const int rh = chains >= 6 * smsp ? 4 : 2 * chains >= 3 * smsp ? 2 : 1;
-    return sizeof(T) == 4 ? rh : (rh < 2 ? 2 : rh);
+    // about one or two warps per sub-partition
+    return chains >= 6 * smsp ? 4 : 2 * chains >= 3 * smsp ? 2 : 1;
 }
 
 template <typename T, bool BWD, int RH>
@@ -382,7 +380,7 @@ static int sweep_rpl(int rpl, const SplitDev& s, int npts, const cx<T>* ab, cons
         case 8: return run_sweep<T, 8, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
         case 9: return run_sweep<T, 9, BWD, RH>(s, npts, ab, ut, ipiv, L, B, active, st, done);
     }
-    if constexpr (sizeof(T) == 4 && RH >= 2)
+    if constexpr (RH >= 2)
         switch (rpl) {
             case kFullWindow + 2: return run_sweep<T, 2, BWD, RH, true>(s, npts, ab, ut, ipiv, L, B, active, st, done);
             case kFullWindow + 3: return run_sweep<T, 3, BWD, RH, true>(s, npts, ab, ut, ipiv, L, B, active, st, done);

@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256) split_residual_kernel(const int64_t* __re
 
 // Right-hand sides per thread of the residual kernels: four where the blocks still fill the device.
 // n = 16384, five-point, 128 points x 32, double-float: 1.28 ms with one (T's values read 32 times a point
-// through L2), 0.68 with four; FP64 residual of 128 points x 16 with its assembly: 3.42 -> 1.23 ms, then
+// through L2), 0.68 with four; FP64 residual of 64 points x 32 with its assembly: 3.42 -> 1.23 ms, then
 // bound by the FP64 units.
 static int residual_rl(int n, int npts, int L) {
     return L >= 4 && (int64_t)ceil_div(n, 256) * npts * ((L + 3) / 4) >= 608 ? 4 : 1;
