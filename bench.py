@@ -141,23 +141,31 @@ def measured_peaks():
 
 
 def lu_flops(n, kl, ku, npts):
-    """Algorithmic real flops of the banded LU: n steps x kl rows x (kl+ku) columns x 8 (complex FMA)."""
-    return 8.0 * n * kl * (kl + ku) * npts
+    """Column steps of kl rows by the ku columns that U fills without interchanges, 8 flops a complex FMA."""
+    return 8.0 * n * kl * ku * npts
 
 
 def solve_flops(n, kl, ku, L, npts):
-    """Forward (kl) plus backward (kl+ku) complex FMAs per row and right-hand side, 8 flops each."""
-    return 8.0 * n * (2 * kl + ku) * L * npts
+    """Forward (kl) plus backward (ku, without interchanges) complex FMAs per row and right-hand side, 8 flops each."""
+    return 8.0 * n * (kl + ku) * L * npts
 
 
-def solve_bytes(n, ldab, L, npts, esz):
-    """Factor band and pivots read once, right-hand sides read and written once."""
-    return npts * (n * ldab * esz + 4 * n + 2 * n * L * esz)
+def solve_bytes(n, kl, ku, L, npts, esz):
+    """L, U without interchanges and pivots read once, right-hand sides read and written once."""
+    return npts * (n * (kl + ku + 1) * esz + 4 * n + 2 * n * L * esz)
 
 
 # DRAM bytes (read + write) of one solve launch from an ncu capture of the same launch,
 # keyed by (workload, precision); None where no capture of the current kernel exists.
-SOLVE_TRAFFIC = {("delay2d_s64", "mixed"): (199.1 + 23.9 + 301.0 + 28.6) * 1e6}
+SOLVE_TRAFFIC = {("delay2d_s64", "mixed"): (386.8 + 50.9) * 1e6}
+
+
+def solve_kernel(split, npts, L, mixed):
+    """Name of the kernel(s) that the library takes for a solve of this shape (csrc/band_lu.cu)."""
+    narrow = split.kl + 1 <= 288 and split.kl + split.ku + 1 <= 288
+    if not mixed or (narrow and (L == 1 or (npts * L <= 1024 and split.kl + split.ku <= 144))):
+        return "band_subst_kernel"
+    return "band_sweep_kernel x2" if narrow else "band_solve_blocked_kernel"
 
 
 def fp32_alu_peak_tflops(sm_mhz):
@@ -743,7 +751,7 @@ def main():
         alu_src = ("derived: 152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz" if mixed else
                    "derived: 152 SMs x 1.75 FP64 FMA/clk (measured) x 2 flop x 2070 MHz")
         s_flops = solve_flops(p.n, split.kl, split.ku, p.L, p.N)
-        s_bytes = solve_bytes(p.n, split.ldab, p.L, p.N, esz)
+        s_bytes = solve_bytes(p.n, split.kl, split.ku, p.L, p.N, esz)
         hbm = peaks.get("hbm_gbs", 6800.0)
         lu = float(np.mean(lu_ms))
         line = {
@@ -757,8 +765,7 @@ def main():
                           "band_mb_per_step": round(p.N * p.n * split.ldab * esz / 1e6),
                           "streams": S, "concurrency": f"{S} independent plans on {S} non-blocking streams, one "
                           "host thread each; every step a full pass of its own"},
-            "roofline": {"kernel": ("band_sweep_kernel x2" if split.kl + 1 <= 288 and split.kl + split.ku + 1 <= 288
-                                    else ("band_solve_blocked_kernel" if mixed else "band_solve_kernel")) +
+            "roofline": {"kernel": solve_kernel(split, p.N, p.L, mixed) +
                                    " (forward + backward banded substitution, "
                                    f"{p.N} points x {p.L} right-hand sides in one launch)",
                          "bound": "hbm", "achieved": s_bytes / (solve_ms * 1e-3) / 1e9, "peak": hbm,
