@@ -59,29 +59,48 @@ __host__ __device__ inline size_t blk_smem_bwd(int kv, int RT) {
                          2 * (size_t)kBlkChunk * kBlkUS);
 }
 
-// acc[q] -= a * x[q] for the H values x (16-byte aligned), read two at a time
-template <int H>
-__device__ __forceinline__ void axpy_row(zf (&acc)[H], zf a, const zf* x) {
-    const float4* x2 = reinterpret_cast<const float4*>(x);
-#pragma unroll
-    for (int h = 0; h < H / 2; ++h) {
-        const float4 v = x2[h];
-        acc[2 * h] = fms(acc[2 * h], a, mk(v.x, v.y));
-        acc[2 * h + 1] = fms(acc[2 * h + 1], a, mk(v.z, v.w));
-    }
+// X, the block's solution rows: the columns 2 p and 2 p + 1 of row k as (re, re, im, im)
+template <int RT>
+__device__ __forceinline__ void x_put(zf* X1, int k, int q, zf v) {
+    float* x = reinterpret_cast<float*>(X1 + k * RT + (q & ~1)) + (q & 1);
+    x[0] = v.re;
+    x[2] = v.im;
 }
 
-// window row s -= sum_k a[k] X[k][..] on one half of the RT columns
+// Window row s -= sum_k a[k] X[k][..] on one half of the RT columns, two columns per packed multiply-add (the
+// operations of fms() in each). Bandwidth 576, 64 points: 16, 24 and 32 columns 10.47, 12.30 and 13.71 -> 10.28,
+// 11.95 and 13.28 ms a solve: shared-memory accesses and the copies bound it, not the multiply-adds.
 template <int RT>
 __device__ __forceinline__ void update_half(zf* W, int s, const zf (&a)[kBlkNB], const zf* X1, int half) {
-    constexpr int H = RT / 2;
-    zf acc[H];
+    constexpr int H = RT / 2, P = H / 2;
+    unsigned long long re[P], im[P];
 #pragma unroll
-    for (int q = 0; q < H; ++q) acc[q] = W[win<RT>(s, half * H + q)];
+    for (int p = 0; p < P; ++p) {
+        const zf w0 = W[win<RT>(s, half * H + 2 * p)], w1 = W[win<RT>(s, half * H + 2 * p + 1)];
+        re[p] = pack2(w0.re, w1.re);
+        im[p] = pack2(w0.im, w1.im);
+    }
 #pragma unroll
-    for (int k = 0; k < kBlkNB; ++k) axpy_row<H>(acc, a[k], X1 + k * RT + half * H);
+    for (int k = 0; k < kBlkNB; ++k) {
+        const ulonglong2* x = reinterpret_cast<const ulonglong2*>(X1 + k * RT + half * H);
+        const unsigned long long nr = pack2(-a[k].re, -a[k].re), ai = pack2(a[k].im, a[k].im), ni = pack2(-a[k].im, -a[k].im);
 #pragma unroll
-    for (int q = 0; q < H; ++q) W[win<RT>(s, half * H + q)] = acc[q];
+        for (int p = 0; p < P; ++p) {
+            const ulonglong2 v = x[p];
+            re[p] = fma2(nr, v.x, re[p]);
+            re[p] = fma2(ai, v.y, re[p]);
+            im[p] = fma2(nr, v.y, im[p]);
+            im[p] = fma2(ni, v.x, im[p]);
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        zf w0, w1;
+        unpack2(re[p], w0.re, w1.re);
+        unpack2(im[p], w0.im, w1.im);
+        W[win<RT>(s, half * H + 2 * p)] = w0;
+        W[win<RT>(s, half * H + 2 * p + 1)] = w1;
+    }
 }
 
 template <int RT>
@@ -179,7 +198,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                     const zf xk = shfl_cx(w, k);
                     if (lane > k && lane < nbc) w = fms(w, P[(size_t)k * PF + lane], xk);
                 }
-                if (lane < NB) X1[lane * RT + q] = w;  // zero beyond the block's nbc rows
+                if (lane < NB) x_put<RT>(X1, lane, q, w);  // zero beyond the block's nbc rows
                 if (lane < nbc) B[(int64_t)q * n + c0 + lane] = w;
             }
             __syncthreads();
@@ -269,7 +288,7 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
                     if (lane == k) w = xk;
                     else if (lane < k) w = fms(w, Ub[lane * (NB + 1) + k], xk);
                 }
-                if (lane < NB) X1[lane * RT + q] = lane < nbc ? w : zero;
+                if (lane < NB) x_put<RT>(X1, lane, q, lane < nbc ? w : zero);
                 if (lane < nbc) B[(int64_t)q * n + top + lane] = w;
             }
             __syncthreads();
@@ -309,7 +328,8 @@ __global__ void __launch_bounds__(kBlkThreads, 1)
 
 // Right-hand sides per CTA (a multiple of 4 up to kBlkRMax whose windows fit in shared memory; 0 if none does):
 // the split of a point's columns with the least time, waves of one CTA per SM times 17.5 + columns (bandwidth
-// 576, 64 points, ms: 16 columns as 2 x 8 10.5, as 16 13.9; 32 as 2 x 16 13.7, as 3 x 12 in two waves 24.8).
+// 576, 64 points, ms, before the packed multiply-adds: 16 columns as 2 x 8 10.5, as 16 13.9; 32 as 2 x 16 13.7,
+// as 3 x 12 in two waves 24.8).
 // The results do not depend on it.
 int band_solve_blocked_rhs(int kl, int ku, int npts, int L) {
     static const int sms = [] {

@@ -73,6 +73,22 @@ __device__ __forceinline__ void set_reg(cx<T> (&a)[RPL], int q, cx<T> v) {
         if (t == q) a[t] = v;
 }
 
+// Packed pairs of floats for fma.rn.f32x2 (sm_100 and later): every lane is an ordinary fused
+// multiply-add with one rounding.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
 // Columns beyond the diagonal that U can reach: ku + the farthest pivot row below its step (kl + ku at
 // most), from the interchanges. Run by the whole CTA; ends with a barrier. Without interchanges the
 // backward substitution then reads and multiplies ku columns of U, not kl + ku.

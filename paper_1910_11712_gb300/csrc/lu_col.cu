@@ -50,22 +50,6 @@ __device__ __forceinline__ int warp_argmax_first(T best, int bi) {
     }
 }
 
-// Packed pairs of floats for fma.rn.f32x2 (sm_100 and later): every lane is an ordinary fused
-// multiply-add with one rounding.
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
 // v, or +0 when z (by bit mask)
 template <typename T>
 __device__ __forceinline__ cx<T> mask_cx(cx<T> v, bool z) {
