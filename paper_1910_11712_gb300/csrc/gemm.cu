@@ -46,19 +46,20 @@ __global__ void __launch_bounds__(256, 2)
         if (tid < TB) ea[tid] = eb[tid] = 0;
         if (tid == 0) bad = 0;
         __syncthreads();
-        // lanes along the contiguous index: A by rows (op A) or by k (op A^H), B by k
+        // lanes along the contiguous index: A by rows (op A) or by k (op A^H), B by k; a warp's 32 entries by k belong
+        // to one row or column, and terms beyond the block count as zeros
         for (int e = tid; e < TB * CH; e += 256) {
             const int m = opA == 0 ? e & (TB - 1) : e / CH, k = opA == 0 ? e / TB : e & (CH - 1);
-            if (k < kn && m < mu) {
-                int x = exp_field(aval(m, k0 + k));
-                if (opA != 0) x = __reduce_max_sync(__activemask(), x);  // one row per warp
-                if (opA == 0 || (tid & 31) == 0) atomicMax(&ea[m], x);
+            const int xa = k < kn ? exp_field(aval(m, k0 + k)) : 0;
+            if (opA == 0) {
+                if (xa) atomicMax(&ea[m], xa);
+            } else {
+                const int x = __reduce_max_sync(0xffffffffu, xa);
+                if (lane == 0 && x) atomicMax(&ea[m], x);
             }
             const int c = e / CH, kk = e & (CH - 1);
-            if (kk < kn && c < nu) {
-                const int x = __reduce_max_sync(__activemask(), exp_field(bval(c, k0 + kk)));
-                if ((tid & 31) == 0) atomicMax(&eb[c], x);
-            }
+            const int xb = __reduce_max_sync(0xffffffffu, kk < kn ? exp_field(bval(c, k0 + kk)) : 0);
+            if (lane == 0 && xb) atomicMax(&eb[c], xb);
         }
         __syncthreads();
         if (tid < TB) {
