@@ -20,7 +20,11 @@ constexpr int S = 8;              // digits
 constexpr int CH = 64;            // complex terms per exact accumulation
 constexpr int EXP_LO = 623, EXP_HI = 1423;  // exponent fields taken (2^-400 .. 2^400)
 
-__device__ __forceinline__ int exp_field(double x) { return (int)((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff; }
+// exponent field of x, 1 for subnormal numbers and 0 for zero alone
+__device__ __forceinline__ int exp_field(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) << 1;
+    return max((int)(b >> 53), b != 0 ? 1 : 0);
+}
 __device__ __forceinline__ int exp_field(zd c) { return max(exp_field(c.re), exp_field(c.im)); }
 
 // x as digits + 128 in the bytes of the result, E the exponent field that scales it
