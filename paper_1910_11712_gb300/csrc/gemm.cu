@@ -1,18 +1,19 @@
 // Dense complex FP64 products C = op(A) B (column-major, op in {A, A^H}) of the extraction, on the tensor core by
 // exact 8-bit digit products (oz.cuh).
 //
-// A CTA of 8 warps computes a 32 x 32 tile, K in blocks of 64: the exponents of the tile's rows and columns over
-// the block, then twice 32 terms as digits in the MMA fragments' order in shared memory (A 64 KB, B 32 KB) and
-// 36 x 4 MMA steps per warp and 8 x 8 subtile (a warp takes 8 rows by 16 columns); the exact sums of a block
+// A CTA of 8 warps computes a 32 x 32 tile, K in blocks of 64: the exponents of the tile's rows and
+// columns over the block, then twice 32 terms as digits in the MMA fragments' order in shared memory (A 64 KB, B 32 KB)
+// and 36 x 4 MMA steps per warp and 8 x 8 subtile (a warp takes 8 rows by 16 columns); the exact sums of a block
 // become FP64 once. Long K splits over CTAs into a workspace reduced in a fixed order, so results never depend
-// on scheduling. Blocks with a non-finite entry or an extreme exponent are summed in FP64 FMAs.
+// on scheduling. Blocks with a non-finite entry or an extreme exponent are summed in FP64 FMAs, and so are the
+// terms of a block for every result that the guard (oz.cuh) finds too small for the digits.
 #include "oz.cuh"
 
 namespace nep {
 
 namespace {
 constexpr int TB = 32, KH = 32, KCH = KH / 8;  // tile, terms per staged half, MMA steps of a half
-constexpr size_t A_WORDS = 4 * KCH * oz::S * 128, B_WORDS = 4 * KCH * oz::S * 64;
+constexpr size_t A_WORDS = 4 * KCH * oz::S * 128, B_WORDS = 4 * KCH * oz::S * 64, G_WORDS = 4 * KCH * 64;
 }  // namespace
 
 __global__ void __launch_bounds__(256, 2)
@@ -22,6 +23,8 @@ __global__ void __launch_bounds__(256, 2)
     extern __shared__ uint4 sm4[];
     unsigned* Af = reinterpret_cast<unsigned*>(sm4);  // [4 row tiles][KCH][S][32 lanes][4]
     unsigned* Bf = Af + A_WORDS;                      // [4 column tiles][KCH][S][32 lanes][2]
+    unsigned* Ag = Bf + B_WORDS;                      // [4 row tiles][KCH][32 lanes][2]: the guard's leading bits
+    unsigned* Bg = Ag + G_WORDS;                      // [4 column tiles][KCH][32 lanes][2]
     __shared__ int ea[TB], eb[TB], bad;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = blockIdx.x * TB, n0 = blockIdx.y * TB;
@@ -65,8 +68,8 @@ __global__ void __launch_bounds__(256, 2)
         if (tid < TB) {
             int x = ea[tid], y = eb[tid];
             if ((x && (x < EXP_LO || x > EXP_HI)) || (y && (y < EXP_LO || y > EXP_HI))) bad = 1;
-            if (x == 0) ea[tid] = 1023;
-            if (y == 0) eb[tid] = 1023;
+            if (x == 0) ea[tid] = E_ZERO;
+            if (y == 0) eb[tid] = E_ZERO;
         }
         __syncthreads();
         if (bad) {
@@ -82,7 +85,7 @@ __global__ void __launch_bounds__(256, 2)
                 }
             continue;
         }
-        float D[2][S][4];
+        float D[2][S][4], G[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -102,6 +105,7 @@ __global__ void __launch_bounds__(256, 2)
                     for (int t = 0; t < S; ++t)
                         *reinterpret_cast<uint2*>(f + t * 128) =
                             make_uint2(digits2(re, ni, S - 1 - t), digits2(im, re, S - 1 - t));
+                    Ag[((m >> 3) * KCH + (k >> 3)) * 64 + ((m & 7) * 4 + (k & 3)) * 2 + ((k & 4) ? 1 : 0)] = lead2(lead(c, E));
                 }
                 const int c = e / KH;
                 if (c < nu) {
@@ -112,6 +116,7 @@ __global__ void __launch_bounds__(256, 2)
                     unsigned* f = Bf + (((c >> 3) * KCH + (k >> 3)) * S) * 64 + ((c & 7) * 4 + (k & 3)) * 2 + ((k & 4) ? 1 : 0);
 #pragma unroll
                     for (int t = 0; t < S; ++t) f[t * 64] = digits2(re, im, S - 1 - t);
+                    Bg[((c >> 3) * KCH + (k >> 3)) * 64 + ((c & 7) * 4 + (k & 3)) * 2 + ((k & 4) ? 1 : 0)] = lead2(lead(y, E));
                 }
             }
             __syncthreads();
@@ -119,6 +124,11 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll 1
             for (int kc = 0; kc < kcs; ++kc) {
                 const uint4* a4 = reinterpret_cast<const uint4*>(Af) + (mt * KCH + kc) * S * 32 + lane;
+                {  // the guard, columns by rows: one step for the warp's 16 columns
+                    const uint2* gb = reinterpret_cast<const uint2*>(Bg) + (nt0 * KCH + kc) * 32 + lane;
+                    const uint2 b0 = gb[0], b1 = gb[KCH * 32], a = reinterpret_cast<const uint2*>(Ag)[(mt * KCH + kc) * 32 + lane];
+                    mma16816(G, make_uint4(b0.x, b1.x, b0.y, b1.y), a.x, a.y);
+                }
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
                     if (8 * mt >= mu || 8 * (nt0 + u) >= nu) continue;
@@ -136,11 +146,30 @@ __global__ void __launch_bounds__(256, 2)
             }
         }
         // columns 2 (lane % 4) + (q & 1); rows lane / 4 (Re for q < 2, else Im)
+        const int Ea = ea[8 * mt + g];
+        double s[2][4];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-                out[u][q] += combine(D[u], q, ea[8 * mt + g], eb[8 * (nt0 + u) + 2 * tq + (q & 1)]);
+            for (int q = 0; q < 4; ++q) s[u][q] = combine(D[u], q, Ea, eb[8 * (nt0 + u) + 2 * tq + (q & 1)]);
+#pragma unroll 1
+        for (int p = 0; p < 4; ++p) {  // (u, q) = (p / 2, p % 2)
+            const int u = p >> 1, q = p & 1, from = 4 * (2 * tq + q) + (g >> 1);  // G's lanes: column lane / 4, rows 2 (lane % 4) + (0, 1)
+            const float g0 = __shfl_sync(0xffffffffu, u ? G[2] : G[0], from), g1 = __shfl_sync(0xffffffffu, u ? G[3] : G[1], from);
+            const bool weak = ((g & 1) ? g1 : g0) < GUARD && Ea != E_ZERO && eb[8 * (nt0 + u) + 2 * tq + q] != E_ZERO;
+            const unsigned todo = __ballot_sync(0xffffffffu, weak);
+            if (!todo) continue;
+            const zd t = fp64_sums(todo, kn, opA == 0 ? A + m0 + 8 * mt + (int64_t)lda * k0 : A + k0 + (int64_t)lda * (m0 + 8 * mt),
+                                   opA == 0 ? 1 : lda, opA == 0 ? lda : 1, opA != 0,
+                                   B + k0 + (int64_t)ldb * (n0 + 8 * (nt0 + u) + q), 2 * (int64_t)ldb, 1);
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (v == p && weak) s[v >> 1][v & 1] = t.re, s[v >> 1][2 + (v & 1)] = t.im;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) out[u][q] += s[u][q];
     }
     zd* Cz = C + (int64_t)blockIdx.z * part_stride;
 #pragma unroll
@@ -171,9 +200,9 @@ int zgemm(int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int l
         cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
         return v > 0 ? v : 152;
     }();
+    const int room = part ? std::max(1, (int)std::min<size_t>(64, part_elems / ((size_t)M * N))) : 1;  // splits of K
     // blocks of 64 terms over as many CTAs as two per SM allow
     const int tiles = ceil_div(M, TB) * ceil_div(N, TB), blocks = std::max(1, ceil_div(K, oz::CH));
-    const int room = part ? (int)std::min<size_t>(64, part_elems / ((size_t)M * N)) : 1;
     int splits = std::max(1, std::min(std::min(blocks, room), 2 * sms / tiles));
     const int kchunk = ceil_div(blocks, splits) * oz::CH;
     splits = std::max(1, ceil_div(K, kchunk));
@@ -181,7 +210,7 @@ int zgemm(int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int l
     const int ldo = splits == 1 ? ldc : M;
     const int64_t ps = splits == 1 ? 0 : (int64_t)M * N;
     NEP_CUDA(allow_max_dynamic_smem(zgemm_oz_kernel));
-    zgemm_oz_kernel<<<dim3(ceil_div(M, TB), ceil_div(N, TB), splits), 256, sizeof(unsigned) * (A_WORDS + B_WORDS), st>>>(
+    zgemm_oz_kernel<<<dim3(ceil_div(M, TB), ceil_div(N, TB), splits), 256, sizeof(unsigned) * (A_WORDS + B_WORDS + 2 * G_WORDS), st>>>(
         M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps);
     NEP_CHECK_LAUNCH();
     if (splits > 1) {

@@ -29,6 +29,33 @@ def _cplx(rng, *shape):
     return rng.standard_normal(shape) + 1j * rng.standard_normal(shape)
 
 
+def _scales(rng, n, s):
+    """1/s, s or 1 for every term, each of them at least once where there is room."""
+    e = rng.integers(-1, 2, n)
+    e[: min(n, 3)] = [-1, 1, 0][: min(n, 3)]
+    return float(s) ** rng.permutation(e)
+
+
+@pytest.mark.parametrize("n,P,nv", [(2, 1, 1), (16, 2, 3), (64, 33, 8), (65, 8, 9), (300, 70, 5)])
+@pytest.mark.parametrize("s", [1e3, 1e6, 1e10, 1e60])
+def test_dense_products(bnd, n, P, nv, s):
+    """D = Y^H V with V scaled by d and Y by 1 / d, then X (D / (z - lambda)) with the columns of X scaled likewise."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(n + P)
+    lam, X, Y, z, V = _cplx(rng, P), _cplx(rng, n, P), _cplx(rng, n, P), 8 + _cplx(rng, 1), _cplx(rng, n, nv)
+    d, e = _scales(rng, n, s), _scales(rng, P, s)
+    V, Y, X = V * d[:, None], Y / d[:, None] * e, X / e
+    out = torch.empty(2 * n * nv, dtype=torch.float64, device="cuda")
+    args = [_dev(torch, a) for a in (lam, X, Y, z, V)]
+    bnd.apply_resolvent(n, P, args[0], args[1], args[2], 1, args[3], nv, args[4], out)
+    got = out.cpu().numpy().view(np.complex128).reshape(nv, n).T
+    w = z[0].astype(np.clongdouble) - lam.astype(np.clongdouble)
+    ref = X.astype(np.clongdouble) @ ((Y.conj().T.astype(np.clongdouble) @ V.astype(np.clongdouble)) / w[:, None])
+    size = np.abs(X) @ ((np.abs(Y).T @ np.abs(V)) / np.abs(w)[:, None])
+    # n + P terms, two roundings each per component, and those of the weights
+    assert (np.abs(got - ref) <= 4 * (n + P + 4) * EPS * size).all()
+
+
 @pytest.mark.parametrize("zeros", [False, True])
 def test_subnormal_columns(bnd, zeros):
     """A column all of whose entries are subnormal is not a zero column; beside exactly zero ones or not."""
