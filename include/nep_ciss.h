@@ -566,8 +566,10 @@ int nep_band_solve_cols(nep_split_t h, int32_t npts, int32_t precision, const vo
 /* Kernel (c): FP64 split-form residual R_j = V - T(z_j) Y_j (npts x n x L complex128). */
 int nep_split_residual(nep_split_t h, int32_t npts, const double *F_dev, int32_t L, const double *V_dev,
                        const double *Y_dev, double *R_dev, void *stream);
-/* Kernel (d): S_k = sum_j coef[j + N*k] Y_j for k < K (Y: N x n x L, S: K x n x L complex128);
- * j summed in ascending order. */
+/* Kernel (d): S_k = sum_j coef[j + N*k] Y_j for k < K (Y: N x n x L, S: K x n x L complex128). The order of the
+ * sum is not specified: up to 192 points the products are summed exactly in fixed point and rounded once per 64 of
+ * them wherever that is at least as accurate as FP64, else in FP64. The error of every element is within N FP64
+ * multiply-adds' bound, and the result does not depend on scheduling. */
 int nep_moments(int32_t n, int32_t L, int32_t N, int32_t K, const double *coef_dev, const double *Y_dev, double *S_dev,
                 void *stream);
 /* One-sided Jacobi SVD (FP64, device): A (rows x cols complex, column-major, rows >= cols)

@@ -4,11 +4,12 @@
 // Gamma keeps only the eigenvalues inside Gamma. With the trapezoid nodes/weights:
 //   S_k = sum_j w_j zeta_j^k Y_j  (Y_j = T(z_j)^{-1} V),    mu_k = V^H S_k,    k < 2M,
 //   H = [mu_{a+b}],  H< = [mu_{a+b+1}]  (a, b < M; LM x LM, column-major).
-// moments_kernel: one thread per entry (i, l) of the n x L block reads Y_j(i, l) once for
-// every point j (ascending) and keeps the K = 2M complex accumulators in registers; the
-// coefficients c_jk = w_j zeta_j^k sit in shared memory. Arithmetic is FP64 (1.75 FMA/clk/SM
-// on this part), so with 2M*4 FMAs per 16 bytes read the kernel is bound by FP64 issue,
-// not by HBM.
+// moments_df_kernel (complex64 factors, Y in double-float pairs): one thread per entry (i, l) of the n x L block reads
+// Y_j(i, l) once for every point j (ascending) and keeps the K = 2M accumulators in registers; the coefficients
+// c_jk = w_j zeta_j^k sit in shared memory. Bound by FP32 issue.
+// moments_oz_kernel (FP64, up to 192 points): exact digit products on the tensor core, below.
+// moments_kernel and moments_kernel_generic (more points): as the first, in FP64 (1.75 FMA/clk/SM on this part, so with
+// 2M*4 FMAs per 16 bytes read bound by FP64 issue, not by HBM).
 // mu_k = V^H S_k is a product of gemm.cu, split over the rows with a fixed-order reduction (no
 // atomics), so results do not depend on scheduling.
 #include <algorithm>
@@ -65,7 +66,8 @@ __global__ void __launch_bounds__(256) moments_kernel_generic(int64_t nl, int N,
 // A warp takes 8 columns: its B fragments come straight from global memory (lane: column lane / 4,
 // nodes lane % 4 and + 4 of each 8; the column's exponent from a first pass over it, the digits from a
 // second that hits L1), the coefficients' digits are built once per CTA in the fragments' order in shared
-// memory. Columns with a non-finite entry or an extreme exponent take FP64 sums as moments_kernel does.
+// memory. Columns with a non-finite entry or an extreme exponent take FP64 sums as moments_kernel does, and so does
+// every result that the guard (oz.cuh) finds too small for the digits.
 // n L = 524288, N = 64, K = 16: 0.486 ms (FP64 FMAs: 3.56, at the FP64 pipe's rate; HBM alone: 0.10). Error
 // against a 113-bit sum: 4.7e-17 (N <= 64) and 8.3e-17 (N = 192) of the result's norm, FP64 FMAs 2.7e-16 to
 // 6.7e-16. What bounds it: issue (the digits' bytes and 72 MMAs per 8 nodes), not the tensor pipe.
@@ -80,12 +82,12 @@ __global__ void __launch_bounds__(256, 2)
     moments_oz_kernel(int64_t nl, int N, int K, int nch, const zd* __restrict__ coef, const zd* __restrict__ Y,
                       zd* __restrict__ Sout) {
     using namespace oz;
-    extern __shared__ uint4 afrag[];  // [chunk][MT][KC][S][32 lanes]
-    __shared__ int ea[8 * MT], bad;
+    extern __shared__ uint4 afrag[];  // [chunk][MT][KC][S][32 lanes], then the guard's [chunk][KC][32 lanes]
+    __shared__ int ea[8 * MT], bad, guarded;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int kbase = blockIdx.y * 8 * MT;
     auto cval = [&](int j, int k) { return j < N && k < K ? coef[j + (int64_t)N * k] : mk(0.0, 0.0); };
-    if (tid == 0) bad = 0;
+    if (tid == 0) bad = guarded = 0;
     if (tid < 8 * MT) ea[tid] = 0;
     __syncthreads();
     for (int e = tid; e < N * 8 * MT; e += blockDim.x) {
@@ -96,7 +98,7 @@ __global__ void __launch_bounds__(256, 2)
     __syncthreads();
     if (tid < 8 * MT) {
         if (ea[tid] != 0 && (ea[tid] < EXP_LO || ea[tid] > EXP_HI)) bad = 1;
-        if (ea[tid] == 0) ea[tid] = 1023;
+        if (ea[tid] == 0) ea[tid] = E_ZERO;
     }
     __syncthreads();
     const bool slow_all = bad != 0;
@@ -112,8 +114,18 @@ __global__ void __launch_bounds__(256, 2)
 #pragma unroll
             for (int t = 0; t < S; ++t) f[t * FRAG] = digits2(p, q, S - 1 - t);  // the highest digit first
         }
+        // the guard's leading bits: rows 0 .. 7 the first tile of 8 moments, rows 8 .. 15 the second. With every
+        // coefficient at least 2/64 of its row's scale it is met, since a column's largest entry has 32/64 of its own
+        for (int e = tid; e < nch * KC * 32 * 4; e += blockDim.x) {
+            const int w = e & 3, l = (e >> 2) & 31, kc = (e >> 7) % KC, ch = (e >> 7) / KC;
+            const int k = l / 4 + ((w & 1) ? 8 : 0), j = ch * CH + kc * 8 + (l & 3) + ((w & 2) ? 4 : 0);
+            const unsigned f = k < 8 * MT ? lead(cval(j, kbase + k), ea[k]) : 0u;
+            reinterpret_cast<unsigned*>(afrag + (size_t)nch * MT * KC * S * 32)[e] = lead2(f);
+            if (f < 2 && k < 8 * MT && j < N && ea[k] != E_ZERO) guarded = 1;
+        }
     }
     __syncthreads();
+    const bool guard = guarded != 0;
     const int64_t tiles = (nl + 7) / 8;
     for (int64_t tile = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; tile < tiles;
          tile += (int64_t)gridDim.x * (blockDim.x >> 5)) {
@@ -140,8 +152,9 @@ __global__ void __launch_bounds__(256, 2)
             }
             continue;
         }
-        if (E == 0) E = 1023;
+        if (E == 0) E = E_ZERO;
         double out[MT][4];
+        float G[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // the guard of both tiles over all nodes
         for (int ch = 0; ch < nch; ++ch) {
             float D[MT][S][4];
 #pragma unroll
@@ -152,11 +165,13 @@ __global__ void __launch_bounds__(256, 2)
                     for (int q = 0; q < 4; ++q) D[m][t][q] = 0.0f;
             const int kcs = min(KC, (N - ch * CH + 7) / 8);
             const uint4* af = afrag + (size_t)ch * MT * KC * S * 32 + lane;
+            const uint4* gf = afrag + (size_t)nch * MT * KC * S * 32 + lane;
 #pragma unroll 1
             for (int kc = 0; kc < kcs; ++kc) {
                 const int j = ch * CH + kc * 8 + jl;
                 const zd y0 = in && j < N ? yc[(int64_t)j * nl] : mk(0.0, 0.0);
                 const zd y1 = in && j + 4 < N ? yc[(int64_t)(j + 4) * nl] : mk(0.0, 0.0);
+                if (guard) mma16816(G, gf[(size_t)(ch * KC + kc) * 32], lead2(lead(y0, E)), lead2(lead(y1, E)));
                 const unsigned long long r0 = fixed62(y0.re, E), i0 = fixed62(y0.im, E);
                 const unsigned long long r1 = fixed62(y1.re, E), i1 = fixed62(y1.im, E);
                 unsigned b0[S], b1[S];
@@ -184,6 +199,21 @@ __global__ void __launch_bounds__(256, 2)
                     out[m][q] = ch == 0 ? sv : out[m][q] + sv;
                 }
         }
+        if (guard) {
+#pragma unroll
+            for (int m = 0; m < MT; ++m)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int Eb = __shfl_sync(0xffffffffu, E, 4 * (2 * (lane & 3) + q));
+                    const bool weak = G[2 * m + q] < GUARD && ea[8 * m + (lane >> 2)] != E_ZERO && Eb != E_ZERO;
+                    const unsigned todo = __ballot_sync(0xffffffffu, weak);
+                    if (todo) {
+                        const zd s = fp64_sums(todo, N, coef + (int64_t)N * (kbase + 8 * m), N, 1, false,
+                                               Y + e0 + q, 2, nl);
+                        if (weak) out[m][q] = s.re, out[m][2 + q] = s.im;
+                    }
+                }
+        }
 #pragma unroll
         for (int m = 0; m < MT; ++m) {
             const int k = kbase + 8 * m + (lane >> 2);
@@ -200,7 +230,7 @@ __global__ void __launch_bounds__(256, 2)
 template <int MT>
 static int launch_moments_oz(int64_t nl, int N, int K, const zd* coef, const zd* Y, zd* S, cudaStream_t st) {
     const int nch = ceil_div(N, oz::CH);
-    const size_t sm = (size_t)nch * MT * oz::KC * oz::S * oz::FRAG * 4;
+    const size_t sm = (size_t)nch * oz::KC * (MT * oz::S + 1) * oz::FRAG * 4;
     static const int sms = [] {
         int dev = 0, v = 0;
         cudaGetDevice(&dev);
@@ -208,7 +238,7 @@ static int launch_moments_oz(int64_t nl, int N, int K, const zd* coef, const zd*
         return v > 0 ? v : 152;
     }();
     NEP_CUDA(allow_max_dynamic_smem(moments_oz_kernel<MT>));
-    const int gy = ceil_div(K, 8 * MT), per = sm <= 100 * 1024 ? 2 : 1;
+    const int gy = ceil_div(K, 8 * MT), per = sm <= 112 * 1024 ? 2 : 1;
     const int gx = (int)std::min<int64_t>((nl + 63) / 64, std::max(1, per * sms / gy));
     moments_oz_kernel<MT><<<dim3(gx, gy), 256, sm, st>>>(nl, N, K, nch, coef, Y, S);
     NEP_CHECK_LAUNCH();

@@ -56,6 +56,25 @@ def test_dense_products(bnd, n, P, nv, s):
     assert (np.abs(got - ref) <= 4 * (n + P + 4) * EPS * size).all()
 
 
+@pytest.mark.parametrize("n,L,N,K", [(1, 1, 2, 1), (37, 3, 7, 3), (64, 8, 64, 16), (50, 3, 65, 9), (33, 2, 192, 17)])
+@pytest.mark.parametrize("s", [1e3, 1e6, 1e10, 1e60])
+def test_moments(bnd, n, L, N, K, s):
+    """Coefficients scaled by d over the nodes and Y by 1 / d, each column of Y with its own d."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(n * N + K)
+    nl = n * L
+    C, Y = _cplx(rng, K, N), _cplx(rng, N, nl)
+    d = _scales(rng, N, s)
+    C *= d[None]
+    Y[:, ::2] /= d[:, None]
+    Y[:, 1::3] *= 10.0 ** rng.uniform(-12, 0, (N, Y[:, 1::3].shape[1]))
+    S = torch.empty(K * nl * 2, dtype=torch.float64, device="cuda")
+    bnd.moments(n, L, N, K, _dev(torch, C.T), torch.from_numpy(Y.view(np.float64).reshape(-1).copy()).cuda(), S)
+    out = S.cpu().numpy().view(np.complex128).reshape(K, nl)
+    ref = C.astype(np.clongdouble) @ Y.astype(np.clongdouble)
+    assert (np.abs(out - ref) <= 4 * N * EPS * (np.abs(C) @ np.abs(Y))).all()
+
+
 @pytest.mark.parametrize("zeros", [False, True])
 def test_subnormal_columns(bnd, zeros):
     """A column all of whose entries are subnormal is not a zero column; beside exactly zero ones or not."""
