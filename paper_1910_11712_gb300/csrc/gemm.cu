@@ -1,12 +1,15 @@
-// Dense complex FP64 products C = op(A) B (column-major, op in {A, A^H}) of the extraction, on the tensor core by
-// exact 8-bit digit products (oz.cuh).
+// Dense complex FP64 products C = op(A) B (column-major, op in {A, A^H}) of the extraction: on the tensor core by
+// exact 8-bit digit products (oz.cuh), small ones in FP64 FMAs.
 //
-// A CTA of 8 warps computes a 32 x 32 tile, K in blocks of 64: the exponents of the tile's rows and
+// Digit products: a CTA of 8 warps computes a 32 x 32 tile, K in blocks of 64: the exponents of the tile's rows and
 // columns over the block, then twice 32 terms as digits in the MMA fragments' order in shared memory (A 64 KB, B 32 KB)
 // and 36 x 4 MMA steps per warp and 8 x 8 subtile (a warp takes 8 rows by 16 columns); the exact sums of a block
 // become FP64 once. Long K splits over CTAs into a workspace reduced in a fixed order, so results never depend
 // on scheduling. Blocks with a non-finite entry or an extreme exponent are summed in FP64 FMAs, and so are the
 // terms of a block for every result that the guard (oz.cuh) finds too small for the digits.
+#include <algorithm>
+#include <cmath>
+
 #include "oz.cuh"
 
 namespace nep {
@@ -181,6 +184,66 @@ __global__ void __launch_bounds__(256, 2)
         }
 }
 
+// ------------------------------------------------------------------ small products, in FP64 FMAs
+// A CTA computes a BM x BN tile with (BM/TM) x (BN/TN) threads of TM x TN outputs, K in steps of GK through shared
+// memory; K splits over CTAs into a workspace reduced in a fixed order. The FP64 units bound it (about two FMAs per
+// clock per SM), so the launcher picks the tile shape and the split that waste the least of them: padding beyond M
+// and N and SMs left idle or doubly loaded.
+constexpr int GK = 8;
+template <int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__((BM / TM) * (BN / TN))
+    zgemm_kernel(int M, int N, int K, int opA, const zd* __restrict__ A, int lda, const zd* __restrict__ B, int ldb,
+                 zd* __restrict__ C, int ldc, int kchunk, int64_t part_stride) {
+    constexpr int TX = BM / TM, TY = BN / TN, NT = TX * TY;
+    __shared__ zd As[GK][BM + 1];
+    __shared__ zd Bs[GK][BN + 1];
+    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
+    const int kb = blockIdx.z * kchunk, ke = min(K, kb + kchunk);
+    zd acc[TM][TN];
+#pragma unroll
+    for (int a = 0; a < TM; ++a)
+#pragma unroll
+        for (int b = 0; b < TN; ++b) acc[a][b] = mk(0.0, 0.0);
+    for (int k0 = kb; k0 < ke; k0 += GK) {
+        // loads run along the contiguous index of each operand
+        for (int t = threadIdx.x; t < GK * BM; t += NT) {
+            const int kk = opA == 0 ? t / BM : t % GK, mm = opA == 0 ? t % BM : t / GK;
+            const int gm = m0 + mm, gk = k0 + kk;
+            zd v = mk(0.0, 0.0);
+            if (gm < M && gk < ke) v = opA == 0 ? A[gm + (int64_t)lda * gk] : conj(A[gk + (int64_t)lda * gm]);
+            As[kk][mm] = v;
+        }
+        for (int t = threadIdx.x; t < GK * BN; t += NT) {
+            const int kk = t % GK, nn = t / GK;
+            const int gn = n0 + nn, gk = k0 + kk;
+            Bs[kk][nn] = (gn < N && gk < ke) ? B[gk + (int64_t)ldb * gn] : mk(0.0, 0.0);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < GK; ++kk) {
+            zd av[TM], bv[TN];
+#pragma unroll
+            for (int a = 0; a < TM; ++a) av[a] = As[kk][tx + TX * a];
+#pragma unroll
+            for (int b = 0; b < TN; ++b) bv[b] = Bs[kk][ty + TY * b];
+#pragma unroll
+            for (int a = 0; a < TM; ++a)
+#pragma unroll
+                for (int b = 0; b < TN; ++b) acc[a][b] = fma_(acc[a][b], av[a], bv[b]);
+        }
+        __syncthreads();
+    }
+    zd* Cz = C + (int64_t)blockIdx.z * part_stride;
+#pragma unroll
+    for (int a = 0; a < TM; ++a)
+#pragma unroll
+        for (int b = 0; b < TN; ++b) {
+            const int gm = m0 + tx + TX * a, gn = n0 + ty + TY * b;
+            if (gm < M && gn < N) Cz[gm + (int64_t)ldc * gn] = acc[a][b];
+        }
+}
+
 __global__ void zgemm_reduce_kernel(int M, int N, int splits, const zd* __restrict__ part, zd* __restrict__ C, int ldc) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (int64_t)M * N) return;
@@ -188,6 +251,75 @@ __global__ void zgemm_reduce_kernel(int M, int N, int splits, const zd* __restri
     zd acc = mk(0.0, 0.0);
     for (int z = 0; z < splits; ++z) acc = acc + part[(int64_t)z * M * N + t];
     C[m + (int64_t)ldc * n] = acc;
+}
+
+namespace {
+struct GemmShape {
+    int bm, bn;
+};
+constexpr GemmShape kGemmShapes[] = {{64, 32}, {64, 24}, {32, 32}, {32, 24}, {24, 24}, {32, 16}, {24, 16}};
+
+template <int BM, int BN, int TM, int TN>
+void zgemm_launch(dim3 grid, int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int ldb, zd* C, int ldc,
+                  int kchunk, int64_t part_stride, cudaStream_t st) {
+    zgemm_kernel<BM, BN, TM, TN><<<grid, (BM / TM) * (BN / TN), 0, st>>>(M, N, K, opA, A, lda, B, ldb, C, ldc, kchunk,
+                                                                       part_stride);
+}
+}  // namespace
+
+static int zgemm_fma(int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int ldb, zd* C, int ldc, zd* part,
+                     int room, int sms, cudaStream_t st) {
+    // score = useful fraction of the padded tiles x SM load balance (mean over max CTAs per SM),
+    // a split costing a little for its partial sums and their reduction
+    int best = 0, best_splits = 1;
+    double best_score = -1.0;
+    for (int c = 0; c < (int)(sizeof(kGemmShapes) / sizeof(kGemmShapes[0])); ++c) {
+        const int bm = kGemmShapes[c].bm, bn = kGemmShapes[c].bn;
+        const int64_t tiles = (int64_t)ceil_div(M, bm) * ceil_div(N, bn);
+        const double pad = (double)M * N / ((double)ceil_div(M, bm) * bm * ceil_div(N, bn) * bn);
+        const int max_splits = std::max(1, std::min(K / (2 * GK), room));
+        for (int sp = 1; sp <= max_splits; ++sp) {
+            const double ctas = (double)tiles * sp;
+            const double waves = std::ceil(ctas / sms);
+            const double score = pad * (ctas / sms) / waves * (sp > 1 ? 0.97 : 1.0);
+            if (score > best_score + 1e-9) {
+                best_score = score;
+                best = c;
+                best_splits = sp;
+            }
+        }
+    }
+    const int bm = kGemmShapes[best].bm, bn = kGemmShapes[best].bn;
+    const int kchunk = ceil_div(ceil_div(K, best_splits), GK) * GK;
+    const int splits = std::max(1, ceil_div(K, kchunk));
+    dim3 grid(ceil_div(M, bm), ceil_div(N, bn), splits);
+    zd* out = splits == 1 ? C : part;
+    const int ldo = splits == 1 ? ldc : M;
+    const int64_t ps = splits == 1 ? 0 : (int64_t)M * N;
+    switch (best) {
+        case 0: zgemm_launch<64, 32, 4, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
+        case 1: zgemm_launch<64, 24, 4, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
+        case 2: zgemm_launch<32, 32, 2, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
+        case 3: zgemm_launch<32, 24, 2, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
+        case 4: zgemm_launch<24, 24, 2, 2>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
+        case 5: zgemm_launch<32, 16, 2, 1>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
+        default: zgemm_launch<24, 16, 2, 1>(grid, M, N, K, opA, A, lda, B, ldb, out, ldo, kchunk, ps, st); break;
+    }
+    NEP_CHECK_LAUNCH();
+    if (splits > 1) {
+        zgemm_reduce_kernel<<<ceil_div((int64_t)M * N, 256), 256, 0, st>>>(M, N, splits, part, C, ldc);
+        NEP_CHECK_LAUNCH();
+    }
+    return NEP_OK;
+}
+
+// FP64 FMAs where the product is small and its K short, or splits to at most 32 terms a CTA: the digits' staging
+// and the guard's sums then cost more than they save. us, digits / FMAs, M x N x K: 64 x 21 x 64 28 / 14, 21 x 21 x 21
+// (triangular factor: a third of it rejected by the guard) 39 / 14, 9409 x 7 x 7 22 / 11, 66 x 66 x 128 31 / 15, 128 x 66 x 128
+// 35 / 22, 96 x 96 x 192 with 192 x 96 x 96 91 / 83; against them 16 x 128 x 64 without room to split 25 / 37,
+// 7 x 7 x 9409 48 / 89, 128 x 128 x 128 twice 100 / 103, 4096 x 66 x 66 81 to 91 / 171.
+static bool zgemm_small(int M, int N, int K, int max_splits) {
+    return (int64_t)M * N * K <= 2000000 && K <= std::min(256, 32 * max_splits);
 }
 
 // C = op(A) B. part: workspace of splits*M*N elements when K is long (nullptr => no split).
@@ -201,6 +333,7 @@ int zgemm(int M, int N, int K, int opA, const zd* A, int lda, const zd* B, int l
         return v > 0 ? v : 152;
     }();
     const int room = part ? std::max(1, (int)std::min<size_t>(64, part_elems / ((size_t)M * N))) : 1;  // splits of K
+    if (zgemm_small(M, N, K, room)) return zgemm_fma(M, N, K, opA, A, lda, B, ldb, C, ldc, room > 1 ? part : nullptr, room, sms, st);
     // blocks of 64 terms over as many CTAs as two per SM allow
     const int tiles = ceil_div(M, TB) * ceil_div(N, TB), blocks = std::max(1, ceil_div(K, oz::CH));
     int splits = std::max(1, std::min(std::min(blocks, room), 2 * sms / tiles));
