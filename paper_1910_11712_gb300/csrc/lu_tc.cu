@@ -759,7 +759,17 @@ static cudaError_t lu_tc_start(int npts, int nsplit, size_t smem, cudaStream_t s
     return cudaLaunchKernelEx(&cfg, lu_tc_kernel, args...);
 }
 
-bool band_lu_tc_can(int kl) { return kl >= NB && lu_tc_smem(kl) <= 227 * 1024; }
+// The panel of kl rows fits the shared memory that a launch may ask for: what a CTA can have less the kernel's
+// static part (kl <= 854; wider bands take lu_wide.cu)
+bool band_lu_tc_can(int kl) {
+    static const size_t room = [] {
+        cudaFuncAttributes a{};
+        const cudaError_t e = cudaFuncGetAttributes(&a, lu_tc_kernel);
+        if (e != cudaSuccess) cudaGetLastError();  // no device: nothing is launched
+        return (size_t)smem_optin_bytes() - (e == cudaSuccess ? a.sharedSizeBytes : 1024);
+    }();
+    return kl >= NB && lu_tc_smem(kl) <= room;
+}
 
 bool band_lu_tc_fits(int kl) { return kl > 64 && band_lu_tc_can(kl); }
 
