@@ -274,9 +274,12 @@ __global__ void __launch_bounds__(512, 1)
     // Pc = cc+kl), the pivot's slot takes the entering row, a(r, k) -= l(r) u(k), U(cc, k) to
     // the band, and the slot of column cc+1 (if this warp holds it) empties for column cc+1+CS.
     // Columns beyond the step's reach (the farthest pivot row so far + ku) are zero in the pivot row: the
-    // complex128 update, bound by the FP64 units, leaves them out (half the window without interchanges:
-    // 64 points at bandwidth 64, n = 4096, 42.8 -> 23.0 ms). The complex64 one, bound by the chain of pivots,
-    // lost more to the test than it saved (3.92 -> 4.41 ms).
+    // complex128 update of windows of more than 32 rows, bound by the FP64 units, leaves them out (half the window
+    // without interchanges: 64 points at bandwidth 64, n = 4096, 42.8 -> 23.0 ms; bandwidth 40, n = 1600,
+    // 16.8 -> 7.0). Narrower windows and complex64, bound by the chain of pivots, lose more to the test than
+    // it saves (complex128, kl = 24, n = 1200: 4.05 ms without, 4.26 with; kl = 5, ku = 60, n = 900: 4.86 and
+    // 5.22; complex64 at bandwidth 64 3.92 and 4.41).
+    constexpr bool LIMIT = !PAIRED && RPL == 2;
     int reach = 0;
     auto run_step = [&](int cc, int Pc, const bool(&ispc)[RPL]) __attribute__((always_inline)) {
         const int e = cc % RING, lb = cc % 3;
@@ -335,7 +338,7 @@ __global__ void __launch_bounds__(512, 1)
             for (int q = 0; q < RPL; ++q) lqc[q] = vr[q] ? lvec[lb][lane + 32 * q] : mk<T>(0, 0);
 #pragma unroll
             for (int p = 0; p < CPW; ++p) {
-                if (toff(p, cc) > reach - cc) continue;
+                if (LIMIT && toff(p, cc) > reach - cc) continue;
                 const cx<T> u = xrow[warp][p];
 #pragma unroll
                 for (int q = 0; q < RPL; ++q) a[q][p] = fms(a[q][p], lqc[q], u);
@@ -399,7 +402,7 @@ __global__ void __launch_bounds__(512, 1)
         }
         const int cb = c % 3, re = c + kl;
         const int P = piv_s[cb];
-        if constexpr (!PAIRED) reach = max(reach, P + ku);
+        if constexpr (LIMIT) reach = max(reach, P + ku);
         bool isp[RPL];
 #pragma unroll
         for (int q = 0; q < RPL; ++q) {
