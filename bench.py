@@ -160,14 +160,6 @@ def solve_bytes(n, kl, ku, L, npts, esz):
 SOLVE_TRAFFIC = {("delay2d_s64", "mixed"): (386.8 + 50.9) * 1e6}
 
 
-def solve_kernel(split, npts, L, mixed):
-    """Name of the kernel(s) that the library takes for a solve of this shape (csrc/band_lu.cu)."""
-    narrow = split.kl + 1 <= 288 and split.kl + split.ku + 1 <= 288
-    if not mixed or (narrow and (L == 1 or (npts * L <= 1024 and split.kl + split.ku <= 144))):
-        return "band_subst_kernel"
-    return "band_sweep_kernel x2" if narrow else "band_solve_blocked_kernel"
-
-
 def fp32_alu_peak_tflops(sm_mhz):
     """152 SMs x 128 FP32 lanes x 2 flops (FMA) x clock."""
     return 152 * 128 * 2 * sm_mhz * 1e6 / 1e12
@@ -765,9 +757,9 @@ def main():
                           "band_mb_per_step": round(p.N * p.n * split.ldab * esz / 1e6),
                           "streams": S, "concurrency": f"{S} independent plans on {S} non-blocking streams, one "
                           "host thread each; every step a full pass of its own"},
-            "roofline": {"kernel": solve_kernel(split, p.N, p.L, mixed) +
+            "roofline": {"kernel": binding.band_solve_kernel(split, p.N, prec, p.L) +
                                    " (forward + backward banded substitution, "
-                                   f"{p.N} points x {p.L} right-hand sides in one launch)",
+                                   f"{p.N} points x {p.L} right-hand sides)",
                          "bound": "hbm", "achieved": s_bytes / (solve_ms * 1e-3) / 1e9, "peak": hbm,
                          "unit": "GB/s", "frac": s_bytes / (solve_ms * 1e-3) / 1e9 / hbm,
                          "traffic": SOLVE_TRAFFIC.get((args.workload, args.precision)),

@@ -547,6 +547,9 @@ int nep_band_factor(nep_split_t h, int32_t npts, int32_t precision, void *ab_dev
  * builds it once and calls nep_band_solve_cols instead. */
 int nep_band_solve(nep_split_t h, int32_t npts, int32_t precision, const void *ab_dev, const int32_t *ipiv_dev,
                    int32_t L, void *B_dev, void *stream);
+/* Name of the kernel that nep_band_solve takes for npts points and L right-hand sides each: "band_subst_kernel",
+ * "band_sweep_kernel", "band_solve_blocked_kernel" or "band_solve_kernel"; NULL for bad arguments. */
+const char *nep_band_solve_kernel(nep_split_t h, int32_t npts, int32_t precision, int32_t L);
 /* Conjugate-transpose solve T(z_j)^* X_j = B_j with the factors of nep_band_factor, in place on
  * B (npts x n x L, column-major per point, element type of the precision): U^* forward, then
  * the L factors' conjugate transposes and the interchanges in reverse order (the factorisation

@@ -130,6 +130,7 @@ SIGNATURES = {
                                     ctypes.POINTER(ctypes.POINTER(c_int32)), ctypes.POINTER(P_double)]),
     "nep_assemble_band": (c_int32, [c_void_p, c_int32, c_void_p, c_int32, c_void_p, c_void_p, c_void_p]),
     "nep_band_factor": (c_int32, [c_void_p, c_int32, c_int32, c_void_p, c_void_p, c_void_p, c_void_p]),
+    "nep_band_solve_kernel": (ctypes.c_char_p, [c_void_p, c_int32, c_int32, c_int32]),
     "nep_band_solve": (c_int32, [c_void_p, c_int32, c_int32, c_void_p, c_void_p, c_int32, c_void_p, c_void_p]),
     "nep_band_transpose_u": (c_int32, [c_void_p, c_int32, c_int32, c_void_p, c_void_p, c_void_p]),
     "nep_band_solve_cols": (c_int32, [c_void_p, c_int32, c_int32, c_void_p, c_void_p, c_void_p, c_int32, c_void_p,
@@ -510,6 +511,12 @@ def band_factor(split, npts, precision, ab_dev, ipiv_dev, info_dev, stream=0):
 
 def band_solve(split, npts, precision, ab_dev, ipiv_dev, L, B_dev, stream=0):
     check(load().nep_band_solve(split.handle, npts, precision, ptr(ab_dev), ptr(ipiv_dev), L, ptr(B_dev), stream))
+
+
+def band_solve_kernel(split, npts, precision, L):
+    """Name of the kernel that band_solve takes for this shape."""
+    name = load().nep_band_solve_kernel(split.handle, npts, precision, L)
+    return name.decode() if name else None
 
 
 def band_transpose_u(split, npts, precision, ab_dev, ut_dev, stream=0):

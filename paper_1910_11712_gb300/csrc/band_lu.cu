@@ -436,6 +436,25 @@ bool band_subst_chosen(int kl, int ku, int npts, int L) {
 template bool band_subst_chosen<float>(int, int, int, int);
 template bool band_subst_chosen<double>(int, int, int, int);
 
+static bool solve_unblocked() {
+    static const bool on = [] {
+        const char* e = std::getenv("NEP_SOLVE_UNBLOCKED");
+        return e && e[0] == '1';
+    }();
+    return on;
+}
+
+// The kernel that launch_band_solve takes.
+template <typename T>
+const char* band_solve_kernel_name(int kl, int ku, int npts, int L) {
+    if (band_subst_chosen<T>(kl, ku, npts, L)) return "band_subst_kernel";
+    if (sizeof(T) == 4 && band_sweeps_fit(kl, ku)) return "band_sweep_kernel";
+    if (sizeof(T) == 4 && !solve_unblocked() && band_solve_blocked_rhs(kl, ku, npts, L) > 0) return "band_solve_blocked_kernel";
+    return "band_solve_kernel";
+}
+template const char* band_solve_kernel_name<float>(int, int, int, int);
+template const char* band_solve_kernel_name<double>(int, int, int, int);
+
 template <typename T>
 int launch_band_solve(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>* ut, const int* ipiv, int L, cx<T>* B,
                       const int* active, cudaStream_t st, int rh_force) {
@@ -448,11 +467,7 @@ int launch_band_solve(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>*
         if (band_sweeps_fit(s.kl, s.ku)) return band_sweeps<T>(s, npts, ab, ut, ipiv, L, B, active, st, rh_force);
     // complex64 factors: blocked substitution (NEP_SOLVE_UNBLOCKED=1 keeps the per-step sweeps below)
     if constexpr (sizeof(T) == 4) {
-        static const bool unblocked = [] {
-            const char* e = std::getenv("NEP_SOLVE_UNBLOCKED");
-            return e && e[0] == '1';
-        }();
-        if (!unblocked) {
+        if (!solve_unblocked()) {
             const int rc = launch_band_solve_blocked(s, npts, ab, ipiv, L, B, active, st);
             if (rc != NEP_ERR_UNSUPPORTED) return rc;
         }

@@ -2188,6 +2188,13 @@ extern "C" int nep_band_solve(nep_split_t h, int32_t npts, int32_t precision, co
                : band_solve_step<double>(s, npts, (const zd*)ab_dev, ipiv_dev, L, (zd*)B_dev, (cudaStream_t)stream);
 }
 
+extern "C" const char* nep_band_solve_kernel(nep_split_t h, int32_t npts, int32_t precision, int32_t L) {
+    if (!h || npts < 1 || L < 1) return nullptr;
+    if (precision == NEP_PREC_MIXED) return band_solve_kernel_name<float>(h->kl, h->ku, npts, L);
+    if (precision == NEP_PREC_FP64) return band_solve_kernel_name<double>(h->kl, h->ku, npts, L);
+    return nullptr;
+}
+
 extern "C" int nep_band_solve_adjoint(nep_split_t h, int32_t npts, int32_t precision, const void* ab_dev,
                                       const int32_t* ipiv_dev, int32_t L, void* B_dev, void* stream) {
     if (!h || !ab_dev || !ipiv_dev || !B_dev || npts < 0 || L < 0) {

@@ -302,6 +302,8 @@ template <typename T>
 int band_subst_batch(int rt, size_t smem, int count, int maxL, const PointDesc* pd, cudaStream_t st);
 template <typename T>
 bool band_subst_chosen(int kl, int ku, int npts, int L);  // band_lu.cu: this solve takes it
+template <typename T>
+const char* band_solve_kernel_name(int kl, int ku, int npts, int L);
 // Narrow-band substitution sweeps (register windows of kl+1 and kl+ku+1 rows, up to 288).
 inline bool band_sweeps_fit(int kl, int ku) { return kl >= 1 && kl + 1 <= 288 && kl + ku + 1 <= 288; }
 // band_solve_blocked.cu: the blocked substitution for complex64 factors of wider bands (NB-step
