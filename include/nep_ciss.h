@@ -541,10 +541,10 @@ int nep_assemble_band(nep_split_t h, int32_t npts, const double *F_dev, int32_t 
 int nep_band_factor(nep_split_t h, int32_t npts, int32_t precision, void *ab_dev, int32_t *ipiv_dev,
                     int32_t *info_dev, void *stream);
 /* Kernel (b): solve T(z_j) X_j = B_j with the factors, in place on B (npts x n x L,
- * column-major per point, element type of the precision). For narrow bands (kl+1 <= 288 and
- * kl+ku+1 <= 288) in complex64 with many right-hand sides the call builds the column copy of U
- * (nep_band_transpose_u) in a temporary of its own; a caller solving repeatedly with the same factors
- * builds it once and calls nep_band_solve_cols instead. */
+ * column-major per point, element type of the precision). Where nep_band_solve_kernel names
+ * "band_sweep_kernel" the call builds the column copy of U (nep_band_transpose_u) in a temporary of
+ * its own; a caller solving repeatedly with the same factors builds it once and calls
+ * nep_band_solve_cols instead. */
 int nep_band_solve(nep_split_t h, int32_t npts, int32_t precision, const void *ab_dev, const int32_t *ipiv_dev,
                    int32_t L, void *B_dev, void *stream);
 /* Name of the kernel that nep_band_solve takes for npts points and L right-hand sides each: "band_subst_kernel",

@@ -416,21 +416,44 @@ __global__ void __launch_bounds__(512)
     }
 }
 
-// Whether a solve takes the blocked substitution (band_subst.cuh) rather than the register-window sweeps.
-// Its chain from step to step is shorter (bandwidth 64: 114 ns against 162 with one right-hand side) and it
-// needs no column copy of U, but its arithmetic costs more instructions per right-hand side: measured, ms
-// per solve, sweeps (without the copy of U) against substitution, points x right-hand sides, both with
-// backward windows of kl + ku rows:
-//   complex64, bandwidth 64: 1 x 1 .661 / .463, 9 x 4 .680 / .549, 64 x 16 .820 / .673, 128 x 16 1.11 / 2.34;
-//   bandwidth 24: 32 x 8 .090 / .065;
-//   bandwidth 40: 64 x 16 .324 / .238, 128 x 32 .562 / .735; bandwidth 97: 64 x 16 2.40 / 2.62;
-//   bandwidth 128: 1 x 1 3.05 / 2.23;
-//   complex128, bandwidth 64: 9 x 1 10.6 / 3.6, 64 x 16 10.7 / 10.5; bandwidth 40: 128 x 32 11.1 / 9.1;
-//   bandwidth 24: 64 x 32 1.25 / 1.27; bandwidth 200 (against one step at a time): 1 x 1 15.4 / 3.9, 64 x 16 24.9 / 19.5.
+// Whether a solve takes the blocked substitution (band_subst.cuh) rather than the register-window sweeps
+// (band_sweep.cuh; both give the same bits). Its chain from step to step is shorter and it needs no column copy
+// of U, but its arithmetic costs more instructions per right-hand side. Measured, ms per solve, sweeps (the copy of U
+// made beforehand; it adds 5 to 20 %) / substitution, without interchanges and, after the semicolon, with
+// interchanges at every step; points x right-hand sides:
+//   complex64, kl = ku = 10, n = 1000: 64 x 8 .105 / .097; .171 / .187, 64 x 16 .129 / .121; .206 / .210, 96 x 16
+//     .167 / .232; .245 / .407;
+//   24, n = 1200: 64 x 16 .159 / .154; .301 / .269, 96 x 16 .202 / .302; .347 / .551;
+//   40, n = 1600: 64 x 16 .320 / .218; .551 / .400, 96 x 16 .394 / .428; .639 / .807, 128 x 32 .564 / .850; .970 / 1.62;
+//   64, n = 2048: 64 x 16 .412 / .313; .759 / .549, 96 x 16 .502 / .613; .896 / 1.10, 128 x 32 .736 / 1.22; 1.45 / 2.20;
+//   72, n = 2500: 64 x 16 .529 / .392; .938 / .680, 96 x 16 .671 / .767; 1.12 / 1.36;
+//   complex128, 10: 64 x 16 1.06 / .871; 1.12 / 1.02, 96 x 16 1.72 / 1.74; 1.74 / 2.04; 16: 64 x 32 2.07 / 1.99; 2.69 / 2.38;
+//   24: 64 x 16 1.27 / 1.17; 1.65 / 1.67, 64 x 32 2.07 / 2.23; 2.69 / 3.05, 96 x 32 3.08 / 4.43; 4.10 / 6.09;
+//   40: 64 x 16 2.47 / 1.89; 3.15 / 2.61, 64 x 32 4.32 / 3.70; 5.22 / 4.92, 96 x 32 6.75 / 7.37; 8.78 / 9.81,
+//     128 x 32 9.66 / 7.38; 11.9 / 9.82;
+//   64: 64 x 16 2.99 / 3.24; 5.22 / 4.77, 96 x 32 8.45 / 12.8; 15.3 / 17.8, 128 x 32 12.1 / 12.8; 19.7 / 17.8;
+//   80, n = 1500: 64 x 32 5.57 / 5.17; 8.42 / 9.50, 96 x 32 8.60 / 10.3; 13.0 / 19.0.
+// complex64: up to N L = 1024 and kl + ku <= 144 (and one right-hand side always). complex128: unless its CTAs of 16
+// columns leave a last wave mostly empty (96 x 32: 192 CTAs on 152 SMs), or, beyond N L = 1024, the sweeps' windows
+// take one register a lane (up to 31 rows, kl > 16 or the wider backward window too).
 template <typename T>
 bool band_subst_chosen(int kl, int ku, int npts, int L) {
     if (npts <= 0 || L <= 0) return false;
-    if (sizeof(T) == 4 && !(band_sweeps_fit(kl, ku) && (L == 1 || ((int64_t)npts * L <= 1024 && kl + ku <= 144)))) return false;
+    const bool fit = band_sweeps_fit(kl, ku);
+    const int64_t chains = (int64_t)npts * L;
+    if (sizeof(T) == 4) {
+        if (!(fit && (L == 1 || (chains <= 1024 && kl + ku <= 144)))) return false;
+    } else if (fit && chains > 1024) {
+        static const int sms = [] {
+            int dev = 0, v = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+            return v > 0 ? v : 152;
+        }();
+        const int64_t ctas = (int64_t)npts * ((L + 15) / 16), waves = (ctas + sms - 1) / sms;
+        if (ctas > sms && 10 * waves * sms >= 14 * ctas) return false;
+        if (kl < 32 && ku < 32 && (kl > 16 || kl + ku < 32)) return false;
+    }
     return band_subst_rt<T>(kl, ku, npts, L) > 0;
 }
 template bool band_subst_chosen<float>(int, int, int, int);
@@ -448,7 +471,7 @@ static bool solve_unblocked() {
 template <typename T>
 const char* band_solve_kernel_name(int kl, int ku, int npts, int L) {
     if (band_subst_chosen<T>(kl, ku, npts, L)) return "band_subst_kernel";
-    if (sizeof(T) == 4 && band_sweeps_fit(kl, ku)) return "band_sweep_kernel";
+    if (band_sweeps_fit(kl, ku)) return "band_sweep_kernel";
     if (sizeof(T) == 4 && !solve_unblocked() && band_solve_blocked_rhs(kl, ku, npts, L) > 0) return "band_solve_blocked_kernel";
     return "band_solve_kernel";
 }
@@ -463,8 +486,7 @@ int launch_band_solve(const SplitDev& s, int npts, const cx<T>* ab, const cx<T>*
     // blocked substitution, or register windows for narrow bands (kl+1 <= 288 and kv+1 <= 288 rows): two sweeps with
     // slot-ordered coefficients
     if (band_subst_chosen<T>(s.kl, s.ku, npts, L)) return band_subst<T>(s, npts, ab, ipiv, L, B, active, st, rh_force);
-    if constexpr (sizeof(T) == 4)
-        if (band_sweeps_fit(s.kl, s.ku)) return band_sweeps<T>(s, npts, ab, ut, ipiv, L, B, active, st, rh_force);
+    if (band_sweeps_fit(s.kl, s.ku)) return band_sweeps<T>(s, npts, ab, ut, ipiv, L, B, active, st, rh_force);
     // complex64 factors: blocked substitution (NEP_SOLVE_UNBLOCKED=1 keeps the per-step sweeps below)
     if constexpr (sizeof(T) == 4) {
         if (!solve_unblocked()) {

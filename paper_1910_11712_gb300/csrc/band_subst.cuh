@@ -35,7 +35,7 @@
 //
 // What bounds it: the chain from block to block (two barriers' worth of shuffles and 16 dependent
 // multiply-adds, 1.8 us a block at bandwidth 64) up to one CTA per SM; beyond that the staging and
-// shared-memory instructions of the update, which is why many columns of complex64 keep the sweeps.
+// shared-memory instructions of the update, which is why many columns keep the sweeps (band_subst_chosen).
 // n = 4096, bandwidth 64, complex64: one right-hand side 0.461 ms (sweeps .661), 64 points x 16 0.612
 // (.820); complex128: 9 x 1 3.62 ms (10.6), 64 x 16 6.5 (10.7), bandwidth 40 at 128 x 32 7.5 (11.1);
 // bandwidth 200 with interchanges throughout, n = 3000, 16 x 16 9.8 (12.5, one step at a time).

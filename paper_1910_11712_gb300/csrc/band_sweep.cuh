@@ -1,5 +1,6 @@
 // Banded forward/backward substitution sweeps for narrow bands (kernel (b), solve part).
-// Instantiated for complex64 in band_sweep_f.cu.
+// Instantiated once per element type (band_sweep_f.cu, band_sweep_d.cu) so the two compile in
+// parallel.
 #pragma once
 #include <algorithm>
 #include <cstdlib>
@@ -14,7 +15,7 @@ namespace nep {
 // row taking its slot ahead of the step's update. That saves a register a lane and its staged coefficients
 // where the sweep is bound by issue (bandwidth 64, 128 points x 32: 1.66 -> 1.44 ms a solve; bandwidth 128,
 // 128 x 16: 5.06 -> 4.83). With one right-hand side a warp the chain bounds the sweep and the
-// extra select costs 4 %.
+// extra select costs 4 %. The widths 160 to 288 have the same spare register; they were not tried.
 constexpr int kFullWindow = 16;
 template <typename T>
 inline int sweep_shape(int W, int rh) {
@@ -362,8 +363,9 @@ static int sweep_rh(int chains) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         return 4 * (sms > 0 ? sms : 152);
     }();
-    // about one or two warps per sub-partition
-    return chains >= 6 * smsp ? 4 : 2 * chains >= 3 * smsp ? 2 : 1;
+    // about one or two warps per sub-partition; complex128, bound by the FP64 units, takes at least two
+    const int rh = chains >= 6 * smsp ? 4 : 2 * chains >= 3 * smsp ? 2 : 1;
+    return sizeof(T) == 4 ? rh : std::max(rh, 2);
 }
 
 template <typename T, bool BWD, int RH>

@@ -1,12 +1,10 @@
-// Banded substitution sweeps, complex64 (complex128 solves take band_subst.cuh at every bandwidth that the
-// sweeps would), and the column copy of U in both types.
+// Banded substitution sweeps, complex64.
 #include "band_sweep.cuh"
 
 namespace nep {
 template int band_sweeps<float>(const SplitDev&, int, const cx<float>*, const cx<float>*, const int*, int, cx<float>*,
                               const int*, cudaStream_t, int);
 template int band_transpose_u<float>(const SplitDev&, int, const cx<float>*, cx<float>*, cudaStream_t);
-template int band_transpose_u<double>(const SplitDev&, int, const cx<double>*, cx<double>*, cudaStream_t);
 template int band_sweeps_batch<float>(int, int, int, int, int, int, const PointDesc*, cudaStream_t);
 template void sweep_key<float>(int, int, int, int, int*, int*, int*, int*, int);
 }  // namespace nep

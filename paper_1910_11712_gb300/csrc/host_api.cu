@@ -1154,15 +1154,13 @@ static int run_solves_batch(const std::vector<nep_plan*>& ps, cudaStream_t st) {
                 smaxL[key] = std::max(smaxL[key], p->L);
                 continue;
             }
-            if constexpr (sizeof(T) == 4) {
-                if (p->ut) {
-                    int a, u, b, r;
-                    sweep_key<T>(s.kl, s.ku, p->Np, p->L, &a, &u, &b, &r, p->solve_rh);
-                    const auto key = std::make_tuple(a, u, b, r);
-                    for (int j = 0; j < p->Np; ++j) groups[key].push_back(point(p, j, p->D, masked ? p->active : nullptr));
-                    maxL[key] = std::max(maxL[key], p->L);
-                    continue;
-                }
+            if (band_solve_needs_ut<T>(s.kl, s.ku, p->Np, p->L)) {
+                int a, u, b, r;
+                sweep_key<T>(s.kl, s.ku, p->Np, p->L, &a, &u, &b, &r, p->solve_rh);
+                const auto key = std::make_tuple(a, u, b, r);
+                for (int j = 0; j < p->Np; ++j) groups[key].push_back(point(p, j, p->D, masked ? p->active : nullptr));
+                maxL[key] = std::max(maxL[key], p->L);
+                continue;
             }
             NEP_TRY(launch_band_solve<T>(s, p->Np, reinterpret_cast<cx<T>*>(p->ab), nullptr, p->ipiv, p->L,
                                          reinterpret_cast<cx<T>*>(p->D), masked ? p->active : nullptr, st, p->solve_rh));
@@ -1172,13 +1170,12 @@ static int run_solves_batch(const std::vector<nep_plan*>& ps, cudaStream_t st) {
             NEP_TRY(upload(g.second, &pd));
             NEP_TRY(band_subst_batch<T>(g.first.first, ssmem[g.first], (int)g.second.size(), smaxL[g.first], pd, st));
         }
-        if constexpr (sizeof(T) == 4)
-            for (auto& g : groups) {
-                PointDesc* pd = nullptr;
-                NEP_TRY(upload(g.second, &pd));
-                NEP_TRY(band_sweeps_batch<T>(std::get<0>(g.first), std::get<1>(g.first), std::get<2>(g.first),
-                                             std::get<3>(g.first), (int)g.second.size(), maxL[g.first], pd, st));
-            }
+        for (auto& g : groups) {
+            PointDesc* pd = nullptr;
+            NEP_TRY(upload(g.second, &pd));
+            NEP_TRY(band_sweeps_batch<T>(std::get<0>(g.first), std::get<1>(g.first), std::get<2>(g.first),
+                                         std::get<3>(g.first), (int)g.second.size(), maxL[g.first], pd, st));
+        }
         return NEP_OK;
     };
     for (nep_plan* p : ps) NEP_TRY(launch_convert_rhs<T>(p->Np, p->h->n, p->L, p->V, reinterpret_cast<cx<T>*>(p->D), st));
