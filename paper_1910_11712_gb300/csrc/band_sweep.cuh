@@ -25,6 +25,16 @@ __host__ __device__ inline bool sweep_covers(int shape, int W) {
     return shape > kFullWindow ? W == 32 * (shape - kFullWindow) : W < 32 * shape;
 }
 
+// Resident CTAs asked of the compiler (0: nothing said), for sweeps of four complex64 right-hand sides a warp: it
+// schedules these instances better with it. 128 points x 32, ms a solve without / with: bandwidth 40, interchanges at
+// every step .969 / .934; 72, none 1.042 / .987; 97, at every step 1.368 / 1.226; 128, none .903 / .873. The others lose by it
+// (fewer CTAs an SM), or were not tried.
+template <typename T, int RPL, bool BWD, int RH>
+constexpr int sweep_min_ctas() {
+    if (sizeof(T) != 4 || RH != 4) return 0;
+    return BWD ? (RPL >= 3 && RPL <= 5 ? 3 : 0) : (RPL == 4 ? 1 : 0);
+}
+
 // One substitution sweep (forward with L and the row interchanges, or backward with U) for
 // narrow bands; each warp carries RH right-hand sides. Step k handles row c = k (forward) or
 // c = n-1-k (backward); the row with step index k' lives in window slot s = k' mod RS,
@@ -51,7 +61,7 @@ __host__ __device__ inline bool sweep_covers(int shape, int W) {
 // work and copy issue stay off the compute warps' dependency chains. One CTA barrier per chunk:
 // each producer arrives once its copies have landed, the compute warps once the chunk is done.
 template <typename T, int RPL, bool BWD, int RH, bool FULL>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, sweep_min_ctas<T, RPL, BWD, RH>())
     band_sweep_kernel(int n, int kl, int ku, int ldab, const cx<T>* __restrict__ ab_all,
                       const cx<T>* __restrict__ ut_all, const int* __restrict__ ipiv_all, int L,
                       cx<T>* __restrict__ B_all, const int* __restrict__ active, int CH,
