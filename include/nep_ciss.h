@@ -254,8 +254,9 @@ int nep_plan_execute_batch(int32_t count, nep_plan_t *plans, const void *const *
 int nep_plan_result(nep_plan_t p, nep_result_t *out);
 int nep_plan_destroy(nep_plan_t p);
 /* Device buffers of a plan (for inspection/tests): name in {"F","coef","ab","ut","ipiv","info",
- * "Y","S","mu","sigma","tnorm","beta","sweeps","H","newton_its","newton_ok","candidates",
- * "newton_lambda"}; returns the device pointer and its bytes ("ut" is empty for bands too wide
+ * "Y","S","mu","sigma","tnorm","beta","sweeps","H","U","W","newton_its","newton_ok","candidates",
+ * "newton_lambda"} (U and W: the Hankel SVD H = U Sigma W^H, L M x L M column-major, of which the columns
+ * up to the Hankel rank are orthonormal); returns the device pointer and its bytes ("ut" is empty for bands too wide
  * for the narrow-band sweeps; plans whose solves do not read it make it when it is first asked for, and
  * fill it at every later execution). */
 int nep_plan_buffer(nep_plan_t p, const char *name, void **dev_ptr, size_t *bytes);

@@ -127,16 +127,23 @@ __device__ __forceinline__ double warp_reduce_scatter4(double v0, double v1, dou
     return k;
 }
 
+// When a pair with a small column counts as orthogonal (jacobi_screened_kernel): alpha, beta and g2 the squared norms
+// and |gamma|^2. Off by default.
+struct Relaxed {
+    double low2 = -1.0;            // squared norm of the small columns
+    double small2 = 0, kept2 = 0;  // squared component that may remain, beside another small column or a larger one
+    __device__ __forceinline__ bool operator()(double al, double be, double g2) const {
+        if (low2 < 0.0) return false;  // known where it is compiled: no FP64 work there
+        const double hi = fmax(al, be);
+        return fmin(al, be) <= low2 && g2 <= (hi <= low2 ? small2 : kept2) * hi;
+    }
+};
 // One column pair by the whole CTA (rows, cols <= 2 blockDim): the warps split the rows, one or two
 // register elements per thread and column, the partial dot products meeting in red4 (double-buffered
 // by buf: a warp writes buffer b of pair k + 2 only after the barrier of pair k + 1, which every warp
-// reaches after reading buffer b of pair k). Returns whether it rotated. low2, th2: a pair with a column
-// of squared norm <= low2 also counts as orthogonal once |gamma|^2 <= th2 max(alpha, beta).
-__device__ __forceinline__ bool jacobi_relaxed(double al, double be, double g2, double low2, double th2) {
-    return fmin(al, be) <= low2 && g2 <= th2 * fmax(al, be);
-}
+// reaches after reading buffer b of pair k). Returns whether it rotated.
 __device__ __forceinline__ bool jacobi_pair_cta(int rows, int cols, zd* ap, zd* aq, zd* vp, zd* vq, double tol,
-                                                double low2, double th2, double (*red4)[8][4], int& buf) {
+                                                const Relaxed& relaxed, double (*red4)[8][4], int& buf) {
     const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, nsub = nthr >> 5;
     const bool two = rows > nthr || cols > nthr;  // second element per thread needed
     zd xa[2], ya[2], xv[2], yv[2];
@@ -170,7 +177,7 @@ __device__ __forceinline__ bool jacobi_pair_cta(int rows, int cols, zd* ap, zd* 
     be = __shfl_sync(0xffffffffu, x, 1);
     const double gr = __shfl_sync(0xffffffffu, x, 2), gi = __shfl_sync(0xffffffffu, x, 3);
     double c, sr, si;
-    if (low2 >= 0.0 && jacobi_relaxed(al, be, fma(gr, gr, gi * gi), low2, th2)) return false;
+    if (relaxed(al, be, fma(gr, gr, gi * gi))) return false;
     if (!jacobi_rotation(al, be, gr, gi, tol, c, sr, si)) return false;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -227,7 +234,7 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int rows, int cols, zd* __r
                 zd* vp = Vm + (int64_t)p * cols;
                 zd* vq = Vm + (int64_t)q * cols;
                 if (rows <= 256 && cols <= 256 && nsub > 1) {
-                    if (jacobi_pair_cta(rows, cols, ap, aq, vp, vq, tol, -1.0, 0.0, red4, buf) && threadIdx.x == 0)
+                    if (jacobi_pair_cta(rows, cols, ap, aq, vp, vq, tol, Relaxed{}, red4, buf) && threadIdx.x == 0)
                         atomicOr(&flags[sweep & 1], 1);
                     continue;
                 }
@@ -277,13 +284,18 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int rows, int cols, zd* __r
 // depend on timing; the first unfinished pair never waits, so the CTAs cannot wait for one another in a
 // circle. Every wait is bounded as the grid barrier's is.
 //
-// A pair needs a rotation when |gamma| > tol sqrt(alpha beta), as in jacobi_kernel, except that a
-// pair with a column of norm <= sqrt(low2) |R_00| (a tenth of the rank threshold: its triplet is not used, only
-// its singular value is reported) needs none once |gamma| <= sqrt(th2) |R_00| max(|a_p|, |a_q|). What such a
-// pair leaves is a component of at most sqrt(th2) |R_00| of the smaller column along the larger one, a fifth
-// of the truncation that the QR applies elsewhere (1e-14 |R_00|). The moments' rounding noise
-// fills the Hankel matrix with columns of norm 1e-15 to 1e-14 sigma_1, and orthogonalising those
-// against each other to full relative accuracy was most of the work.
+// A pair needs a rotation when |gamma| > tol sqrt(alpha beta), as in jacobi_kernel, except where a column is small,
+// of norm <= low |R_00| (a tenth of the rank threshold: its triplet is not used, only its singular value is
+// reported). Such a pair needs none once the smaller column's component along the larger one, |gamma| / max(|a_p|,
+// |a_q|), is at most, with t the QR's truncation (1e-14),
+//   t |R_00| / sqrt(cols) beside a larger column: all small columns together leave at most t |R_00| along it, so the
+//     triplets in use are those of a matrix within the truncation that the QR applies elsewhere;
+//   t |R_00| / 5 beside another small one, each pair's share only: it moves no triplet in use. The singular values of
+//     such columns are reported as their norms, within 4.2e-15 sigma_1 of LAPACK's for 16 Hankel matrices of order
+//     64 to 256 (full sweeps after the truncation: 4.2e-15).
+// The moments' rounding noise fills the Hankel matrix with columns of norm 1e-15 to 1e-14 sigma_1, and orthogonalising
+// those against each other to full relative accuracy was most of the work. With t / sqrt(cols) between small columns
+// too there is no gain: n = 16384, bandwidth 128, a pass takes 102 ms, 105 with full sweeps, 96 so.
 constexpr int kScreenMax = 256;     // rows and columns at most
 struct ScreenWork {
     int count[2];                                    // pairs that need a rotation, by sweep parity
@@ -296,7 +308,7 @@ struct ScreenWork {
 size_t jacobi_screen_bytes(int n) { return n <= kScreenMax ? sizeof(ScreenWork) : 0; }
 
 __global__ void __launch_bounds__(128) jacobi_screened_kernel(int rows, int cols, zd* __restrict__ A, zd* __restrict__ Vm,
-                                                              int max_sweeps, double tol, double low2, double th2,
+                                                              int max_sweeps, double tol, Relaxed relaxed,
                                                               ScreenWork* __restrict__ sw,
                                                               int* __restrict__ sweeps_out, GridBar bar) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
@@ -308,8 +320,9 @@ __global__ void __launch_bounds__(128) jacobi_screened_kernel(int rows, int cols
     const int P = cols + (cols & 1), G = gridDim.x, R = P - 1;
     unsigned int epoch = 0;
     const double s1 = norm2(ldcg(A));
-    low2 *= s1;
-    th2 *= s1;
+    relaxed.low2 *= s1;
+    relaxed.small2 *= s1;
+    relaxed.kept2 *= s1;
     auto pos = [&](int k, int r) { return k == 0 ? 0 : ((k - 1 + r) % R) + 1; };  // round r, place k: column
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + tid; t < (int64_t)cols * cols; t += (int64_t)G * blockDim.x)
         Vm[t] = mk((t % cols) == (t / cols) ? 1.0 : 0.0, 0.0);
@@ -365,7 +378,7 @@ __global__ void __launch_bounds__(128) jacobi_screened_kernel(int rows, int cols
                 const double g2 = fma(gr, gr, gi * gi);
                 if (todo[u]) {
                     const bool need =
-                        g2 > (tol * tol) * (a1 * b1) && a1 != 0.0 && b1 != 0.0 && !jacobi_relaxed(a1, b1, g2, low2, th2);
+                        g2 > (tol * tol) * (a1 * b1) && a1 != 0.0 && b1 != 0.0 && !relaxed(a1, b1, g2);
                     if (lane == 0) sw->need[p * cols + q0 + u] = need ? 1 : 0;
                     found += need;
                 }
@@ -464,7 +477,7 @@ __global__ void __launch_bounds__(128) jacobi_screened_kernel(int rows, int cols
             }
             __syncthreads();
             const bool rot = jacobi_pair_cta(rows, cols, A + (int64_t)p * rows, A + (int64_t)q * rows,
-                                             Vm + (int64_t)p * cols, Vm + (int64_t)q * cols, tol, low2, th2, red4, buf);
+                                             Vm + (int64_t)p * cols, Vm + (int64_t)q * cols, tol, relaxed, red4, buf);
             __syncthreads();  // the columns are written
             if (tid < 2) {
                 if (rot) sw->changed[mine] = 1;
@@ -477,8 +490,8 @@ __global__ void __launch_bounds__(128) jacobi_screened_kernel(int rows, int cols
     if (blockIdx.x == 0 && tid == 0) *sweeps_out = sweep + 1;
 }
 
-// (every CTA finds the norms and ranks itself and writes its share of U and W)
-// sigma_i = |a_i|, descending order; U(:, r) = a_(i)/sigma, W(:, r) = V(:, i) for rank r of i.
+// sigma_i = |a_i|, descending order; U(:, r) = a_(i)/sigma, W(:, r) = V(:, i) for rank r of i. Every CTA finds the
+// norms and ranks itself and writes its share of U and W.
 __global__ void svd_finish_kernel(int rows, int cols, const zd* __restrict__ A, const zd* __restrict__ Vm,
                                   zd* __restrict__ U, zd* __restrict__ W, double* __restrict__ sigma) {
     extern __shared__ double nrm[];
@@ -709,10 +722,10 @@ static bool launch_jacobi_cluster(int rows, int cols, zd* A, zd* Vm, int max_swe
     return false;
 }
 
-// A is destroyed; U (rows x cols) may be nullptr; W (cols x cols); sigma (cols). low, theta > 0 (with
-// w.screen): the relaxed rule of jacobi_screened_kernel for columns of norm <= low |A(0,0)|.
+// A is destroyed; U (rows x cols) may be nullptr; W (cols x cols); sigma (cols). low > 0 (with w.screen): the
+// rule of jacobi_screened_kernel for columns of norm <= low |A(0,0)|, with the truncation trunc.
 static int jacobi_svd_run(int rows, int cols, zd* A, zd* U, zd* W, double* sigma, JacobiWork w, double low,
-                          double theta, cudaStream_t st) {
+                          double trunc, cudaStream_t st) {
     if (cols <= 0) return NEP_OK;
     NEP_CUDA(cudaMemsetAsync(w.flags, 0, 2 * sizeof(int), st));
     NEP_CUDA(cudaMemsetAsync(w.bar, 0, 2 * sizeof(unsigned), st));
@@ -735,10 +748,10 @@ static int jacobi_svd_run(int rows, int cols, zd* A, zd* U, zd* W, double* sigma
     if (low > 0.0 && w.screen && rows <= kScreenMax && cols <= kScreenMax) {
         NEP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_screened_kernel, 128, 0));
         blocks = std::max(1, std::min(P / 2, sms * std::max(per_sm, 1)));
-        double low2 = low * low, th2 = theta * theta;
+        Relaxed relaxed{low * low, 0.04 * trunc * trunc, trunc * trunc / cols};
         ScreenWork* sw = static_cast<ScreenWork*>(w.screen);
         max_sweeps = 60;
-        void* args[] = {&rows, &cols, &A, &w.Vm, &max_sweeps, &tol, &low2, &th2, &sw, &w.sweeps, &gb};
+        void* args[] = {&rows, &cols, &A, &w.Vm, &max_sweeps, &tol, &relaxed, &sw, &w.sweeps, &gb};
         NEP_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_screened_kernel, dim3(blocks), dim3(128), args, 0, st));
         count_launch();
     } else if (!launch_jacobi_cluster(rows, cols, A, w.Vm, max_sweeps, tol, w.sweeps, st)) {
@@ -1215,7 +1228,7 @@ __global__ void permute_rows_kernel(int n, int ncols, const int* __restrict__ pe
 // R(0:mq, :)^H only. Singular values and vectors beyond mq are returned as zero.
 // With keep > trunc (and w.screen, n <= 256) the QR already stops where ||R_22||_F <= keep |R_00|, and Jacobi
 // takes the unreduced block with the rest: columns that small only need their singular values
-// (jacobi_screened_kernel's relaxed rule), for which reducing them further is wasted. Their U and W columns
+// (jacobi_screened_kernel's rule), for which reducing them further is wasted. Their W columns
 // are then not orthogonal to full accuracy; those of larger columns are.
 int qrcp_jacobi_svd(int n, zd* A, zd* U, zd* W, double* sigma, zd* work1, zd* work2, zd* work3, zd* tau, int* perm,
                     double* nrm2, int* steps_dev, int* steps_host, double trunc, double keep, JacobiWork w,
@@ -1249,7 +1262,7 @@ int qrcp_jacobi_svd(int n, zd* A, zd* U, zd* W, double* sigma, zd* work1, zd* wo
         rh_from_qr_kernel<<<ceil_div((int64_t)n * mq, 256), 256, 0, st>>>(n, mq, nref, A, work1);
         NEP_CHECK_LAUNCH();
         // Jacobi on R(0:mq, :)^H: work1 -> Uj (work2, n x mq), Wj (work3, mq x mq)
-        NEP_TRY(jacobi_svd_run(n, mq, work1, work2, work3, sigma, w, kept ? keep : 0.0, 0.2 * trunc, st));
+        NEP_TRY(jacobi_svd_run(n, mq, work1, work2, work3, sigma, w, kept ? keep : 0.0, trunc, st));
     }
     qr_pad_kernel<<<ceil_div((int64_t)n * n, 256), 256, 0, st>>>(n, mq, work3, U, W, sigma);
     NEP_CHECK_LAUNCH();

@@ -1502,7 +1502,8 @@ extern "C" int nep_plan_buffer(nep_plan_t p, const char* name, void** dev_ptr, s
         {"S", p->S, sizeof(zd) * K * n * L},        {"mu", p->mu, sizeof(zd) * K * L * L},
         {"sigma", p->sigma, sizeof(double) * p->LM}, {"tnorm", p->tnorm, sizeof(double) * N},
         {"beta", p->beta, sizeof(double) * N},      {"sweeps", p->sweeps, sizeof(int) * N},
-        {"H", p->H, sizeof(zd) * p->LM * p->LM},
+        {"H", p->H, sizeof(zd) * p->LM * p->LM},    {"U", p->U, sizeof(zd) * p->LM * p->LM},
+        {"W", p->W, sizeof(zd) * p->LM * p->LM},
         {"newton_its", p->its, sizeof(int) * p->LM},  {"newton_ok", p->ok, sizeof(int) * p->LM},
         {"candidates", p->cand, sizeof(zd) * p->LM},  {"newton_lambda", p->lamn, sizeof(zd) * p->LM},
     };
