@@ -12,12 +12,6 @@ __device__ __forceinline__ cx<T> shfl_cx(cx<T> v, int src) {
     return r;
 }
 
-__device__ __forceinline__ int posmod(int a, int m) {
-    int r = a % m;
-    return r < 0 ? r + m : r;
-}
-
-
 // Asynchronous global->shared copy of one complex element (8 or 16 bytes); completion is
 // awaited with cp_async_wait_all() before the barrier that publishes the data.
 template <typename T>

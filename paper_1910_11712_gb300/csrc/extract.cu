@@ -288,8 +288,8 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int rows, int cols, zd* __r
 // of norm <= low |R_00| (a tenth of the rank threshold: its triplet is not used, only its singular value is
 // reported). Such a pair needs none once the smaller column's component along the larger one, |gamma| / max(|a_p|,
 // |a_q|), is at most, with t the QR's truncation (1e-14),
-//   t |R_00| / sqrt(cols) beside a larger column: all small columns together leave at most t |R_00| along it, so the
-//     triplets in use are those of a matrix within the truncation that the QR applies elsewhere;
+//   t |R_00| / sqrt(cols) beside a column that is not small: all small ones together leave at most t |R_00| along it,
+//     the truncation that the QR applies elsewhere;
 //   t |R_00| / 5 beside another small one, each pair's share only: it moves no triplet in use. The singular values of
 //     such columns are reported as their norms, within 4.2e-15 sigma_1 of LAPACK's for 16 Hankel matrices of order
 //     64 to 256 (full sweeps after the truncation: 4.2e-15).

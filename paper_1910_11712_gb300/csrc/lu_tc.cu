@@ -723,7 +723,10 @@ bool lu_tc_enabled() {
     return on;
 }
 
-// CTAs per point: two where the device then still holds every CTA at once
+// CTAs per point: two where the device then still holds every CTA at once. Both factor the whole panel: latency
+// bought with work. A pass alone takes 41.1 ms with two and 42.8 with one at bandwidth 97, 155 and 204 at 576 (64 points
+// each); with other passes on the device one CTA gives the higher throughput: bandwidth 97, 8 pipelines, 29.7 and 23.6 ms
+// a pass, though at 576 with 2 pipelines two still lead, 132 and 150.
 static int lu_tc_split(int npts) {
     static const int sms = [] {
         int dev = 0, v = 0;

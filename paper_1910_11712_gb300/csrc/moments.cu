@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(256) moments_kernel_generic(int64_t nl, int N,
 // every result that the guard (oz.cuh) finds too small for the digits.
 // n L = 524288, N = 64, K = 16: 0.486 ms (FP64 FMAs: 3.56, at the FP64 pipe's rate; HBM alone: 0.10). Error
 // against a 113-bit sum: 4.7e-17 (N <= 64) and 8.3e-17 (N = 192) of the result's norm, FP64 FMAs 2.7e-16 to
-// 6.7e-16. What bounds it: issue (the digits' bytes and 72 MMAs per 8 nodes), not the tensor pipe.
+// 6.7e-16. On an ellipse the guard takes part: 0.534 ms. What bounds it: latency with 16 warps an SM (128 registers); the
+// MMA pipe of mma.sync is the busiest unit, 54 % (issue 42 %, DRAM 17 %).
 namespace oz {
 constexpr int KC = CH / 8;        // 16-wide MMA steps per chunk (8 nodes)
 constexpr int FRAG = 32 * 4;      // words of one A fragment

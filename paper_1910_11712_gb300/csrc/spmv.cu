@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(256) split_residual_kernel(const int64_t* __re
     if (threadIdx.x < 3 * nl) atomic_max_nonneg_d(nrm + ((int64_t)j * L + l0) * 3 + threadIdx.x, sqrt(top));
 }
 
-// Right-hand sides per thread of the residual kernels: four where the blocks still fill the device.
+// Right-hand sides per thread of the residual kernels: four where the blocks still fill the device (608: four an SM
+// on 152 SMs).
 // n = 16384, five-point, 128 points x 32, double-float: 1.28 ms with one (T's values read 32 times a point
 // through L2), 0.68 with four; FP64 residual of 64 points x 32 with its assembly: 3.42 -> 1.23 ms, then
 // bound by the FP64 units.
