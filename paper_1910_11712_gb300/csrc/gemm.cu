@@ -319,7 +319,7 @@ static int zgemm_fma(int M, int N, int K, int opA, const zd* A, int lda, const z
 // 35 / 22, 96 x 96 x 192 with 192 x 96 x 96 91 / 83; against them 16 x 128 x 64 without room to split 25 / 37,
 // 7 x 7 x 9409 48 / 89, 128 x 128 x 128 twice 100 / 103, 4096 x 66 x 66 81 to 91 / 171.
 static bool zgemm_small(int M, int N, int K, int max_splits) {
-    return (int64_t)M * N * K <= 2000000 && K <= std::min(256, 32 * max_splits);
+    return K > 0 && (int64_t)M * N * K <= 2000000 && K <= std::min(256, 32 * max_splits);
 }
 
 // C = op(A) B. part: workspace of splits*M*N elements when K is long (nullptr => no split).
