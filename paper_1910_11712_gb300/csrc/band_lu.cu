@@ -427,13 +427,15 @@ __global__ void __launch_bounds__(512)
 //   40, n = 1600: 64 x 16 .320 / .218; .551 / .400, 96 x 16 .394 / .428; .639 / .807, 128 x 32 .564 / .850; .970 / 1.62;
 //   64, n = 2048: 64 x 16 .412 / .313; .759 / .549, 96 x 16 .502 / .613; .896 / 1.10, 128 x 32 .736 / 1.22; 1.45 / 2.20;
 //   72, n = 2500: 64 x 16 .529 / .392; .938 / .680, 96 x 16 .671 / .767; 1.12 / 1.36;
+//   80, n = 1500: 64 x 16 .320 / .249; .607 / .440, 96 x 16 .408 / .488; .725 / .879; 97: 64 x 16 .366 / .283; .659 / .454;
 //   complex128, 10: 64 x 16 1.06 / .871; 1.12 / 1.02, 96 x 16 1.72 / 1.74; 1.74 / 2.04; 16: 64 x 32 2.07 / 1.99; 2.69 / 2.38;
 //   24: 64 x 16 1.27 / 1.17; 1.65 / 1.67, 64 x 32 2.07 / 2.23; 2.69 / 3.05, 96 x 32 3.08 / 4.43; 4.10 / 6.09;
 //   40: 64 x 16 2.47 / 1.89; 3.15 / 2.61, 64 x 32 4.32 / 3.70; 5.22 / 4.92, 96 x 32 6.75 / 7.37; 8.78 / 9.81,
 //     128 x 32 9.66 / 7.38; 11.9 / 9.82;
 //   64: 64 x 16 2.99 / 3.24; 5.22 / 4.77, 96 x 32 8.45 / 12.8; 15.3 / 17.8, 128 x 32 12.1 / 12.8; 19.7 / 17.8;
 //   80, n = 1500: 64 x 32 5.57 / 5.17; 8.42 / 9.50, 96 x 32 8.60 / 10.3; 13.0 / 19.0.
-// complex64: up to N L = 1024 and kl + ku <= 144 (and one right-hand side always). complex128: unless its CTAs of 16
+// complex64: up to N L = 1024 and kl + ku <= 144 (and one right-hand side always); wider bands were slower when the line was
+// drawn, with backward windows of kl + ku rows, and no longer are. complex128: unless its CTAs of 16
 // columns leave a last wave mostly empty (96 x 32: 192 CTAs on 152 SMs), or, beyond N L = 1024, the sweeps' windows
 // take one register a lane (up to 31 rows, kl > 16 or the wider backward window too).
 template <typename T>
